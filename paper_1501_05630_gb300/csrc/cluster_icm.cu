@@ -763,6 +763,7 @@ __device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const
         S.s[li] ^= f0;
         if (G > 1) S.s[nls + li] ^= f1;
     }
+    if (S.gord) __syncthreads();                     // below a thread reads sites that others reversed
     if (!(act0 | act1)) {
         __syncthreads();
         return;                                      // the same decision in every CTA

@@ -184,3 +184,21 @@ def test_diluted_couplings_keep_the_cluster_layout(icm, lattice, L, K, threads):
     b.load(couplings=J)                                   # back to undiluted couplings
     assert b.cluster() == K
     b.close()
+
+
+def test_block_growth_sees_the_reversed_spins(icm):
+    """2D L=128 on 8 x 512 (2 x 2 growth blocks: a thread grows sites that
+    other threads reversed in step 2a) with two CTAs on some SMs: the same
+    chain as without blocks (8 x 1024), bit for bit, and the same twice."""
+    icmpt, ctx = icm
+    T = I.ladder(0.2, 1.5, 32)
+    g, J, s0, _ = _setup(O.SQUARE2D, 128, I.PM_J, 20, T, 0x1503)
+    runs = []
+    for threads in (1024, 512, 512):
+        b = icmpt.Batch(ctx, O.SQUARE2D, 128, I.PM_J, J, T, 1.0, 0x1503, spins=s0)
+        b.set_cluster(8, threads)
+        b.run(16)
+        runs.append((b.read_spins(), b.read_energies()))
+        b.close()
+    for s, e in runs[1:]:
+        assert np.array_equal(s, runs[0][0]) and np.array_equal(e, runs[0][1])
