@@ -127,7 +127,6 @@ struct CS {
     int *cntloc, *flags, *seed, *csz, *cnt_n, *cnt_d;
     uint32_t *flipw;
     uint32_t *swap_x;
-    int *swap_list, *swap_n;
     uint64_t *swap_mask;
     double *accE;
     long long *acc64, *nmeas;
@@ -167,8 +166,6 @@ __device__ __forceinline__ CS make_cs(unsigned char *smem, const ClusterLayout &
     S.cnt_d = (int *)(smem + L.cnt_d);
     S.flipw = (uint32_t *)(smem + L.flipw);
     S.swap_x = (uint32_t *)(smem + L.swap_x);
-    S.swap_list = (int *)(smem + L.swap_list);
-    S.swap_n = (int *)(smem + L.swap_n);
     S.swap_mask = (uint64_t *)(smem + L.swap_mask);
     S.accE = (double *)(smem + L.accE);
     S.acc64 = (long long *)(smem + L.acc64);
@@ -991,22 +988,16 @@ __device__ void cl_pt_pass(const KParams &P, const CS &S, uint32_t t, uint32_t i
 {
     using ET = typename std::conditional<GAUSS, float, int>::type;
     const int nT = P.nT, np = nT - 1, nls = S.nls;
-    for (int i = threadIdx.x; i < 2 * np; i += blockDim.x) {
-        const int c = i / np, k = i % np;
-        uint32_t x[4];
-        philox10k((uint32_t)k, t, (uint32_t)c, (2u << 24) | inst, P.key, x);
-        if constexpr (GAUSS) S.swap_x[c * 32 + k] = pt_word_gauss(x[0]);
-        else S.swap_x[c * 32 + k] = pt_word_pmj(x[0], P.thr_swap + P.swap_off[k], P.swap_len[k], P.dbeta_l2e[k]);
-    }
+    for (int i = threadIdx.x; i < 2 * np; i += blockDim.x)
+        pt_draw<GAUSS>(i, np, t, inst, P.key, S.swap_x, P.thr_swap, P.swap_off, P.swap_len, P.dbeta_l2e);
     __syncthreads();
     // every CTA decides alike (the same energies and draws); rank 0 traces
     if (threadIdx.x < 32)
-        pt_warp<GAUSS, ET>((ET *)S.E, P.R, np, S.swap_x, P.dbeta_l2e, S.swap_list, S.swap_n, S.swap_mask,
+        pt_warp<GAUSS, ET>((ET *)S.E, P.R, np, S.swap_x, P.dbeta_l2e, S.swap_mask,
                            trace && S.rank == 0 ? P.tr_swap + (size_t)slot * 2 * np : nullptr);
     __syncthreads();
-    const int n0 = S.swap_n[0], n1 = S.swap_n[1];
-    if (n0 + n1 > 0) {
-        const SwapMasks m = swap_masks(S.swap_list, n0, n1, S.swap_mask);
+    SwapMasks m;
+    if (swap_masks(S.swap_mask, m)) {
         const bool two = P.G > 1;
         for (int li = threadIdx.x; li < nls; li += blockDim.x) {
             const uint64_t x = (uint64_t)S.s[li] | (two ? (uint64_t)S.s[nls + li] << 32 : 0ull);
@@ -1295,9 +1286,7 @@ ClusterLayout cluster_layout(int N, int Z, int R, int G, int nT, int K, int nwar
     L.flipw = take(2 * 4);
     L.csz = take(32 * 4);
     L.swap_x = take(2 * 32 * 4);
-    L.swap_list = take(2 * 32 * 4);
-    L.swap_n = take(2 * 4);
-    L.swap_mask = take(2 * 8);
+    L.swap_mask = take(6 * 8);
     L.cnt_n = take(32 * 4);
     L.cnt_d = take(32 * 4);
     L.accE = take(nT * 8);

@@ -1303,7 +1303,7 @@ static icm_status apply_threads(icm_batch *b, int threads)
     P.wide = wide ? 1 : 0;
     P.scratch = wide ? b->scratch : nullptr;
     P.scratch_words = wide ? words : 0;
-    P.small_counts = (((half + threads - 1) / threads) * P.Z < 16 && (P.N + threads - 1) / threads < 16) ? 1 : 0;
+    P.cnt_planes = icm::count_planes((P.N + threads - 1) / threads, (half + threads - 1) / threads, P.Z);
     b->threads = threads;
     b->ctas_per_sm = ctas;
     b->grid = grid;
@@ -1385,7 +1385,7 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
     b->grid = b->n_clusters * K;
     // CTAs per SM when the most clusters are resident
     b->ctas_per_sm = (clusters * K + b->ctx->num_sms - 1) / b->ctx->num_sms;
-    P.small_counts = 0;
+    P.cnt_planes = icm::count_planes((2 * hs + threads - 1) / threads, (hs + threads - 1) / threads, P.Z);
     return ICM_OK;
 }
 
@@ -1564,7 +1564,7 @@ static int team_fit(const icm_batch *b, int w, int max_smem, icm::KParams &P)
     P.wide = 0;
     P.scratch = nullptr;
     P.scratch_words = 0;
-    P.small_counts = (((half + w - 1) / w) * B.Z < 16 && (B.N + w - 1) / w < 16) ? 1 : 0;
+    P.cnt_planes = icm::count_planes((B.N + w - 1) / w, (half + w - 1) / w, B.Z);
     return k;
 }
 

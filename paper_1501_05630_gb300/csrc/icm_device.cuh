@@ -108,27 +108,59 @@ __device__ __forceinline__ uint32_t pt_word_pmj(uint32_t x, const uint32_t *thr,
     // thr[d-1] > x iff exp(-2 d dbeta) 2^32 >= x + 1 iff d <= (32 - log2(x + 1)) / (2 dbl),
     // dbl = dbeta log2(e): start there, then step to the exact count against
     // the table (from any start: up while thr[d] > x, down while thr[d-1] <= x)
-    const float est = (32.f - __log2f((float)x + 1.f)) / (2.f * dbl);
+    const float est = __fdividef(32.f - __log2f((float)x + 1.f), 2.f * dbl);
     int d = est >= (float)len ? len : (est > 0.f ? (int)est : 0);
-    while (d < len && __ldg(thr + d) > x) ++d;
-    while (d > 0 && __ldg(thr + d - 1) <= x) --d;
+    // both neighbours of the guess in one pair of loads: it is mostly the count itself
+    const uint32_t up = d < len ? __ldg(thr + d) : 0u, dn = d > 0 ? __ldg(thr + d - 1) : ~0u;
+    if (up > x) {
+        do ++d;
+        while (d < len && __ldg(thr + d) > x);
+    } else if (dn <= x) {
+        do --d;
+        while (d > 0 && __ldg(thr + d - 1) <= x);
+    }
     return (uint32_t)d;
+}
+
+// The PT draw of (copy, pair) i = c np + k at sweep t, as the word of its test.
+template <bool GAUSS>
+__device__ __forceinline__ void pt_draw(int i, int np, uint32_t t, uint32_t inst, const uint32_t (&key)[20],
+                                        uint32_t *w, const uint32_t *thr_swap, const int *off, const int *len,
+                                        const float *dbl)
+{
+    const int c = i >= np, k = i - c * np;
+    uint32_t x[4];
+    philox10k((uint32_t)k, t, (uint32_t)c, (2u << 24) | inst, key, x);
+    if constexpr (GAUSS) w[c * 32 + k] = pt_word_gauss(x[0]);
+    else w[c * 32 + k] = pt_word_pmj(x[0], thr_swap + off[k], len[k], dbl[k]);
+}
+
+// Bit k of x on bit 2k.
+__device__ __forceinline__ uint32_t spread16(uint32_t x)
+{
+    x = (x | (x << 8)) & 0x00FF00FFu;
+    x = (x | (x << 4)) & 0x0F0F0F0Fu;
+    x = (x | (x << 2)) & 0x33333333u;
+    return (x | (x << 1)) & 0x55555555u;
+}
+__device__ __forceinline__ uint64_t spread32(uint32_t x)
+{
+    return (uint64_t)spread16(x & 0xFFFFu) | ((uint64_t)spread16(x >> 16) << 32);
 }
 
 // The passes of both copies, run by one warp: lanes 16c .. 16c+15 run copy c.
 // Each lane runs its copy's sequential decisions (loads and compares only:
 // the energies at positions k+1 are read as they were before the pass); then
 // lane h of copy c, for the positions k = h and h + 16, writes the energy of
-// position k after the pass, the run of accepted swaps that starts at k as a
-// (source, destination) pair of replica slots, and its trace byte; lane 0 of
-// each half writes its copy's run count and the mask of replica slots whose
-// configuration moves down one position.
+// position k after the pass and its trace byte; and lanes h = 0, 1, 2 write
+// the configuration moves of the pass as masks of replica bits (see
+// SwapMasks): the starts of the runs of accepted swaps, their ends, and the
+// bits that move down one position.
 //   E [R] energies, slot 2k + c; w [2][32] words of pt_word_* (copy c at 32 c);
-//   dbl [np] (beta_k - beta_{k+1}) log2(e) (Gaussian); list [2][32];
-//   nlist [2]; down [2]; trace [2][np] or null.
+//   dbl [np] (beta_k - beta_{k+1}) log2(e) (Gaussian); mask [3][2]; trace [2][np] or null.
 template <bool GAUSS, typename ET>
-__device__ __forceinline__ void pt_warp(ET *E, int R, int np, const uint32_t *w, const float *dbl, int *list,
-                                        int *nlist, uint64_t *down, uint8_t *trace)
+__device__ __forceinline__ void pt_warp(ET *E, int R, int np, const uint32_t *w, const float *dbl, uint64_t *mask,
+                                        uint8_t *trace)
 {
     const int lane = threadIdx.x & 31, c = lane >> 4, h = lane & 15;
     const uint32_t *wc = w + 32 * c;
@@ -165,25 +197,15 @@ __device__ __forceinline__ void pt_warp(ET *E, int R, int np, const uint32_t *w,
         }
     }
     __syncwarp();
-    const uint32_t starts = acc & ~(acc << 1);
 #pragma unroll
     for (int it = 0; it < 2; ++it) {
         const int k = h + 16 * it;
         if (k <= np) E[2 * k + c] = en[it];
-        if (k < np) {
-            if ((starts >> k) & 1u) {
-                const int end = k + __ffs(~(acc >> k)) - 1;    // the first rejected swap above k (or np)
-                list[32 * c + ICM_IDX(__popc(starts & ((1u << k) - 1u)), 32, 12)] = ((2 * k + c) << 8) | (2 * end + c);
-            }
-            if (trace) trace[c * np + k] = (uint8_t)((acc >> k) & 1u);
-        }
+        if (k < np && trace) trace[c * np + k] = (uint8_t)((acc >> k) & 1u);
     }
-    if (h == 0) {
-        nlist[c] = __popc(starts);
-        uint64_t D = 0;
-        for (uint32_t b = acc; b; b &= b - 1u) D |= 1ull << (2 * (__ffs(b) - 1) + 2 + c);
-        down[c] = D;
-    }
+    // a run k..m of accepted swaps: start bit k, end bit m + 1 <= np
+    const uint32_t up = acc << 1;
+    if (h < 3) mask[2 * h + c] = spread32(h == 0 ? acc & ~up : h == 1 ? up & ~acc : up) << c;
 }
 
 // Bit position of the rank-th set bit of w, counting from bit 0 (rank <
@@ -207,34 +229,29 @@ __device__ __forceinline__ int nth_set_bit(uint32_t w, uint32_t rank)
 }
 
 // The configuration moves of one PT pass as masks of the 64 replica bits of a
-// site (two words).  A run of accepted swaps k..m, list entry
-// (2k + c) << 8 | 2(m + 1) + c, moves the configuration at bit s = 2k + c up
-// to e = 2(m + 1) + c, and the others of the run down one position (mask
-// down).  With fw = the sum of 2^e - 2^s over the runs of copy c,
-// ((x & st) + fw) & en carries every start bit to its end bit at once: the
-// runs of one copy cover disjoint bit ranges, so no carry leaves its run.
+// site (two words).  A run of accepted swaps k..m moves the configuration at
+// bit s = 2k + c up to e = 2(m + 1) + c, and the others of the run down one
+// position (mask down).  With fw = the sum of 2^e - 2^s over the runs of copy
+// c (the end mask minus the start mask), ((x & st) + fw) & en carries every
+// start bit to its end bit at once: the runs of one copy cover disjoint bit
+// ranges, so no carry leaves its run.
 struct SwapMasks {
     uint64_t keep, down, st[2], fw[2], en[2];
 };
 
-__device__ __forceinline__ SwapMasks swap_masks(const int *list, int n0, int n1, const uint64_t *down)
+// mask: pt_warp's [3][2] (starts, ends, bits moving down, per copy).  Returns
+// false when no swap was accepted.
+__device__ __forceinline__ bool swap_masks(const uint64_t *mask, SwapMasks &m)
 {
-    SwapMasks m;
-    m.down = down[0] | down[1];
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-        m.st[c] = m.fw[c] = m.en[c] = 0ull;
-        const int n = c ? n1 : n0;
-        for (int j = 0; j < n; ++j) {
-            const int mv = list[32 * c + j];
-            const uint64_t s = 1ull << (mv >> 8), e = 1ull << (mv & 0xff);
-            m.st[c] |= s;
-            m.en[c] |= e;
-            m.fw[c] += e - s;
-        }
+        m.st[c] = mask[c];
+        m.en[c] = mask[2 + c];
+        m.fw[c] = m.en[c] - m.st[c];
     }
+    m.down = mask[4] | mask[5];
     m.keep = ~(m.down | m.st[0] | m.st[1]);
-    return m;
+    return (m.st[0] | m.st[1]) != 0ull;
 }
 
 __device__ __forceinline__ uint64_t swap_apply(const SwapMasks &m, uint64_t x)
@@ -416,6 +433,177 @@ __device__ __forceinline__ uint32_t ge_bitsliced(uint32_t c0, uint32_t c1, uint3
         eq &= ~(c[i] ^ kb);
     }
     return gt | eq;
+}
+
+// Warp totals of vertical counters: as warp_vsum, plane by plane.  The 32 x 32
+// bit transpose of a plane puts counter b's bits of all lanes into lane b,
+// whose popcount is the plane's total: 5 shuffles per plane where the
+// butterfly of warp_vsum takes 5 and two more for its carries, and one rolled
+// body for any number of planes np <= NPL (the planes above are zero).
+template <int NPL>
+__device__ __forceinline__ int warp_vcount(uint32_t (&pl)[NPL], int np, int lane)
+{
+    int v = 0;
+#pragma unroll 1
+    for (int i = 0; i < np; ++i) {
+        v += __popc(warp_transpose32(pl[0], lane)) << i;
+#pragma unroll
+        for (int j = 0; j + 1 < NPL; ++j) pl[j] = pl[j + 1];
+    }
+    return v;
+}
+
+// One bit per pair and site: pair j (copies at bits 2j, 2j + 1 of the first
+// word) on bit 2j, pair 16 + j (the second word) on bit 2j + 1.
+__device__ __forceinline__ uint32_t pair_bits(uint32_t e0, uint32_t e1)
+{
+    return (e0 & 0x55555555u) | ((e1 << 1) & 0xAAAAAAAAu);
+}
+// set where q = s^a s^b = -1
+__device__ __forceinline__ uint32_t overlap_word(uint32_t w0, uint32_t w1)
+{
+    return pair_bits(w0 ^ (w0 >> 1), w1 ^ (w1 >> 1));
+}
+// the spins of copy cb
+__device__ __forceinline__ uint32_t copy_word(uint32_t w0, uint32_t w1, int cb) { return pair_bits(w0 >> cb, w1 >> cb); }
+// the pair of a bit of such a word
+__device__ __forceinline__ int pair_of_bit(int bit) { return (bit >> 1) + 16 * (bit & 1); }
+
+// Per bit lane: u == k, where u's binary digits are the bit-planes (k < 0 or k > 15: none).
+__device__ __forceinline__ uint32_t eq_bitsliced(const uint32_t (&c)[4], int k)
+{
+    uint32_t eq = (k & ~15) ? 0u : ~0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) eq &= ~(c[i] ^ (0u - (uint32_t)((k >> i) & 1)));
+    return eq;
+}
+
+// ---------------------------------------------------------------------------
+// +-J Metropolis update of the replica bits [8 q0, 8 q1) of one site word.
+//   c    : bit-planes of u = # unsatisfied bonds of the site, per replica
+//   z    : bonds present at the site
+//   thr  : the threshold rows of the word's 16 temperatures, kThrRow words
+//          each: m = 2, 4, 6, 8, then m = 1, 3, 5, 7 (m = s h = z - 2u)
+//   rq   : Philox counter word 2 (replica position / 4) of the word's bit 0
+// Returns the flips: every replica with m <= 0 of the whole word (the caller
+// masks its own groups) and those with x < thr[m].  With h = ceil(z / 2) the
+// classes of positive m are u = h-1, h-2, ..: entry j of the parity's row
+// belongs to u = h - 1 - j, so each draw is compared with the same Z/2
+// uniform thresholds and the class masks pick the result afterwards: Z/2
+// compares and as many conditional ORs per update, where extracting u bit by
+// bit and looking its threshold up took about 14 instructions.
+constexpr int kThrRow = 8;
+
+// The rows of all temperatures from the batch's table thr_metro[r][m] (stride
+// thr_stride(Z); both copies of a temperature have the same thresholds), 0 for
+// the ghost replicas of a partly used last word.
+template <int Z>
+__device__ __forceinline__ void load_thr_rows(uint32_t *thr, const uint32_t *thr_metro, int R, int G, int tid, int nth)
+{
+    for (int i = tid; i < 16 * G * kThrRow; i += nth) {
+        const int k = i / kThrRow, w = i % kThrRow;
+        const int m = w < 4 ? 2 * w + 2 : 2 * w - 7;
+        thr[i] = 2 * k < R && m <= Z ? thr_metro[2 * k * thr_stride(Z) + m] : 0u;
+    }
+}
+
+template <int Z, bool DIL>
+__device__ __forceinline__ uint32_t pmj_flips(const uint32_t (&c)[4], int z, bool tie, uint32_t live,
+                                              const uint32_t *thr, uint32_t site, uint32_t t, uint32_t rq,
+                                              uint32_t inst, const uint32_t (&key)[20], int q0, int q1)
+{
+    constexpr int NJ = Z / 2;               // classes of positive m
+    uint32_t m[NJ], flip;
+    [[maybe_unused]] uint32_t mt = 0u;      // m = 0 on a diluted instance: accepted with probability 1/2
+    if constexpr (DIL) {
+        const int h = (z + 1) >> 1;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) m[j] = eq_bitsliced(c, h - 1 - j);
+        flip = ge_bitsliced(c[0], c[1], c[2], c[3], tie ? (z >> 1) + 1 : h);
+        if (tie && !(z & 1)) mt = eq_bitsliced(c, z >> 1) & live;
+    } else if constexpr (Z == 8) {          // h = 4
+        flip = c[3] | c[2];
+        m[0] = c[0] & c[1] & ~flip;
+        m[1] = c[1] & ~c[0] & ~flip;
+        m[2] = c[0] & ~c[1] & ~flip;
+        m[3] = ~(c[0] | c[1] | flip);
+    } else if constexpr (Z == 6) {          // h = 3 (z = 5, 6)
+        flip = c[2] | (c[1] & c[0]);
+        m[0] = c[1] & ~c[0] & ~c[2];
+        m[1] = c[0] & ~c[1] & ~c[2];
+        m[2] = ~(c[0] | c[1] | c[2]);
+        if (z <= 4) {                       // h = 2 (chimera C_1)
+            flip = c[2] | c[1];
+            m[0] = m[1];
+            m[1] = m[2];
+            m[2] = 0u;
+        }
+    } else {                                // z = 4: h = 2
+        flip = c[2] | c[1];
+        m[0] = c[0] & ~flip;
+        m[1] = ~(c[0] | flip);
+    }
+    // 4-entry half row of the degree's parity (odd degrees: chimera and diluted lattices)
+    const uint32_t *row = thr + q0 * 4 * kThrRow;
+    if (DIL || Z == 6) row += (z & 1) << 2;
+    uint32_t acc = 0u;
+#pragma unroll 1
+    for (int q = q0; q < q1; ++q, row += 4 * kThrRow) {
+        uint32_t x[4], y[4];
+        philox10x2(site, t, rq + 2u * (uint32_t)q, inst, key, x, y);
+        uint32_t a[NJ];
+        [[maybe_unused]] uint32_t at = 0u;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) a[j] = 0u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {       // one temperature: two replicas
+            uint32_t th[4];
+            if constexpr (NJ == 2) {
+                const uint2 v = *reinterpret_cast<const uint2 *>(row + k * kThrRow);
+                th[0] = v.x;
+                th[1] = v.y;
+            } else {
+                const uint4 v = *reinterpret_cast<const uint4 *>(row + k * kThrRow);
+                th[0] = v.x;
+                th[1] = v.y;
+                th[2] = v.z;
+                th[3] = v.w;
+            }
+#pragma unroll
+            for (int i = 2 * k; i < 2 * k + 2; ++i) {
+                const uint32_t xr = i < 4 ? x[i] : y[i - 4];
+#pragma unroll
+                for (int j = 0; j < NJ; ++j)
+                    if (xr < th[j]) a[j] |= 1u << i;
+                if constexpr (DIL)
+                    if (xr < 0x80000000u) at |= 1u << i;
+            }
+        }
+        uint32_t f = 0u;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) f |= a[j] & (m[j] >> (8 * q));
+        if constexpr (DIL) f |= at & (mt >> (8 * q));
+        acc |= f << (8 * q);
+    }
+    return flip | acc;
+}
+
+// Add the site's unsatisfied bonds after the flips (z - u where flipped, u
+// elsewhere; only the replicas of `mask`) to the vertical counters of the
+// energies: E = 2 U - (bonds present).
+template <int NPL>
+__device__ __forceinline__ void pmj_count(uint32_t (&pl)[NPL], const uint32_t (&c)[4], int z, uint32_t flip,
+                                          uint32_t mask)
+{
+    uint32_t u[4], cy = ~0u;                // z - u = z + ~u + 1, mod 16
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t zb = 0u - (uint32_t)((z >> i) & 1), n = ~c[i];
+        const uint32_t v = n ^ zb ^ cy;
+        cy = (n & zb) | (cy & (n | zb));
+        u[i] = ((flip & v) | (~flip & c[i])) & mask;
+    }
+    vadd4(pl, u[0], u[1], u[2], u[3]);
 }
 
 }  // namespace

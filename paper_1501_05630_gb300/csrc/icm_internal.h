@@ -20,6 +20,24 @@ __host__ __device__
 #endif
 constexpr int thr_stride(int Z) { return Z > 7 ? 16 : 8; }
 
+// Words from one pair's overlap mask to the next: odd, so that the threads of
+// the seed search (one per pair) read different banks.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+constexpr int mask_stride(int NW) { return NW | 1; }
+
+// Bit-planes for the counts of a thread that takes `sites` sites, `half_sites`
+// of them of colour 1 with Z bonds each (at most kPlanes: the launch-shape
+// checks bound both counts by 255).
+inline int count_planes(int sites, int half_sites, int Z)
+{
+    const int most = half_sites * Z > sites ? half_sites * Z : sites;
+    int n = 1;
+    while (n < kPlanes && (most >> n)) ++n;
+    return n;
+}
+
 // Byte offsets into the fused kernel's dynamic shared memory.  In the
 // global-resident ("wide") layout the spins, couplings, neighbour table,
 // overlap masks and cluster words stay in global memory (size 0 here).
@@ -30,13 +48,11 @@ struct SmemLayout {
     int coup;       // float [N][Z] (Gaussian) or uint8 [N] bit d = (J < 0) (+-J)
     int E;          // float or int32 [R]
     int Epart;      // float or int32 [nwarps][max(R, 32)]
-    int rtab;       // uint32 [R][thr_stride(Z)] thresholds (+-J) or float [R] -2 beta log2(e) (Gaussian)
-    int icm_mask;   // uint32 [n_icm][NW] overlap masks per ICM pair
+    int rtab;       // uint32 [16 G][8] threshold rows (+-J) or float [32 G] -2 beta log2(e) (Gaussian)
+    int icm_mask;   // uint32 [n_icm][mask_stride(NW)] overlap masks per ICM pair
     int icm_C;      // uint32 [N]        cluster bits of every pair (bit 2k: pair k, bit 2k + 1: pair 16 + k)
     int swap_x;     // uint32 [2][32]
-    int swap_list;  // int32 [2][32]   per run: (source bit << 8) | destination bit
-    int swap_n;     // int32 [2]       runs per copy
-    int swap_mask;  // uint64 [2]      bits moving down one slot, per copy
+    int swap_mask;  // uint64 [3][2]   PT moves as bit masks (pt_warp), per copy
     int swap_tab;   // [3][32]         per neighbouring pair k: dbeta log2(e) (float), +-J table offset and length
     int flipw;      // uint32 [2]      step-2a reversal masks of the two words
     int icm_seed;   // int32 [32]      seed position per ICM pair (-1: none)
@@ -58,7 +74,7 @@ struct KParams {
     int diluted;                  // 1: some instance has absent bonds (J = 0): per-instance tables below
     int scratch_words;            // wide layout: uint32 words of scratch per CTA (cluster words, masks)
     uint32_t *scratch;            // wide layout: [grid][scratch_words]
-    int small_counts;             // per-thread observable counts fit 4 bit-planes
+    int cnt_planes;               // bit-planes that hold a thread's counts of sites and bonds
     // geometry, shared by all instances of the batch
     const uint16_t *nbr;          // [N][Z]
     const uint8_t *zdeg;          // [N]
@@ -175,7 +191,7 @@ struct ClusterLayout {
     int esum;       // float or int32 [32]
     int flipw;      // uint32 [2]
     int csz;        // int32 [32]               this CTA's cluster sites per pair (read remotely)
-    int swap_x, swap_list, swap_n, swap_mask;   // as in SmemLayout
+    int swap_x, swap_mask;                      // as in SmemLayout
     int cnt_n, cnt_d;   // int32 [32]           this CTA's observable counts (read remotely)
     int accE, acc64, nmeas;                     // observables (rank 0)
     int icmst;      // uint64 [2]               cluster moves and growth scans of this instance (rank 0)
@@ -190,8 +206,8 @@ cudaError_t launch_cluster(const KParams &P, const ClusterLayout &CL, bool gauss
 cudaError_t cluster_occupancy(bool gauss, int Z, bool dil, int K, int threads, int smem, int *clusters);
 int fused_threads(int N);
 int fused_threads_wide(int N);
-// uint32 words of per-CTA scratch of the wide layout (2 N cluster words, 32
-// overlap-mask rows of NW words), rounded to 16 bytes.
+// uint32 words of per-CTA scratch of the wide layout (the cluster words and the
+// overlap-mask rows), rounded to 16 bytes.
 int wide_scratch_words(int N);
 
 // Host-callable launchers (pt_icm.cu).  Return a cudaError_t.

@@ -97,8 +97,6 @@ struct Sm {
     uint32_t *mask;
     uint32_t *C;
     uint32_t *swap_x;
-    int *swap_list;
-    int *swap_n;
     uint64_t *swap_mask;
     float *sw_dbl;       // [32] (beta_k - beta_{k+1}) log2(e)
     int *sw_off, *sw_len;  // [32] +-J swap threshold table of pair k
@@ -130,8 +128,6 @@ __device__ __forceinline__ Sm make_sm(unsigned char *base, const SmemLayout &L)
     S.mask = (uint32_t *)(base + L.icm_mask);
     S.C = (uint32_t *)(base + L.icm_C);
     S.swap_x = (uint32_t *)(base + L.swap_x);
-    S.swap_list = (int *)(base + L.swap_list);
-    S.swap_n = (int *)(base + L.swap_n);
     S.swap_mask = (uint64_t *)(base + L.swap_mask);
     S.sw_dbl = (float *)(base + L.swap_tab);
     S.sw_off = (int *)(base + L.swap_tab + 128);
@@ -205,20 +201,19 @@ __device__ __forceinline__ void load_nbrs(const uint16_t *nbr, int p, int (&q)[Z
 }
 
 // ---------------------------------------------------------------------------
-// Step 1: one pass of a checkerboard half-sweep (colour COLOR) over the 16
-// replica bits [32 g + 16 H, 32 g + 16 H + 16) of every site word of that
-// colour.  Bits at or above R ("ghost" replicas of a partly used last word)
-// are updated at beta = 0 and never read, so the inner loop has no guards.
-// Two Philox4x32-10 blocks are generated together (8 draws) so that their
-// dependency chains interleave.  The sites are taken by threads j0, j0 +
-// jstride, ...; when other threads run another pass over the same words at
-// the same time (tiny instances), the flips go in by atomic XOR (each pass
-// owns its 16 bits, so the result does not depend on the order).
-template <bool GAUSS, int Z, bool WIDE, bool DIL, bool SHARED>
-__device__ __forceinline__ void sweep_pass(const KParams &P, const uint32_t (&key)[20], const Sm &S, const Team &T,
+// Step 1, Gaussian couplings: one pass of a checkerboard half-sweep (colour
+// COLOR) over the 16 replica bits [32 g + 16 H, 32 g + 16 H + 16) of every
+// site word of that colour.  Bits at or above R ("ghost" replicas of a partly
+// used last word) are updated at beta = 0 and never read, so the inner loop
+// has no guards.  Two Philox4x32-10 blocks are generated together (8 draws)
+// so that their dependency chains interleave.  The sites are taken by threads
+// j0, j0 + jstride, ...; when other threads run another pass over the same
+// words at the same time (SHARED: tiny instances), the flips go in by atomic
+// XOR (each pass owns its bits, so the result does not depend on the order).
+template <int Z, bool WIDE, bool DIL, bool SHARED>
+__device__ __forceinline__ void gauss_pass(const KParams &P, const uint32_t (&key)[20], const Sm &S, const Team &T,
                                            uint32_t t, uint32_t inst, int g, int COLOR, int H, int j0, int jstride)
 {
-    using ET = typename std::conditional<GAUSS, float, int>::type;
     const int lane = threadIdx.x & 31, warp = T.tid >> 5;
     const int N = P.N, half = P.half;
     [[maybe_unused]] const int nth = T.nth;   // the bound of a checked index
@@ -226,203 +221,225 @@ __device__ __forceinline__ void sweep_pass(const KParams &P, const uint32_t (&ke
     const int sh0 = 16 * H;                       // first bit of this pass inside the word
     const int npairs8 = (P.R - rbase + 7) >> 3;   // 8-bit groups holding at least one live replica (1 or 2)
     uint32_t *sg = S.s + g * N;
-    ET acc[16];
+    float acc[16];
 #pragma unroll
-    for (int b = 0; b < 16; ++b) acc[b] = ET(0);
+    for (int b = 0; b < 16; ++b) acc[b] = 0.f;
     for (int j = j0; j < half; j += jstride) {
         const int p = COLOR * half + j;
         const uint32_t sw0 = sg[p];
         const uint32_t sw = sw0 >> sh0;                 // this pass's bits at 0..15: constant shifts below
         const uint32_t site = __ldg(P.pos2site + p);
         uint32_t flip = 0;                              // bits 0..15 of this pass
-        if constexpr (GAUSS) {
-            // h = sum_d J_d s_d = Jsum - 2 sum_{d: s_d = -1} J_d: one bit test and one
-            // predicated add per neighbour and bit
-            float J2[Z];
-            uint32_t nw[Z];
-            int q[Z];
-            load_nbrs<Z>(S.nbr, p, q);
-            float Jsum = 0.f;
+        // h = sum_d J_d s_d = Jsum - 2 sum_{d: s_d = -1} J_d: one bit test and one
+        // predicated multiply-add (exact product, one rounding) per neighbour and bit
+        float J[Z];
+        uint32_t nw[Z];
+        int q[Z];
+        load_nbrs<Z>(S.nbr, p, q);
+        float Jsum = 0.f;
 #pragma unroll
-            for (int d = 0; d < Z; ++d) {
-                nw[d] = sg[ICM_IDX(q[d], N, 1)] >> sh0;
-                const float J = S.Jd[ICM_IDX(p * Z + d, N * Z, 2)];
-                Jsum += J;
-                J2[d] = 2.f * J;
-            }
-            const float *b2l = S.b2l + rbase;
+        for (int d = 0; d < Z; ++d) {
+            nw[d] = sg[ICM_IDX(q[d], N, 1)] >> sh0;
+            J[d] = S.Jd[ICM_IDX(p * Z + d, N * Z, 2)];
+            Jsum += J[d];
+        }
+        const float *b2l = S.b2l + rbase;
 #pragma unroll
-            for (int qq = 0; qq < 2; ++qq) {
-                if (qq < npairs8) {
-                    uint32_t x[4], y[4];
-                    philox10x2(site, t, (uint32_t)(rbase >> 2) + 2 * qq, inst, key, x, y);
-                    uint32_t f8 = 0u;                           // this group's accepted bits
+        for (int qq = 0; qq < 2; ++qq) {
+            if (qq < npairs8) {
+                uint32_t x[4], y[4];
+                philox10x2(site, t, (uint32_t)(rbase >> 2) + 2 * qq, inst, key, x, y);
+                uint32_t f8 = 0u;                           // this group's accepted bits
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int b = 8 * qq + i;               // compile-time bit of the pass
-                        float h = Jsum;
+                for (int i = 0; i < 8; ++i) {
+                    const int b = 8 * qq + i;               // compile-time bit of the pass
+                    float h = Jsum;
 #pragma unroll
-                        for (int d = 0; d < Z; ++d)
-                            if ((nw[d] >> b) & 1u) h -= J2[d];
-                        // sh = s_i h_i, Delta E = 2 sh; accept iff x < 2^32 exp(-2 beta sh),
-                        // compared as rz(x) < 2^(32 + b2l sh) in fp32 (b2l = -2 beta log2 e):
-                        // for sh <= 0 the right side is >= 2^32 > rz(x), so Delta E <= 0 is
-                        // always accepted
-                        const float sh = ((sw >> b) & 1u) ? -h : h;
-                        const uint32_t xr = i < 4 ? x[i] : y[i - 4];
-                        const float lim = ex2_approx(fmaf(b2l[b], sh, 32.f));
-                        bool a;
-                        if constexpr (DIL) {
-                            // diluted instance: Delta E = 0 (a site without bonds) is
-                            // accepted with probability 1/2
-                            a = (sh < 0.f) || (sh == 0.f ? (!S.tie || xr < 0x80000000u) : (__uint2float_rz(xr) < lim));
-                        } else {
-                            a = __uint2float_rz(xr) < lim;
-                        }
-                        f8 |= (uint32_t)a << i;
-                        acc[b] -= sh;                           // e = -s'h: -sh, or +sh after a flip
-                        if (a) acc[b] += 2.f * sh;
+                    for (int d = 0; d < Z; ++d)
+                        if ((nw[d] >> b) & 1u) h = fmaf(J[d], -2.f, h);
+                    // sh = s_i h_i, Delta E = 2 sh; accept iff x < 2^32 exp(-2 beta sh),
+                    // compared as rz(x) < 2^(32 + b2l sh) in fp32 (b2l = -2 beta log2 e):
+                    // for sh <= 0 the right side is >= 2^32 > rz(x), so Delta E <= 0 is
+                    // always accepted
+                    const float sh = ((sw >> b) & 1u) ? -h : h;
+                    const uint32_t xr = i < 4 ? x[i] : y[i - 4];
+                    const float lim = ex2_approx(fmaf(b2l[b], sh, 32.f));
+                    bool a;
+                    if constexpr (DIL) {
+                        // diluted instance: Delta E = 0 (a site without bonds) is
+                        // accepted with probability 1/2
+                        a = (sh < 0.f) || (sh == 0.f ? (!S.tie || xr < 0x80000000u) : (__uint2float_rz(xr) < lim));
+                    } else {
+                        a = __uint2float_rz(xr) < lim;
                     }
-                    flip |= f8 << (8 * qq);
+                    f8 |= (uint32_t)a << i;
+                    acc[b] -= sh;                           // e = -s'h: -sh, or +sh after a flip
+                    if (a) acc[b] += 2.f * sh;
                 }
-            }
-        } else {
-            uint32_t c0 = 0, c1 = 0, c2 = 0, c3 = 0;   // bit-planes of u = # unsatisfied bonds
-            const uint32_t jb = S.Jb[ICM_IDX(p, N, 3)];
-            int q[Z];
-            load_nbrs<Z>(S.nbr, p, q);
-            uint32_t u[Z];
-#pragma unroll
-            for (int d = 0; d < Z; ++d) u[d] = sw0 ^ sg[ICM_IDX(q[d], N, 1)] ^ (0u - ((jb >> d) & 1u));
-            csa_count<Z>(u, c0, c1, c2, c3);
-            c0 >>= sh0;
-            c1 >>= sh0;
-            c2 >>= sh0;
-            c3 >>= sh0;
-            const int z = (!DIL && P.const_z) ? P.const_z : (int)S.zdeg[ICM_IDX(p, N, 3)];   // degree = bonds present
-            // m = z - 2u <= 0  <=>  u >= ceil(z/2): always accepted; on a diluted
-            // instance only m < 0 (u >= floor(z/2) + 1), m = 0 takes the 1/2 entry
-            if constexpr (DIL) {
-                flip = ge_bitsliced(c0, c1, c2, c3, S.tie ? (z >> 1) + 1 : (z + 1) >> 1) & 0xFFFFu;
-            } else if constexpr (Z > 7) {
-                flip = (c3 | c2) & 0xFFFFu;         // z = 8: u >= 4
-            } else {
-                flip = ((z <= 4) ? (c2 | c1) : (c2 | (c1 & c0))) & 0xFFFFu;
-            }
-            constexpr int TS = thr_stride(Z);
-            const uint32_t *thr = S.thr + rbase * TS;
-#pragma unroll
-            for (int qq = 0; qq < 2; ++qq) {
-                if (qq < npairs8) {
-                    uint32_t x[4], y[4];
-                    philox10x2(site, t, (uint32_t)(rbase >> 2) + 2 * qq, inst, key, x, y);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int b = 8 * qq + i;
-                        const int u = (int)(((c0 >> b) & 1u) | (((c1 >> b) & 1u) << 1) | (((c2 >> b) & 1u) << 2) |
-                                            (((c3 >> b) & 1u) << 3));
-                        const int m = z - 2 * u;
-                        const uint32_t xr = i < 4 ? x[i] : y[i - 4];
-                        const uint32_t th = thr[b * TS + ICM_IDX(m > 0 ? m : 0, TS, 4)];
-                        flip |= (uint32_t)(xr < th) << b;
-                        acc[b] += ((flip >> b) & 1u) ? m : -m;
-                    }
-                }
+                flip |= f8 << (8 * qq);
             }
         }
         if constexpr (SHARED) atomicXor(sg + p, flip << sh0);
         else sg[p] = sw0 ^ (flip << sh0);
     }
     if (COLOR == 1) {   // energies: every bond touches exactly one colour-1 site
-        const ET v = transpose_reduce16(acc, lane);
+        const float v = transpose_reduce16(acc, lane);
         const int r = rbase + (lane >> 1);
-        if (!(lane & 1) && r < P.R) ((ET *)S.Epart)[ICM_IDX(warp * P.R + r, (nth >> 5) * (P.R > 32 ? P.R : 32), 5)] = v;
+        if (!(lane & 1) && r < P.R) ((float *)S.Epart)[ICM_IDX(warp * P.R + r, (nth >> 5) * (P.R > 32 ? P.R : 32), 5)] = v;
     }
 }
 
-// Tiny instances with at least twice the threads a colour needs: the
+// Step 1, +-J couplings: the replica bits [8 q0, 8 q1) of word g of every site
+// of colour COLOR (see pmj_flips).  The whole word is one pass: the
+// unsatisfied-bond planes are formed once for 32 replicas, and the energies
+// are counted bit-sliced after the flips, one vertical counter per replica,
+// so no per-replica accumulators stay live across the sites.  Bound by ALU
+// issue.  Chimera C_8 x 10^4, 16 sweeps: 14.0 to 11.1 ms against the sweep in
+// two 16-bit passes with a threshold lookup per replica; 2D L=64 x 40 in wide
+// CTAs: 2.29 to 1.83 ms.
+template <int Z, bool WIDE, bool DIL>
+__device__ __forceinline__ void pmj_pass(const KParams &P, const uint32_t (&key)[20], const Sm &S, const Team &T,
+                                         uint32_t t, uint32_t inst, int g, int COLOR, int q0, int q1, int j0,
+                                         int jstride, bool shared)
+{
+    const int lane = threadIdx.x & 31, warp = T.tid >> 5;
+    const int N = P.N, half = P.half;
+    uint32_t *sg = S.s + g * N;
+    const int left = P.R - 32 * g;
+    const uint32_t live = left >= 32 ? kFull : (1u << left) - 1u;
+    // this pass's bits; ghost replicas follow up to a multiple of 16
+    const int end = 8 * q1 < left ? 8 * q1 : min(32, (left + 15) & ~15);
+    const uint32_t mine = (kFull >> (32 - end)) & (kFull << (8 * q0));
+    uint32_t pl[kPlanes];
+#pragma unroll
+    for (int i = 0; i < kPlanes; ++i) pl[i] = 0u;
+    for (int j = j0; j < half; j += jstride) {
+        const int p = COLOR * half + j;
+        const uint32_t sw = sg[p];
+        const uint32_t site = __ldg(P.pos2site + p);
+        const uint32_t jb = S.Jb[ICM_IDX(p, N, 3)];
+        int q[Z];
+        load_nbrs<Z>(S.nbr, p, q);
+        uint32_t u[Z], c[4];
+#pragma unroll
+        for (int d = 0; d < Z; ++d) u[d] = sw ^ sg[ICM_IDX(q[d], N, 1)] ^ (0u - ((jb >> d) & 1u));
+        csa_count<Z>(u, c[0], c[1], c[2], c[3]);
+        // degree = bonds present: Z on the lattices, per site on chimera and diluted batches
+        const int z = (!DIL && Z != 6) ? Z : (!DIL && P.const_z) ? P.const_z : (int)S.zdeg[ICM_IDX(p, N, 3)];
+        const uint32_t flip = pmj_flips<Z, DIL>(c, z, S.tie, live, S.thr + 16 * g * kThrRow, site, t, 8u * (uint32_t)g, inst,
+                                                 key, q0, q1) & mine;
+        if (shared) atomicXor(sg + p, flip);
+        else sg[p] = sw ^ flip;
+        if (COLOR == 1) pmj_count(pl, c, z, flip, mine & live);
+    }
+    if (COLOR == 1) {   // energies: every bond touches exactly one colour-1 site
+        const int v = warp_vcount(pl, P.cnt_planes, lane);
+        if (lane < left) ((int *)S.Epart)[ICM_IDX(warp * P.R + 32 * g + lane, (T.nth >> 5) * (P.R > 32 ? P.R : 32), 5)] = v;
+    }
+}
+
+// Tiny Gaussian instances with at least twice the threads a colour needs: the
 // threads split into groups of whole warps that run different passes at the
 // same time; every warp writes its energy slots, the ones of passes it did not
 // run as 0.
-template <bool GAUSS, int Z, bool WIDE, bool DIL>
-__device__ __forceinline__ void metropolis_sweep_concurrent(const KParams &P, const uint32_t (&key)[20], const Sm &S,
-                                                         const Team &T, uint32_t t, uint32_t inst, int npass, int gthr,
-                                                         int conc)
+template <int Z, bool WIDE, bool DIL>
+__device__ __forceinline__ void gauss_sweep_concurrent(const KParams &P, const uint32_t (&key)[20], const Sm &S,
+                                                       const Team &T, uint32_t t, uint32_t inst, int npass, int gthr,
+                                                       int conc)
 {
-    using ET = typename std::conditional<GAUSS, float, int>::type;
     const int group = T.tid / gthr;
     const int nslot = (T.nth >> 5) * P.R;
-    for (int i = T.tid; i < nslot; i += T.nth) ((ET *)S.Epart)[i] = ET(0);
+    for (int i = T.tid; i < nslot; i += T.nth) ((float *)S.Epart)[i] = 0.f;
     team_sync(T);
     for (int color = 0; color < 2; ++color) {
         for (int p0 = 0; p0 < npass; p0 += conc) {
             const int pass = p0 + group;
             if (group < conc && pass < npass)    // whole warps: gthr is a multiple of 32
-                sweep_pass<GAUSS, Z, WIDE, DIL, true>(P, key, S, T, t, inst, pass >> 1, color, pass & 1,
-                                                      T.tid - group * gthr, gthr);
+                gauss_pass<Z, WIDE, DIL, true>(P, key, S, T, t, inst, pass >> 1, color, pass & 1, T.tid - group * gthr,
+                                               gthr);
         }
         team_sync(T);
     }
 }
 
-// Step 1 for all replicas: colour 0 then colour 1, each as 16-bit passes over
-// the site words.  One call site, so the pass body exists once in the kernel
-// (the instruction cache is shared by all CTAs of the SM).
+// Step 1 for all replicas: colour 0 then colour 1, each as passes over the
+// site words.  One call site per kernel, so the pass body exists once (the
+// instruction cache is shared by all CTAs of the SM).  A +-J team with at least
+// twice the threads a colour needs splits into groups of whole warps that
+// take the replicas in shares of 8 at the same time.
 template <bool GAUSS, int Z, bool WIDE, bool DIL>
 __device__ __forceinline__ void metropolis_sweep(const KParams &P, const uint32_t (&key)[20], const Sm &S, const Team &T,
                                                  uint32_t t, uint32_t inst)
 {
-    const int npass = (P.R + 15) >> 4;          // 16-bit passes per colour
     const int gthr = (P.half + 31) & ~31;        // threads of one pass
-    const int conc = min(T.nth / gthr, npass);   // passes at a time
-    if (conc >= 2) {
-        metropolis_sweep_concurrent<GAUSS, Z, WIDE, DIL>(P, key, S, T, t, inst, npass, gthr, conc);
-        return;
-    }
-    for (int it = 0; it < 2 * npass; ++it) {
-        const int color = it >= npass;
-        const int pass = it - color * npass;
-        sweep_pass<GAUSS, Z, WIDE, DIL, false>(P, key, S, T, t, inst, pass >> 1, color, pass & 1, T.tid, T.nth);
-        if (pass == npass - 1) team_sync(T);
+    if constexpr (GAUSS) {
+        const int npass = (P.R + 15) >> 4;          // 16-bit passes per colour
+        const int conc = min(T.nth / gthr, npass);   // passes at a time
+        if (conc >= 2) {
+            gauss_sweep_concurrent<Z, WIDE, DIL>(P, key, S, T, t, inst, npass, gthr, conc);
+            return;
+        }
+        for (int it = 0; it < 2 * npass; ++it) {
+            const int color = it >= npass;
+            const int pass = it - color * npass;
+            gauss_pass<Z, WIDE, DIL, false>(P, key, S, T, t, inst, pass >> 1, color, pass & 1, T.tid, T.nth);
+            if (pass == npass - 1) team_sync(T);
+        }
+    } else {
+        const int n8 = (P.R + 7) >> 3;              // groups of 8 replicas
+        const int conc = min(T.nth / gthr, n8);
+        const bool split = conc >= 2;
+        const int group = split ? T.tid / gthr : 0;
+        const int per = split ? (n8 + conc - 1) / conc : n8;
+        const int lo = group * per, hi = min(lo + per, n8);
+        const int j0 = T.tid - (split ? group * gthr : 0), jstride = split ? gthr : T.nth;
+        if (split) {                                // a warp leaves the slots of other shares 0
+            for (int i = T.tid; i < (T.nth >> 5) * P.R; i += T.nth) ((int *)S.Epart)[i] = 0;
+            team_sync(T);
+        }
+        for (int color = 0; color < 2; ++color) {
+            for (int g = lo >> 2; lo < hi && 4 * g < hi; ++g)
+                pmj_pass<Z, WIDE, DIL>(P, key, S, T, t, inst, g, color, max(lo - 4 * g, 0), min(hi - 4 * g, 4), j0,
+                                       jstride, split);
+            team_sync(T);
+        }
     }
 }
 
 // ---------------------------------------------------------------------------
 // Energies of copy cb (bit 2k + cb; cb = 0: copy a) of the pairs flagged in
 // act0/act1 (bit 2k), from the spins: +-J via bit-sliced unsatisfied-bond
-// counts (E = 2U - N_b), Gaussian via per-bit fp32 local fields; summed in a
-// fixed order.  Every thread ends with partial sums in S.Epart[warp][k]; the
-// caller adds warps.
+// counts of all pairs at once (U per pair; E = 2U - N_b), Gaussian via
+// per-bit fp32 local fields; summed in a fixed order.  Every thread ends with
+// partial sums in S.Epart[warp][k]; the caller adds warps.
 template <bool GAUSS, int Z, bool WIDE>
 __device__ __forceinline__ void pair_energies(const KParams &P, const Sm &S, const Team &T, uint32_t act0, uint32_t act1,
                                               int cb)
 {
-    using ET = typename std::conditional<GAUSS, float, int>::type;
     const int lane = threadIdx.x & 31, warp = T.tid >> 5;
     const int N = P.N, half = P.half, nth = T.nth;
-    ET *part = (ET *)S.Epart;
-    for (int g = 0; g < P.G; ++g) {
-        const uint32_t act = g ? act1 : act0;
-        if (!act) continue;                      // uniform
-        const uint32_t *sg = S.s + g * N;
-        ET acc[16];
+    if constexpr (GAUSS) {
+        float *part = (float *)S.Epart;
+        for (int g = 0; g < P.G; ++g) {
+            const uint32_t act = g ? act1 : act0;
+            if (!act) continue;                      // uniform
+            const uint32_t *sg = S.s + g * N;
+            float acc[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) acc[j] = ET(0);
-        for (int i = T.tid; i < half; i += nth) {
-            const int p = half + i;              // colour-1 sites: every bond once
-            const uint32_t sw = sg[p] >> cb;
-            int q[Z];
-            load_nbrs<Z>(S.nbr, p, q);
-            if constexpr (GAUSS) {
-                float J2[Z];
+            for (int j = 0; j < 16; ++j) acc[j] = 0.f;
+            for (int i = T.tid; i < half; i += nth) {
+                const int p = half + i;              // colour-1 sites: every bond once
+                const uint32_t sw = sg[p] >> cb;
+                int q[Z];
+                load_nbrs<Z>(S.nbr, p, q);
+                float J[Z];
                 uint32_t nw[Z];
                 float Jsum = 0.f;
 #pragma unroll
                 for (int d = 0; d < Z; ++d) {
                     nw[d] = sg[ICM_IDX(q[d], N, 6)] >> cb;
-                    const float J = S.Jd[ICM_IDX(p * Z + d, N * Z, 2)];
-                    Jsum += J;
-                    J2[d] = 2.f * J;
+                    J[d] = S.Jd[ICM_IDX(p * Z + d, N * Z, 2)];
+                    Jsum += J[d];
                 }
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
@@ -431,26 +448,35 @@ __device__ __forceinline__ void pair_energies(const KParams &P, const Sm &S, con
                     float h = Jsum;                            // h = sum_d J_d s_d
 #pragma unroll
                     for (int d = 0; d < Z; ++d)
-                        if ((nw[d] >> b) & 1u) h -= J2[d];
+                        if ((nw[d] >> b) & 1u) h = fmaf(J[d], -2.f, h);
                     acc[j] += ((sw >> b) & 1u) ? h : -h;       // e = -s_p h_p
                 }
-            } else {
-                uint32_t c0 = 0, c1 = 0, c2 = 0, c3 = 0;
-                const uint32_t jb = S.Jb[ICM_IDX(p, N, 3)];
-                uint32_t u[Z];
-#pragma unroll
-                for (int d = 0; d < Z; ++d) u[d] = sw ^ (sg[ICM_IDX(q[d], N, 6)] >> cb) ^ (0u - ((jb >> d) & 1u));
-                csa_count<Z>(u, c0, c1, c2, c3);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int b = 2 * j;
-                    acc[j] += (int)(((c0 >> b) & 1u) | (((c1 >> b) & 1u) << 1) | (((c2 >> b) & 1u) << 2) |
-                                    (((c3 >> b) & 1u) << 3));
-                }
             }
+            const float v = transpose_reduce16(acc, lane);
+            if (!(lane & 1)) part[ICM_IDX(warp * 32 + 16 * g + (lane >> 1), (nth >> 5) * 32, 7)] = v;
         }
-        const ET v = transpose_reduce16(acc, lane);
-        if (!(lane & 1)) part[ICM_IDX(warp * 32 + 16 * g + (lane >> 1), (nth >> 5) * 32, 7)] = v;
+    } else {
+        const bool two = P.G > 1;
+        uint32_t pl[kPlanes];
+#pragma unroll
+        for (int i = 0; i < kPlanes; ++i) pl[i] = 0u;
+        for (int i = T.tid; i < half; i += nth) {
+            const int p = half + i;                  // colour-1 sites: every bond once
+            const uint32_t y = copy_word(S.s[p], two ? S.s[N + p] : 0u, cb);
+            const uint32_t jb = S.Jb[ICM_IDX(p, N, 3)];
+            int q[Z];
+            load_nbrs<Z>(S.nbr, p, q);
+            uint32_t u[Z], c0, c1, c2, c3;
+#pragma unroll
+            for (int d = 0; d < Z; ++d) {
+                const int qd = ICM_IDX(q[d], N, 6);
+                u[d] = y ^ copy_word(S.s[qd], two ? S.s[N + qd] : 0u, cb) ^ (0u - ((jb >> d) & 1u));
+            }
+            csa_count<Z>(u, c0, c1, c2, c3);
+            vadd4(pl, c0, c1, c2, c3);
+        }
+        const int v = warp_vcount(pl, P.cnt_planes, lane);
+        ((int *)S.Epart)[ICM_IDX(warp * 32 + pair_of_bit(lane), (nth >> 5) * 32, 7)] = v;
     }
 }
 
@@ -470,66 +496,68 @@ __device__ __forceinline__ void pair_energies(const KParams &P, const Sm &S, con
 //      E_a + E_b of the two recomputed energies, so that the trace tests the
 //      conservation of E_a + E_b instead of restating it.
 template <bool GAUSS, int Z, bool WIDE>
-__device__ void cluster_moves(const KParams &P, const uint32_t (&key)[20], const Sm &S, const Team &T, uint32_t t,
-                              uint32_t inst, int slot, bool trace)
+__device__ void cluster_moves(const KParams &P, const Sm &S, const Team &T, int slot, bool trace)
 {
     using ET = typename std::conditional<GAUSS, float, int>::type;
     const int lane = threadIdx.x & 31, warp = T.tid >> 5, nwarps = T.nth >> 5;
     const int tid = T.tid, nth = T.nth;
-    const int N = P.N, NW = P.NW, nicm = P.n_icm, G = P.G;
+    const int N = P.N, NW = P.NW, NS = mask_stride(P.NW), nicm = P.n_icm, G = P.G;
     ET *E = (ET *)S.E;
     ET *esum = (ET *)S.icm_esum_raw;
     ICM_SUB_INIT();
 
-    // (a) masks; clear the cluster words
+    // (a) masks and their counts; clear the cluster words
+    const int kp = pair_of_bit(lane);
+    int cnt = 0;
     for (int m = warp; m < NW; m += nwarps) {
         const int p = 32 * m + lane;
-        uint32_t x = 0u;       // bit 2j: q of pair j (first word); bit 2j + 1: q of pair 16 + j
-        if (p < N) {
-            const uint32_t w0 = S.s[p];
-            x = (w0 ^ (w0 >> 1)) & 0x55555555u;
-            if (G > 1) {
-                const uint32_t w1 = S.s[N + p];
-                x |= ((w1 ^ (w1 >> 1)) & 0x55555555u) << 1;
-            }
-        }
+        const uint32_t x = p < N ? overlap_word(S.s[p], G > 1 ? S.s[N + p] : 0u) : 0u;
         const uint32_t col = warp_transpose32(x, lane);   // lane l: bit l of the 32 sites' x
-        const int k = (lane >> 1) + 16 * (lane & 1);
-        if (k < nicm) S.mask[ICM_IDX(k * NW + m, nicm * NW, 8)] = col;
+        cnt += __popc(col);
+        if (kp < nicm) S.mask[ICM_IDX(kp * NS + m, nicm * NS, 8)] = col;
     }
+    if (kp < nicm && cnt) atomicAdd(&S.cnt_n[kp], cnt);
     for (int i = tid; i < N; i += nth) S.C[i] = 0u;
     if (tid < 2) S.flipw[tid] = 0u;
     team_sync(T);
 
     // (b) per pair: n, step 2a, seed (planted into C)
     for (int k = tid; k < nicm; k += nth) {
-        uint32_t *Mk = S.mask + k * NW;
-        int n = 0;
-        for (int m = 0; m < NW; ++m) n += __popc(Mk[m]);
+        const uint32_t *Mk = S.mask + k * NS;
+        int n = S.cnt_n[k];
+        S.cnt_n[k] = 0;                        // as the observables expect it
         const int n_pre = n;
-        int flipped = 0;
-        if (P.enable_2a && 2 * n > N) {
-            for (int m = 0; m < NW; ++m) {
-                const int rem = N - 32 * m;
-                Mk[m] = ~Mk[m] & (rem >= 32 ? kFull : ((1u << rem) - 1u));
-            }
+        const bool flipped = P.enable_2a && 2 * n > N;
+        if (flipped) {
             n = N - n;
-            flipped = 1;
             atomicOr(&S.flipw[(2 * k + 1) >> 5], 1u << ((2 * k + 1) & 31));
         }
         int seed = -1;
         if (n > 0) {
-            uint32_t x[4];
-            philox10k((uint32_t)k, t, 0u, (1u << 24) | inst, key, x);
-            uint32_t rank = (uint32_t)(((uint64_t)x[0] * (uint32_t)n) >> 32);
-            for (int m = 0; m < NW; ++m) {
-                const uint32_t w = Mk[m];
-                const uint32_t c = (uint32_t)__popc(w);
-                if (rank < c) {
-                    seed = 32 * m + nth_set_bit(w, rank);
+            uint32_t rank = (uint32_t)(((uint64_t)(uint32_t)S.icm_seed[k] * (uint32_t)n) >> 32);   // see step_draws
+            // the word that holds the rank-th site, four words a step (their loads
+            // and counts overlap); bits beyond N follow every site, so rank < n
+            // never reaches the ones that the complement sets there
+            const uint32_t inv = flipped ? kFull : 0u;
+            for (int m = 0; m < NW; m += 4) {
+                uint32_t w[4];
+                uint32_t c[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    w[i] = m + i < NW ? Mk[m + i] ^ inv : 0u;
+                    c[i] = (uint32_t)__popc(w[i]);
+                }
+                c[1] += c[0];
+                c[2] += c[1];
+                c[3] += c[2];
+                if (rank < c[3]) {
+                    const int i = rank < c[1] ? (rank < c[0] ? 0 : 1) : (rank < c[2] ? 2 : 3);
+                    const uint32_t ww = i == 0 ? w[0] : i == 1 ? w[1] : i == 2 ? w[2] : w[3];
+                    rank -= i == 0 ? 0u : i == 1 ? c[0] : i == 2 ? c[1] : c[2];
+                    seed = 32 * (m + i) + nth_set_bit(ww, rank);
                     break;
                 }
-                rank -= c;
+                rank -= c[3];
             }
             atomicOr(&S.C[ICM_IDX(seed, N, 9)], 1u << (2 * (k & 15) + (k >> 4)));
         }
@@ -538,7 +566,7 @@ __device__ void cluster_moves(const KParams &P, const uint32_t (&key)[20], const
         if (trace) {
             const size_t o = (size_t)slot * P.nT + k;
             P.tr_n_pre[o] = n_pre;
-            P.tr_flip2a[o] = flipped;
+            P.tr_flip2a[o] = flipped ? 1 : 0;
             P.tr_seed[o] = seed >= 0 ? (int)__ldg(P.pos2site + seed) : -1;
             P.tr_csize[o] = 0;
             P.tr_eb[o] = (float)(E[2 * k] + E[2 * k + 1]);
@@ -598,7 +626,7 @@ __device__ void cluster_moves(const KParams &P, const uint32_t (&key)[20], const
                     w1 = S.s[N + p] ^ f1;
                     S.s[N + p] = w1;
                 }
-                dm[j] = (((w0 ^ (w0 >> 1)) & 0x55555555u) | (((w1 ^ (w1 >> 1)) & 0x55555555u) << 1)) & actc;
+                dm[j] = overlap_word(w0, w1) & actc;
                 cw[j] = C[p];
                 if (dm[j] != cw[j]) todo |= 1u << j;
             }
@@ -651,8 +679,7 @@ __device__ void cluster_moves(const KParams &P, const uint32_t (&key)[20], const
             do {
                 grew = 0;
                 for (int p = tid; p < N; p += nth) {
-                    const uint32_t w0 = S.s[p], w1 = G > 1 ? S.s[N + p] : 0u;
-                    const uint32_t d = (((w0 ^ (w0 >> 1)) & 0x55555555u) | (((w1 ^ (w1 >> 1)) & 0x55555555u) << 1)) & actc;
+                    const uint32_t d = overlap_word(S.s[p], G > 1 ? S.s[N + p] : 0u) & actc;
                     const uint32_t c = C[p];
                     if (d == c) continue;
                     int q[Z];
@@ -736,33 +763,45 @@ __device__ void cluster_moves(const KParams &P, const uint32_t (&key)[20], const
 }
 
 // ---------------------------------------------------------------------------
+// The draws of steps 2b and 3 at sweep t: the seed draws of the ICM pairs
+// (into S.icm_seed, which the seed search replaces) and the words of the PT
+// tests (S.swap_x).  They depend on (t, inst) alone, so they are taken where
+// threads are free: beside the sum of the sweep's energies, which the first R
+// threads run (at: the first thread of the draws, whole warps).  Together with
+// the PT moves as closed-form masks (pt_warp): one 2D L=8 instance 702 to 651
+// us per 64 sweeps, 3D Gaussian L=8 x 1000 2.43 to 2.36 ms per 32.
+template <bool GAUSS>
+__device__ __forceinline__ void step_draws(const KParams &P, const uint32_t (&key)[20], const Sm &S, const Team &T,
+                                           uint32_t t, uint32_t inst, int at, bool icm, bool pt)
+{
+    const int nicm = icm ? P.n_icm : 0, np = P.nT - 1, n = nicm + (pt ? 2 * np : 0);
+    for (int i = T.tid < at ? T.tid + T.nth - at : T.tid - at; i < n; i += T.nth) {
+        if (i < nicm) {
+            uint32_t x[4];
+            philox10k((uint32_t)i, t, 0u, (1u << 24) | inst, key, x);
+            S.icm_seed[i] = (int)x[0];
+        } else {
+            pt_draw<GAUSS>(i - nicm, np, t, inst, key, S.swap_x, P.thr_swap, S.sw_off, S.sw_len, P.dbeta_l2e);
+        }
+    }
+}
+
 // Step 3: the PT pass of each copy (see pt_warp), then the configuration swaps.
 template <bool GAUSS, bool WIDE>
-__device__ void pt_pass(const KParams &P, const uint32_t (&key)[20], const Sm &S, const Team &T, uint32_t t,
-                        uint32_t inst, int slot, bool trace)
+__device__ void pt_pass(const KParams &P, const Sm &S, const Team &T, int slot, bool trace)
 {
     using ET = typename std::conditional<GAUSS, float, int>::type;
-    const int nT = P.nT, np = nT - 1, N = P.N;
-    // draws of all (copy, pair) in parallel, in the form of their test
-    for (int i = T.tid; i < 2 * np; i += T.nth) {
-        const int c = i / np, k = i % np;
-        uint32_t x[4];
-        philox10k((uint32_t)k, t, (uint32_t)c, (2u << 24) | inst, key, x);
-        if constexpr (GAUSS) S.swap_x[c * 32 + k] = pt_word_gauss(x[0]);
-        else S.swap_x[c * 32 + k] = pt_word_pmj(x[0], P.thr_swap + S.sw_off[k], S.sw_len[k], P.dbeta_l2e[k]);
-    }
-    team_sync(T);
+    const int np = P.nT - 1, N = P.N;
     // warp 0 runs both copies (a half-warp each).  Accepted swaps (k,k+1), ...,
     // (m,m+1) in a row form a run: the configuration at k bubbles up to m+1
-    // and those at k+1..m+1 move down one slot; the words are permuted below
-    // from the runs and the mask of bits that move down.
+    // and those at k+1..m+1 move down one slot; every site word is permuted
+    // by the masks of the runs.
     if (T.tid < 32)
-        pt_warp<GAUSS, ET>((ET *)S.E, P.R, np, S.swap_x, S.sw_dbl, S.swap_list, S.swap_n, S.swap_mask,
+        pt_warp<GAUSS, ET>((ET *)S.E, P.R, np, S.swap_x, S.sw_dbl, S.swap_mask,
                            trace ? P.tr_swap + (size_t)slot * 2 * np : nullptr);
     team_sync(T);
-    const int n0 = S.swap_n[0], n1 = S.swap_n[1];
-    if (n0 + n1 > 0) {
-        const SwapMasks m = swap_masks(S.swap_list, n0, n1, S.swap_mask);
+    SwapMasks m;
+    if (swap_masks(S.swap_mask, m)) {
         const bool two = P.G > 1;
         for (int p = T.tid; p < N; p += T.nth) {
             const uint64_t x = (uint64_t)S.s[p] | (two ? (uint64_t)S.s[N + p] << 32 : 0ull);
@@ -775,40 +814,47 @@ __device__ void pt_pass(const KParams &P, const uint32_t (&key)[20], const Sm &S
 }
 
 // ---------------------------------------------------------------------------
-// Observables: per pair k, n = #{q_i = -1} and d = #{bonds, q_i q_j = -1}.
-template <bool GAUSS, int Z, int NPL, bool WIDE>
+// Observables: per pair k, n = #{q_i = -1} and d = #{bonds, q_i q_j = -1},
+// bit-sliced for all pairs at once (one overlap word per site, as in the
+// cluster moves).
+template <bool GAUSS, int Z, bool WIDE>
 __device__ void measure(const KParams &P, const Sm &S, const Team &T, int slot)
 {
     using ET = typename std::conditional<GAUSS, float, int>::type;
     const int lane = threadIdx.x & 31;
     const int N = P.N, half = P.half, nT = P.nT;
-    for (int g = 0; g < P.G; ++g) {
-        const int npair = min(16, nT - 16 * g);
-        const uint32_t *sg = S.s + g * N;
-        uint32_t pl[NPL];   // even bit 2k: q = -1 sites of pair k; odd bit 2k+1: its q_i q_j = -1 bonds
+    const bool two = P.G > 1;
+    uint32_t pn[kPlanes], pd[kPlanes];
 #pragma unroll
-        for (int i = 0; i < NPL; ++i) pl[i] = 0u;
-        for (int p = T.tid; p < N; p += T.nth) {
-            const uint32_t w = sg[p];
-            vadd(pl, (w ^ (w >> 1)) & 0x55555555u);
-        }
-        for (int p = half + T.tid; p < N; p += T.nth) {
-            const uint32_t w = sg[p];
-            const uint32_t qp = (w ^ (w >> 1)) & 0x55555555u;
-            int qn[Z];
-            load_nbrs<Z>(S.nbr, p, qn);
-            uint32_t x[Z];                 // an absent bond points at p itself: x = 0
+    for (int i = 0; i < kPlanes; ++i) pn[i] = pd[i] = 0u;
+    for (int p = T.tid; p < N; p += T.nth) {
+        const uint32_t x = overlap_word(S.s[p], two ? S.s[N + p] : 0u);
+        vadd(pn, x);
+        if (p < half) continue;
+        int qn[Z];
+        load_nbrs<Z>(S.nbr, p, qn);
+        uint32_t y[Z];                     // an absent bond points at p itself: y = 0
 #pragma unroll
-            for (int d = 0; d < Z; ++d) {
-                const uint32_t wq = sg[ICM_IDX(qn[d], N, 13)];
-                x[d] = (qp ^ ((wq ^ (wq >> 1)) & 0x55555555u)) << 1;
-            }
-            uint32_t c0, c1, c2, c3;
-            csa_count<Z>(x, c0, c1, c2, c3);
-            vadd4(pl, c0, c1, c2, c3);
+        for (int d = 0; d < Z; ++d) {
+            const int qd = ICM_IDX(qn[d], N, 13);
+            y[d] = x ^ overlap_word(S.s[qd], two ? S.s[N + qd] : 0u);
         }
-        const int v = warp_vsum(pl, lane);   // lane 2k: n of pair k, lane 2k+1: d of pair k
-        if (lane < 2 * npair) atomicAdd(((lane & 1) ? S.cnt_d : S.cnt_n) + 16 * g + (lane >> 1), v);
+        uint32_t c0, c1, c2, c3;
+        csa_count<Z>(y, c0, c1, c2, c3);
+        vadd4(pd, c0, c1, c2, c3);
+    }
+    if (two) {
+        const int k = pair_of_bit(lane);
+        const int n = warp_vcount(pn, P.cnt_planes, lane), d = warp_vcount(pd, P.cnt_planes, lane);
+        if (k < nT) {
+            atomicAdd(S.cnt_n + k, n);
+            atomicAdd(S.cnt_d + k, d);
+        }
+    } else {                               // one word: even bits only, so both counts share one set of planes
+#pragma unroll
+        for (int i = 0; i < kPlanes; ++i) pn[i] |= pd[i] << 1;
+        const int v = warp_vcount(pn, P.cnt_planes, lane);
+        if (lane < 2 * nT) atomicAdd(((lane & 1) ? S.cnt_d : S.cnt_n) + (lane >> 1), v);
     }
     team_sync(T);
     for (int k = T.tid; k < nT; k += T.nth) {
@@ -854,8 +900,7 @@ __device__ __forceinline__ void load_tables(const KParams &P, Sm &S, const Team 
     if constexpr (GAUSS) {
         for (int r = tid; r < 32 * G; r += nth) S.b2l[r] = r < R ? P.b2l[r] : 0.f;
     } else {
-        constexpr int TS = thr_stride(Z);
-        for (int i = tid; i < 32 * G * TS; i += nth) S.thr[i] = i < R * TS ? P.thr_metro[i] : 0u;
+        load_thr_rows<Z>(S.thr, P.thr_metro, R, G, tid, nth);
     }
     if (tid < 32) {
         S.cnt_n[tid] = 0;
@@ -940,26 +985,26 @@ __device__ __forceinline__ void run_instance(const KParams &P, const uint32_t (&
                 for (int i = tid; i < 2 * N; i += nth) P.tr_cmask[(size_t)slot * 2 * N + i] = 0u;
             team_sync(T);
         }
+        const bool icm = P.icm_every > 0 && t % (uint32_t)P.icm_every == 0 && P.n_icm > 0;
+        const bool pt = P.swap_every > 0 && t % (uint32_t)P.swap_every == 0 && nT > 1;
         if (P.enable_metropolis) {  // step 1
             metropolis_sweep<GAUSS, Z, WIDE, DIL>(P, key, S, T, t, inst);
             for (int r = tid; r < R; r += nth) {
                 ET e = ET(0);
                 for (int w = 0; w < nwarps; ++w) e += ((const ET *)S.Epart)[w * R + r];
+                if constexpr (!GAUSS) e = 2 * e - S.nb;      // E = 2 U - (bonds present)
                 ((ET *)S.E)[r] = e;
             }
-            team_sync(T);
         }
+        const int free_at = (R + 31) & ~31;                  // the threads that sum no energy
+        step_draws<GAUSS>(P, key, S, T, t, inst, free_at < nth ? free_at : 0, icm, pt);
+        team_sync(T);
         PHASE_MARK(0);
-        if (P.icm_every > 0 && t % (uint32_t)P.icm_every == 0 && P.n_icm > 0)  // steps 2a, 2b
-            cluster_moves<GAUSS, Z, WIDE>(P, key, S, T, t, inst, slot, trace);
+        if (icm) cluster_moves<GAUSS, Z, WIDE>(P, S, T, slot, trace);   // steps 2a, 2b
         PHASE_MARK(1);
-        if (P.swap_every > 0 && t % (uint32_t)P.swap_every == 0 && nT > 1)  // step 3
-            pt_pass<GAUSS, WIDE>(P, key, S, T, t, inst, slot, trace);
+        if (pt) pt_pass<GAUSS, WIDE>(P, S, T, slot, trace);              // step 3
         PHASE_MARK(2);
-        if ((long long)t >= t_meas) {
-            if (P.small_counts) measure<GAUSS, Z, 4, WIDE>(P, S, T, slot);   // every per-thread count < 16
-            else measure<GAUSS, Z, kPlanes, WIDE>(P, S, T, slot);
-        }
+        if ((long long)t >= t_meas) measure<GAUSS, Z, WIDE>(P, S, T, slot);
         PHASE_MARK(3);
     }
 
@@ -1009,7 +1054,7 @@ __device__ __forceinline__ void fused_body(const KParams &P, uint32_t n_sweeps)
         S.nbr = const_cast<uint16_t *>(P.nbr);
         S.zdeg = const_cast<uint8_t *>(P.zdeg);
         S.C = P.scratch + (size_t)blockIdx.x * P.scratch_words;
-        S.mask = S.C + 2 * P.N;
+        S.mask = S.C + P.N;
     }
     load_tables<GAUSS, Z, WIDE, DIL>(P, S, T);
     for (int slot = blockIdx.x; slot < P.n_inst; slot += gridDim.x) {
@@ -1280,12 +1325,11 @@ SmemLayout smem_layout(int N, int Z, int R, int G, int nT, int n_icm, int nwarps
     L.E = take(R * 4, 16);
     L.Epart = take(nwarps * (R > 32 ? R : 32) * 4, 16);
     L.rtab = take(gauss ? G * 32 * 4 : G * 32 * thr_stride(Z) * 4, 16);   // every bit of the G words
-    L.icm_mask = take(in_smem * n_icm * NW * 4, 16);
+    const int mask_bytes = in_smem * n_icm * mask_stride(NW) * 4;
+    L.icm_mask = take(mask_bytes, 16);
     L.icm_C = take(in_smem * N * 4, 16);
     L.swap_x = take(2 * 32 * 4, 16);
-    L.swap_list = take(2 * 32 * 4, 16);
-    L.swap_n = take(2 * 4, 16);
-    L.swap_mask = take(2 * 8, 16);
+    L.swap_mask = take(6 * 8, 16);
     L.swap_tab = take(3 * 32 * 4, 16);
     L.flipw = take(2 * 4, 16);
     L.icm_seed = take(32 * 4, 16);
@@ -1296,6 +1340,10 @@ SmemLayout smem_layout(int N, int Z, int R, int G, int nT, int n_icm, int nwarps
     L.acc64 = take(4 * nT * 8, 16);
     L.nmeas = take(8, 16);
     L.icmst = take(16, 16);
+    // The size that decides between the layouts stays where it was with
+    // unpadded mask rows and the PT pass's run lists (240 bytes): the line was
+    // measured there, and Gaussian sums depend on the CTA width it picks.
+    take(240 + align_up(in_smem * n_icm * NW * 4, 16) - align_up(mask_bytes, 16), 16);
     L.total = align_up(o, 16);
     return L;
 }
@@ -1321,7 +1369,7 @@ int fused_threads_wide(int N)
 int wide_scratch_words(int N)
 {
     const int NW = (N + 31) / 32;
-    return (2 * N + 32 * NW + 3) / 4 * 4;
+    return (2 * N + 32 * NW + 3) / 4 * 4;   // N cluster words, 32 rows of mask_stride(NW) <= N + 32 NW words in all
 }
 
 cudaError_t fused_occupancy(bool gauss, int Z, bool wide, int threads, int smem, int *ctas)

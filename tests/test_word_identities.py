@@ -221,3 +221,61 @@ def test_pt_moves_need_one_carry_per_copy():
         merged = _carry_moves(x, (r0 + r1, []), d0 | d1)
         differs += merged != _sequential_swaps(x, accs, n_pairs)
     assert differs > 0
+
+
+# --- PT moves as masks -------------------------------------------------------
+
+def _spread(x):
+    return sum(((x >> k) & 1) << (2 * k) for k in range(32))
+
+
+def test_pt_move_masks_equal_the_sequential_swaps():
+    """Starts, ends and moving bits of the runs of accepted swaps, straight
+    from the decision bits, against swapping configurations one pair at a time."""
+    rng = random.Random(11)
+    for trial in range(400):
+        np_ = rng.randint(1, 31)
+        full = (1 << np_) - 1
+        acc = [full if trial == 0 else rng.getrandbits(32) & full for _ in range(2)]
+        x = rng.getrandbits(2 * np_ + 2)
+        want = [(x >> b) & 1 for b in range(2 * np_ + 2)]
+        for c in range(2):
+            for k in range(np_):
+                if (acc[c] >> k) & 1:
+                    i, j = 2 * k + c, 2 * k + 2 + c
+                    want[i], want[j] = want[j], want[i]
+        M64 = (1 << 64) - 1
+        up = [(a << 1) & M32 for a in acc]
+        st = [(_spread(acc[c] & ~up[c] & M32) << c) & M64 for c in range(2)]
+        en = [(_spread(up[c] & ~acc[c] & M32) << c) & M64 for c in range(2)]
+        down = ((_spread(up[0])) | (_spread(up[1]) << 1)) & M64
+        y = (x & ~(down | st[0] | st[1])) | ((x & down) >> 2)
+        for c in range(2):
+            y |= (((x & st[c]) + en[c] - st[c]) & M64) & en[c]
+        assert [(y >> b) & 1 for b in range(2 * np_ + 2)] == want
+
+
+def test_unsatisfied_bonds_after_a_flip():
+    """z - u as z + ~u + 1 modulo 16 over four planes, for every degree and count."""
+    for z in range(9):
+        for u in range(z + 1):
+            cy, v = 1, 0
+            for i in range(4):
+                zb, n = (z >> i) & 1, 1 - ((u >> i) & 1)
+                v |= (n ^ zb ^ cy) << i
+                cy = (n & zb) | (cy & (n | zb))
+            assert v == z - u
+
+
+def test_threshold_classes_cover_every_positive_local_field():
+    """Entry j of the half row of the degree's parity (m = 2, 4, 6, 8 or 1, 3, 5, 7)
+    belongs to u = ceil(z / 2) - 1 - j."""
+    for z in range(9):
+        h = (z + 1) // 2
+        row = [2 * j + 2 for j in range(4)] if z % 2 == 0 else [2 * j + 1 for j in range(4)]
+        for u in range(z + 1):
+            m = z - 2 * u
+            js = [j for j in range(4) if u == h - 1 - j]
+            assert (m > 0) == (len(js) == 1)
+            if js:
+                assert row[js[0]] == m
