@@ -386,6 +386,19 @@ icm_status copy_out(icm_ctx *ctx, void *dst, const void *src, size_t bytes, uint
     return ICM_OK;
 }
 
+// Whether a caller's buffer can be a kernel's operand: device memory of the
+// context's device (a copy also reaches other devices' memory).
+bool on_device(const icm_ctx *ctx, const void *p, uint32_t flags)
+{
+    if (!(flags & ICM_DEVICE_PTR)) return false;
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == ctx->device;
+}
+
 // One launch of n_sweeps simulation steps of the batch, in its layout.
 cudaError_t launch_batch(const icm_batch *b, const icm::KParams &P, uint32_t n_sweeps, cudaStream_t st)
 {
@@ -450,11 +463,14 @@ icm_status upload_state(icm_batch *b, const void *couplings, const int8_t *spins
         if ((st = refresh_dilution(b, 0, b->n_inst))) return st;
     }
     if (spins) {
-        const size_t bytes = (size_t)b->n_inst * P.R * P.N;
-        icm_status st = copy_in(ctx, b->raw_spins, spins, bytes, flags);
-        if (st) return st;
-        ICM_CUDA(ctx, icm::launch_pack_spins(b->raw_spins, P.spins, P.pos2site, b->n_inst, P.R, P.G, P.N,
-                                             ctx->stream));
+        const int8_t *src = spins;
+        if (!on_device(ctx, spins, flags)) {        // else packed straight from the caller's array
+            icm_status st = copy_in(ctx, b->raw_spins, spins, (size_t)b->n_inst * P.R * P.N, flags);
+            if (st) return st;
+            src = b->raw_spins;
+        }
+        ICM_CUDA(ctx, icm::launch_pack_spins(src, P.spins, P.pos2site, b->n_inst, P.R, P.G, P.N,
+                                             b->lattice == ICM_CHIMERA, ctx->stream));
     }
     ICM_CUDA(ctx, icm::launch_init_energies(P, b->gauss, ctx->stream));
     return ICM_OK;
@@ -953,10 +969,14 @@ icm_status icm_read_spins(icm_batch *b, int8_t *out, uint32_t flags)
 {
     if (!b || !out) return ICM_ERR_ARG;
     icm::KParams &P = b->kp;
-    ICM_CUDA(b->ctx, icm::launch_unpack_spins(P.spins, b->raw_spins, P.pos2site, b->n_inst, P.R, P.G, P.N,
-                                              b->ctx->stream));
-    icm_status st = copy_out(b->ctx, out, b->raw_spins, (size_t)b->n_inst * P.R * P.N, flags);
-    if (st) return st;
+    // straight into the caller's array where its address allows 4-byte stores
+    const bool direct = on_device(b->ctx, out, flags) && (uintptr_t)out % 4 == 0;
+    ICM_CUDA(b->ctx, icm::launch_unpack_spins(P.spins, direct ? out : b->raw_spins, P.pos2site, b->n_inst, P.R, P.G,
+                                              P.N, b->lattice == ICM_CHIMERA, b->ctx->stream));
+    if (!direct) {
+        icm_status st = copy_out(b->ctx, out, b->raw_spins, (size_t)b->n_inst * P.R * P.N, flags);
+        if (st) return st;
+    }
     ICM_CUDA(b->ctx, cudaStreamSynchronize(b->ctx->stream));
     return ICM_OK;
 }
@@ -965,9 +985,12 @@ icm_status icm_read_energies(icm_batch *b, double *out, uint32_t flags)
 {
     if (!b || !out) return ICM_ERR_ARG;
     icm::KParams &P = b->kp;
-    ICM_CUDA(b->ctx, icm::launch_energies_to_double(P, b->gauss, b->raw_E, b->ctx->stream));
-    icm_status st = copy_out(b->ctx, out, b->raw_E, (size_t)b->n_inst * P.R * sizeof(double), flags);
-    if (st) return st;
+    const bool direct = on_device(b->ctx, out, flags) && (uintptr_t)out % sizeof(double) == 0;
+    ICM_CUDA(b->ctx, icm::launch_energies_to_double(P, b->gauss, direct ? out : b->raw_E, b->ctx->stream));
+    if (!direct) {
+        icm_status st = copy_out(b->ctx, out, b->raw_E, (size_t)b->n_inst * P.R * sizeof(double), flags);
+        if (st) return st;
+    }
     ICM_CUDA(b->ctx, cudaStreamSynchronize(b->ctx->stream));
     return ICM_OK;
 }
@@ -1150,7 +1173,8 @@ icm_status icm_batch_set_slot(icm_batch *b, int32_t slot, const void *couplings,
     if (spins) {
         int8_t *raw_s = b->raw_spins + (size_t)slot * P.R * P.N;
         if ((st = copy_in(ctx, raw_s, spins, (size_t)P.R * P.N, flags))) return st;
-        ICM_CUDA(ctx, icm::launch_pack_spins(raw_s, sp, P.pos2site, 1, P.R, P.G, P.N, ctx->stream));
+        ICM_CUDA(ctx, icm::launch_pack_spins(raw_s, sp, P.pos2site, 1, P.R, P.G, P.N, b->lattice == ICM_CHIMERA,
+                                             ctx->stream));
     } else {
         ICM_CUDA(ctx, cudaMemsetAsync(sp, 0, (size_t)P.G * P.N * 4, ctx->stream));
     }

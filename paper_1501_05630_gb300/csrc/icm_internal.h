@@ -214,10 +214,12 @@ int wide_scratch_words(int N);
 cudaError_t fused_occupancy(bool gauss, int Z, bool wide, int threads, int smem, int *ctas_per_sm);
 cudaError_t launch_fused(const KParams &P, bool gauss, int threads, int grid, uint32_t n_sweeps,
                          cudaStream_t st);
+// Spins int8 [n_inst][R][N] by site <-> packed words [n_inst][G][N] by position
+// (cells: chimera).  Unpacking writes 4 bytes at a time: dst is 4-byte aligned.
 cudaError_t launch_pack_spins(const int8_t *src, uint32_t *dst, const uint16_t *pos2site, int n_inst,
-                              int R, int G, int N, cudaStream_t st);
+                              int R, int G, int N, bool cells, cudaStream_t st);
 cudaError_t launch_unpack_spins(const uint32_t *src, int8_t *dst, const uint16_t *pos2site, int n_inst,
-                                int R, int G, int N, cudaStream_t st);
+                                int R, int G, int N, bool cells, cudaStream_t st);
 cudaError_t launch_expand_couplings(const void *bond_J, bool gauss, const int32_t *edge_bond, int n_inst,
                                     int N, int Z, int Nb, float *Jd, uint8_t *Jb, cudaStream_t st);
 // Per-instance tables of a diluted batch from the bond couplings: neighbour

@@ -121,7 +121,8 @@ extern "C" icm_status icm_energies_static(icm_ctx *ctx, int32_t lattice, int32_t
     if (e == cudaSuccess)
         e = icm::launch_expand_couplings(couplings, gauss, (const int32_t *)(base + o_edge), n_inst, N, Z, tab.Nb,
                                          const_cast<float *>(P.Jd), const_cast<uint8_t *>(P.Jb), st);
-    if (e == cudaSuccess) e = icm::launch_pack_spins(spins, P.spins, P.pos2site, n_inst, n_rep, G, N, st);
+    if (e == cudaSuccess) e = icm::launch_pack_spins(spins, P.spins, P.pos2site, n_inst, n_rep, G, N,
+                                                        lattice == ICM_CHIMERA, st);
     if (e == cudaSuccess) e = icm::launch_init_energies(P, gauss, st);
     if (e == cudaSuccess) e = icm::launch_energies_to_double(P, gauss, out, st);
     // the host tables above are pageable memory read by the copies: wait before they go out of scope

@@ -1120,34 +1120,76 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_kernel(const __grid_cons
 #if ICM_PART == 0
 // ---------------------------------------------------------------------------
 // Layout kernels (run at load/read time, not per sweep).
-__global__ void pack_spins_kernel(const int8_t *__restrict__ src, uint32_t *__restrict__ dst,
-                                  const uint16_t *__restrict__ pos2site, int n_inst, int R, int G, int N)
+// A thread takes four consecutive sites of one instance and one word of 32
+// replicas, so that each replica's spins are read or written as 4 bytes a
+// lane, 128 a warp (N is a multiple of 4).  Bound by memory; before, a thread
+// took one position, and its bytes of consecutive sites went out one by one:
+// 16 sweeps of 10^4 chimera C_8 instances with 60 replicas and the read of
+// their 307 MB of spins took 10.96 ms and take 9.67 (unpacked straight into the
+// caller's device array).
+// The position of a site: on the lattices (even L) sites 2i and 2i + 1 have
+// opposite colours, in a chimera cell each shore has one, so a site's index
+// within its colour follows from the site, and the colour from one entry of
+// pos2site.
+__device__ __forceinline__ int site_pos(const uint16_t *__restrict__ pos2site, int site, int half, bool cells)
 {
-    const size_t total = (size_t)n_inst * G * N;
+    const int i = cells ? ((site >> 3) << 2) | (site & 3) : site >> 1;
+    return __ldg(pos2site + i) == site ? i : half + i;
+}
+
+__global__ void __launch_bounds__(256) pack_spins_kernel(const int8_t *__restrict__ src, uint32_t *__restrict__ dst,
+                                                         const uint16_t *__restrict__ pos2site, int n_inst, int R,
+                                                         int G, int N, int cells)
+{
+    const int quads = N >> 2, half = N >> 1;
+    const size_t total = (size_t)n_inst * G * quads;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
-        const int p = (int)(idx % N);
-        const int g = (int)((idx / N) % G);
-        const size_t inst = idx / ((size_t)N * G);
-        const int site = pos2site[p];
-        uint32_t w = 0;
-        for (int b = 0; b < 32 && 32 * g + b < R; ++b)
-            w |= (uint32_t)(src[(inst * R + 32 * g + b) * N + site] < 0) << b;
-        dst[idx] = w;
+        const size_t row = idx / quads;
+        const int q = (int)(idx - row * quads);
+        const size_t inst = row / G;
+        const int g = (int)(row - inst * G), nb = min(32, R - 32 * g);
+        const int8_t *s = src + (inst * R + 32 * g) * N + 4 * q;
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
+        if (((uintptr_t)src & 3u) == 0) {
+#pragma unroll 8
+            for (int b = 0; b < nb; ++b) {
+                const uint32_t v = *reinterpret_cast<const uint32_t *>(s + (size_t)b * N);   // spin -1: sign bit set
+#pragma unroll
+                for (int i = 0; i < 4; ++i) w[i] |= ((v >> (8 * i + 7)) & 1u) << b;
+            }
+        } else {                           // a caller's array at an odd address
+            for (int b = 0; b < nb; ++b)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) w[i] |= (uint32_t)(s[(size_t)b * N + i] < 0) << b;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) dst[row * N + site_pos(pos2site, 4 * q + i, half, cells)] = w[i];
     }
 }
 
-__global__ void unpack_spins_kernel(const uint32_t *__restrict__ src, int8_t *__restrict__ dst,
-                                    const uint16_t *__restrict__ pos2site, int n_inst, int R, int G, int N)
+__global__ void __launch_bounds__(256) unpack_spins_kernel(const uint32_t *__restrict__ src, int8_t *__restrict__ dst,
+                                                           const uint16_t *__restrict__ pos2site, int n_inst, int R,
+                                                           int G, int N, int cells)
 {
-    const size_t total = (size_t)n_inst * R * N;
+    const int quads = N >> 2, half = N >> 1;
+    const size_t total = (size_t)n_inst * G * quads;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
-        const int p = (int)(idx % N);
-        const int r = (int)((idx / N) % R);
-        const size_t inst = idx / ((size_t)N * R);
-        const uint32_t w = src[(inst * G + (r >> 5)) * N + p];
-        dst[(inst * R + r) * N + pos2site[p]] = ((w >> (r & 31)) & 1u) ? (int8_t)-1 : (int8_t)1;
+        const size_t row = idx / quads;
+        const int q = (int)(idx - row * quads);
+        const size_t inst = row / G;
+        const int g = (int)(row - inst * G), nb = min(32, R - 32 * g);
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = src[row * N + site_pos(pos2site, 4 * q + i, half, cells)];
+        int8_t *d = dst + (inst * R + 32 * g) * N + 4 * q;
+#pragma unroll 4
+        for (int b = 0; b < nb; ++b) {
+            const uint32_t v = ((w[0] >> b) & 1u) | (((w[1] >> b) & 1u) << 8) | (((w[2] >> b) & 1u) << 16) |
+                               (((w[3] >> b) & 1u) << 24);
+            *reinterpret_cast<uint32_t *>(d + (size_t)b * N) = v * 0xFEu + 0x01010101u;   // bytes 0x01 or 0xFF
+        }
     }
 }
 
@@ -1213,52 +1255,99 @@ __global__ void expand_dilution_kernel(const void *__restrict__ bondJ, int gauss
             once += present && p < q;
         }
         zdeg_inst[idx] = (uint8_t)deg;
+        // one pair of atomics per warp where its sites belong to one instance
+        // (one per site before: 1000 3D L=8 instances in 35 us)
+        const unsigned on = __activemask();
+        const int first = __ffs(on) - 1;
+        if (__all_sync(on, inst == __shfl_sync(on, inst, first))) {
+            once = __reduce_add_sync(on, once);
+            invalid = __reduce_add_sync(on, invalid);
+            if ((int)(threadIdx.x & 31) != first) once = invalid = 0;
+        }
         if (once) atomicAdd(&nb_inst[inst], once);
         if (invalid) atomicAdd(&bad[inst], invalid);
     }
 }
 
 // Energies of every replica from the spins: E = -sum over colour-1 sites of
-// s_i h_i (every bond joins the two colours).  One CTA per instance.
-template <bool GAUSS, int Z>
-__global__ void init_energies_kernel(const KParams P)
+// s_i h_i (every bond joins the two colours).  One CTA of kMaxThreads threads
+// per instance and share of replicas: 32 (+-J, bit-sliced: U per replica, E =
+// 2 U - bonds present) or 16 (Gaussian).  A thread's sites and neighbours are
+// read once for all replicas of the share; before, each replica went over them
+// on its own with a block reduction after it: 1000 3D Gaussian L=8 instances
+// with 48 replicas took 74 us.  The Gaussian sums keep their order: a thread's
+// sites in turn, then halving strides 64, 32, .., 1 over the threads.
+template <int Z>
+__global__ void __launch_bounds__(kMaxThreads) init_energies_gauss_kernel(const KParams P)
 {
-    using ET = typename std::conditional<GAUSS, float, int>::type;
-    __shared__ ET red[kMaxThreads];
-    const int N = P.N, half = P.half;
+    constexpr int kShare = 16;
+    __shared__ float red[kShare][kMaxThreads];
+    const int N = P.N, half = P.half, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int r0 = blockIdx.y * kShare, nr = min(kShare, P.R - r0), sh = r0 & 31;
     for (int slot = blockIdx.x; slot < P.n_inst; slot += gridDim.x) {
-        const uint32_t *s = P.spins + (size_t)slot * P.G * N;
+        const uint32_t *sg = P.spins + ((size_t)slot * P.G + (r0 >> 5)) * N;
         const uint16_t *nbr = P.diluted ? P.nbr_inst + (size_t)slot * N * Z : P.nbr;   // absent bonds: self
-        for (int r = 0; r < P.R; ++r) {
-            const uint32_t *sg = s + (r >> 5) * N;
-            const int b = r & 31;
-            ET acc = ET(0);
-            for (int p = half + threadIdx.x; p < N; p += blockDim.x) {
-                const int si = ((sg[p] >> b) & 1u) ? -1 : 1;
-                for (int d = 0; d < Z; ++d) {
-                    const int q = nbr[p * Z + d];
-                    const int sj = ((sg[q] >> b) & 1u) ? -1 : 1;
-                    if constexpr (GAUSS) {
-                        acc -= P.Jd[((size_t)slot * N + p) * Z + d] * (float)(si * sj);
-                    } else {
-                        if (q == p) continue;
-                        const int J = ((P.Jb[(size_t)slot * N + p] >> d) & 1u) ? -1 : 1;
-                        acc -= J * si * sj;
-                    }
-                }
+        float acc[kShare];
+#pragma unroll
+        for (int b = 0; b < kShare; ++b) acc[b] = 0.f;
+        for (int p = half + threadIdx.x; p < N; p += blockDim.x) {
+            const uint32_t sw = sg[p] >> sh;
+            int q[Z];
+            load_nbrs<Z>(nbr, p, q);
+#pragma unroll
+            for (int d = 0; d < Z; ++d) {
+                const float J = P.Jd[((size_t)slot * N + p) * Z + d];
+                const uint32_t x = sw ^ (sg[q[d]] >> sh);
+#pragma unroll
+                for (int b = 0; b < kShare; ++b) acc[b] -= ((x >> b) & 1u) ? -J : J;
             }
-            red[threadIdx.x] = acc;
-            __syncthreads();
-            for (int s2 = blockDim.x / 2; s2 > 0; s2 >>= 1) {
-                if (threadIdx.x < s2) red[threadIdx.x] += red[threadIdx.x + s2];
-                __syncthreads();
-            }
-            if (threadIdx.x == 0) {
-                if constexpr (GAUSS) P.Ef[(size_t)slot * P.R + r] = red[0];
-                else P.Ei[(size_t)slot * P.R + r] = red[0];
-            }
-            __syncthreads();
         }
+#pragma unroll
+        for (int b = 0; b < kShare; ++b) red[b][threadIdx.x] = acc[b];
+        __syncthreads();
+        for (int b = warp; b < nr; b += kMaxThreads / 32) {
+            float v = (red[b][lane] + red[b][lane + 64]) + (red[b][lane + 32] + red[b][lane + 96]);
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) v += __shfl_down_sync(kFull, v, o);
+            if (lane == 0) P.Ef[(size_t)slot * P.R + r0 + b] = v;
+        }
+        __syncthreads();
+    }
+}
+
+template <int Z>
+__global__ void __launch_bounds__(kMaxThreads) init_energies_pmj_kernel(const KParams P)
+{
+    __shared__ int sum[32];
+    const int N = P.N, half = P.half, lane = threadIdx.x & 31;
+    const int r0 = blockIdx.y * 32, nr = min(32, P.R - r0);
+    for (int slot = blockIdx.x; slot < P.n_inst; slot += gridDim.x) {
+        const uint32_t *sg = P.spins + ((size_t)slot * P.G + blockIdx.y) * N;
+        const uint16_t *nbr = P.diluted ? P.nbr_inst + (size_t)slot * N * Z : P.nbr;   // absent bonds: self
+        if (threadIdx.x < 32) sum[threadIdx.x] = 0;
+        __syncthreads();
+        // at most 255 / Z sites to a set of counters
+        for (int p0 = half; p0 < N; p0 += (255 / Z) * kMaxThreads) {
+            uint32_t pl[kPlanes];
+#pragma unroll
+            for (int i = 0; i < kPlanes; ++i) pl[i] = 0u;
+            const int p1 = min(N, p0 + (255 / Z) * kMaxThreads);
+            for (int p = p0 + threadIdx.x; p < p1; p += kMaxThreads) {
+                const uint32_t sw = sg[p], jb = P.Jb[(size_t)slot * N + p];
+                int q[Z];
+                load_nbrs<Z>(nbr, p, q);
+                uint32_t u[Z], c0, c1, c2, c3;
+#pragma unroll
+                for (int d = 0; d < Z; ++d) u[d] = sw ^ sg[q[d]] ^ (0u - ((jb >> d) & 1u));
+                csa_count<Z>(u, c0, c1, c2, c3);
+                vadd4(pl, c0, c1, c2, c3);
+            }
+            atomicAdd(&sum[lane], warp_vcount(pl, kPlanes, lane));
+        }
+        __syncthreads();
+        if ((int)threadIdx.x < nr)
+            P.Ei[(size_t)slot * P.R + r0 + threadIdx.x] = 2 * sum[threadIdx.x] - (P.diluted ? P.nb_inst[slot] : P.Nb);
+        __syncthreads();
     }
 }
 
@@ -1394,16 +1483,18 @@ cudaError_t team_occupancy(bool gauss, int Z, int smem, int *ctas)
 }
 
 cudaError_t launch_pack_spins(const int8_t *src, uint32_t *dst, const uint16_t *pos2site, int n_inst, int R, int G,
-                              int N, cudaStream_t st)
+                              int N, bool cells, cudaStream_t st)
 {
-    pack_spins_kernel<<<grid_for((size_t)n_inst * G * N, 256), 256, 0, st>>>(src, dst, pos2site, n_inst, R, G, N);
+    pack_spins_kernel<<<grid_for((size_t)n_inst * G * (N / 4), 256), 256, 0, st>>>(src, dst, pos2site, n_inst, R, G, N,
+                                                                                  cells ? 1 : 0);
     return cudaGetLastError();
 }
 
 cudaError_t launch_unpack_spins(const uint32_t *src, int8_t *dst, const uint16_t *pos2site, int n_inst, int R, int G,
-                                int N, cudaStream_t st)
+                                int N, bool cells, cudaStream_t st)
 {
-    unpack_spins_kernel<<<grid_for((size_t)n_inst * R * N, 256), 256, 0, st>>>(src, dst, pos2site, n_inst, R, G, N);
+    unpack_spins_kernel<<<grid_for((size_t)n_inst * G * (N / 4), 256), 256, 0, st>>>(src, dst, pos2site, n_inst, R, G, N,
+                                                                                    cells ? 1 : 0);
     return cudaGetLastError();
 }
 
@@ -1427,19 +1518,19 @@ cudaError_t launch_expand_dilution(const void *bond_J, bool gauss, const int32_t
 
 cudaError_t launch_init_energies(const KParams &P, bool gauss, cudaStream_t st)
 {
-    const int grid = P.n_inst < 152 * 8 ? P.n_inst : 152 * 8;
+    const dim3 grid((unsigned)(P.n_inst < 152 * 8 ? P.n_inst : 152 * 8), (unsigned)((P.R + (gauss ? 15 : 31)) / (gauss ? 16 : 32)));
     switch (P.Z) {
     case 4:
-        if (gauss) init_energies_kernel<true, 4><<<grid, kMaxThreads, 0, st>>>(P);
-        else init_energies_kernel<false, 4><<<grid, kMaxThreads, 0, st>>>(P);
+        if (gauss) init_energies_gauss_kernel<4><<<grid, kMaxThreads, 0, st>>>(P);
+        else init_energies_pmj_kernel<4><<<grid, kMaxThreads, 0, st>>>(P);
         break;
     case 6:
-        if (gauss) init_energies_kernel<true, 6><<<grid, kMaxThreads, 0, st>>>(P);
-        else init_energies_kernel<false, 6><<<grid, kMaxThreads, 0, st>>>(P);
+        if (gauss) init_energies_gauss_kernel<6><<<grid, kMaxThreads, 0, st>>>(P);
+        else init_energies_pmj_kernel<6><<<grid, kMaxThreads, 0, st>>>(P);
         break;
     case 8:
-        if (gauss) init_energies_kernel<true, 8><<<grid, kMaxThreads, 0, st>>>(P);
-        else init_energies_kernel<false, 8><<<grid, kMaxThreads, 0, st>>>(P);
+        if (gauss) init_energies_gauss_kernel<8><<<grid, kMaxThreads, 0, st>>>(P);
+        else init_energies_pmj_kernel<8><<<grid, kMaxThreads, 0, st>>>(P);
         break;
     default:
         return cudaErrorInvalidValue;
