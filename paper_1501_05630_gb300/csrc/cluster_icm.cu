@@ -4,24 +4,34 @@
 //
 // CTA r of the cluster owns the positions [c half + r hs, c half + (r+1) hs)
 // of each colour c and keeps their spin words, couplings, cluster words and
-// neighbour table in its own shared memory.  A neighbour's word is read
-// through the cluster's distributed shared memory: the neighbour table holds
-// the 32-bit cluster-window address (mapa) of the neighbour's spin word in
-// its owner CTA, read with ld.shared::cluster.  Phases are separated by
-// cluster barriers (barrier.cluster arrive.release / wait.acquire):
-//  * sweep: colour 0, barrier, colour 1; each CTA sums its sites' energies,
-//    barrier, every CTA adds the K shares in rank order (the same E in all);
-//  * ICM: per-CTA overlap counts, barrier, every CTA finds the seed's owner
-//    from the K counts (position order = (colour, rank, local)), the owner
-//    plants it, barrier; growth in rounds of a few in-place scans without
+// neighbour table in its own shared memory, with copies (the halo) of the
+// spin and cluster words of every site in another CTA that borders one of
+// its own.  The neighbour table holds the shared-memory offset of the
+// neighbour's cluster word, own or halo, in 16 bits, so every neighbour access
+// is a plain shared-memory load; reading the owner's word through the cluster
+// window (ld.shared::cluster) cost two to nine times the latency and most of
+// the growth's time.  What changes a word keeps its copies up to date:
+//  * the sweep and the growth store a changed border word into the halos that
+//    hold it (st.shared::cluster; one writer per word, nobody waits for it);
+//  * step 2a, the cluster flip and the PT permutation are the same function of
+//    a site's words everywhere, so every CTA applies them to its halo itself.
+// Phases are separated by cluster barriers (barrier.cluster arrive.release /
+// wait.acquire):
+//  * sweep: colour 0, barrier, colour 1; each CTA stores its energy sums into
+//    every CTA, barrier, every CTA adds the K shares in rank order (the same E
+//    in all);
+//  * ICM: overlap counts stored into every CTA, barrier, every CTA finds the
+//    seed's owner from the K counts (position order = (colour, rank, local)),
+//    the owner plants it; growth in rounds of a few in-place scans without
 //    barriers, each round ending with a barrier after which every CTA reads
-//    the round stamp that growing warps pushed into all CTAs; flip, barrier,
-//    copy-a energies summed as above;
+//    the round stamp that growing warps stored into all CTAs; flip, copy-a
+//    energies exchanged as above;
 //  * PT: every CTA holds the same energies and draws the same numbers, so
-//    all make the same decisions and permute their own words; barrier;
-//  * observables: per-CTA counts, barrier, rank 0 accumulates.
-// Every buffer another CTA reads is rewritten only after a barrier that
-// both have passed since the read.  Random keys are those of the
+//    all make the same decisions and permute their own and halo words;
+//  * observables: counts stored into rank 0, the barrier that ends the step,
+//    rank 0 accumulates.
+// Every buffer another CTA writes is written only after a barrier that
+// both have passed since its last read.  Random keys are those of the
 // single-CTA kernels, so the chain is the same, bit for bit for +-J.
 #include "icm_internal.h"
 #include "icm_device.cuh"
@@ -56,6 +66,7 @@ __device__ __forceinline__ uint32_t cl_count()
 // across the cluster (release before, acquire after).
 __device__ __forceinline__ void cl_sync()
 {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
@@ -68,6 +79,7 @@ __device__ __forceinline__ uint32_t cl_map(uint32_t local, uint32_t rank)
     return r;
 }
 
+// (trace only: everything else is stored into the CTA that reads it)
 __device__ __forceinline__ uint32_t cl_ld(uint32_t addr)
 {
     uint32_t v;
@@ -106,25 +118,19 @@ __device__ __forceinline__ uint32_t cl_cas(uint32_t addr, uint32_t cmp, uint32_t
     return old;
 }
 
-template <typename T>
-__device__ __forceinline__ T cl_ldT(uint32_t addr)
-{
-    const uint32_t v = cl_ld(addr);
-    if constexpr (std::is_same<T, float>::value) return __uint_as_float(v);
-    else return (T)(int)v;
-}
-
 // This CTA's view: pointers into its shared memory and cluster addresses.
 struct CS {
-    uint32_t *s, *C, *nb;
+    uint32_t *s, *C;
+    uint16_t *nb, *xoff;
+    uint32_t *xl, *hlab;
     float *Jd;
     uint8_t *Jb, *zdeg;
-    void *E, *Epart, *Esw, *Epair, *esum;
+    void *E, *Epart, *Esw, *Epair, *esum;   // Esw [K][R], Epair [K][32]: every CTA's share
     uint32_t *thr;
     float *b2l;
     uint32_t *mask, *lab, *sadr, *sroot;
     uint16_t *gord;
-    int *cntloc, *flags, *seed, *csz, *cnt_n, *cnt_d;
+    int *cntloc, *cntobs, *flags, *seed, *csz, *cnt_n, *cnt_d;   // cntloc [K][2][32], cntobs [2][K][2][32]
     uint32_t *flipw;
     uint32_t *swap_x;
     uint64_t *swap_mask;
@@ -132,9 +138,10 @@ struct CS {
     long long *acc64, *nmeas;
     unsigned long long *icmst;
     uint32_t base;        // shared-window address of this CTA's dynamic shared memory
-    uint32_t dCs;         // a neighbour-table entry (the neighbour's cluster word) minus this: its spin word 0
+    uint32_t win;         // where this CTA's shared window starts (its rank << 24)
+    uint32_t dCs;         // a cluster word's address minus this: the site's spin word 0
     uint32_t rank, K;
-    int hs, nls;
+    int hs, nls, ns;      // ns: own and halo sites, the stride of the two spin words
 };
 
 __device__ __forceinline__ CS make_cs(unsigned char *smem, const ClusterLayout &L)
@@ -142,7 +149,10 @@ __device__ __forceinline__ CS make_cs(unsigned char *smem, const ClusterLayout &
     CS S;
     S.s = (uint32_t *)(smem + L.s);
     S.C = (uint32_t *)(smem + L.C);
-    S.nb = (uint32_t *)(smem + L.nb);
+    S.nb = (uint16_t *)(smem + L.nb);
+    S.xoff = (uint16_t *)(smem + L.xoff);
+    S.xl = (uint32_t *)(smem + L.xl);
+    S.hlab = (uint32_t *)(smem + L.hlab);
     S.Jd = (float *)(smem + L.coup);
     S.Jb = (uint8_t *)(smem + L.coup);
     S.zdeg = (uint8_t *)(smem + L.zdeg);
@@ -159,6 +169,7 @@ __device__ __forceinline__ CS make_cs(unsigned char *smem, const ClusterLayout &
     S.sroot = (uint32_t *)(smem + L.sroot);
     S.gord = L.gord >= 0 ? (uint16_t *)(smem + L.gord) : nullptr;
     S.cntloc = (int *)(smem + L.cntloc);
+    S.cntobs = (int *)(smem + L.cntobs);
     S.flags = (int *)(smem + L.flags);
     S.seed = (int *)(smem + L.seed);
     S.csz = (int *)(smem + L.csz);
@@ -172,50 +183,87 @@ __device__ __forceinline__ CS make_cs(unsigned char *smem, const ClusterLayout &
     S.nmeas = (long long *)(smem + L.nmeas);
     S.icmst = (unsigned long long *)(smem + L.icmst);
     S.base = (uint32_t)__cvta_generic_to_shared(smem);
+    S.win = S.base & 0xFF000000u;
     S.dCs = (uint32_t)(L.C - L.s);
     S.rank = cl_rank();
     S.K = (uint32_t)L.K;
     S.hs = L.hs;
     S.nls = L.nls;
+    S.ns = L.ns;
     return S;
 }
 
-// The Z neighbour addresses of own site li, in 16-byte loads when Z is a
-// multiple of 4 (a row starts 16-byte aligned), else 8-byte loads: one
-// shared-memory instruction instead of four for a 2D site.
+// The neighbour row of own site li: the offsets of the neighbours' cluster
+// words in the CTA's shared window, two to a 32-bit word.
 template <int Z>
-__device__ __forceinline__ void nb_row(const uint32_t *nb, int li, uint32_t (&e)[Z])
+__device__ __forceinline__ void nb_row(const uint16_t *nb, int li, uint32_t (&e)[Z / 2])
 {
-    const uint32_t *row = nb + li * Z;
-    if constexpr (Z % 4 == 0) {
-#pragma unroll
-        for (int d = 0; d < Z; d += 4) {
-            const uint4 v = *reinterpret_cast<const uint4 *>(row + d);
-            e[d] = v.x;
-            e[d + 1] = v.y;
-            e[d + 2] = v.z;
-            e[d + 3] = v.w;
-        }
-    } else if constexpr (Z % 2 == 0) {
-#pragma unroll
-        for (int d = 0; d < Z; d += 2) {
-            const uint2 v = *reinterpret_cast<const uint2 *>(row + d);
-            e[d] = v.x;
-            e[d + 1] = v.y;
-        }
+    const uint16_t *row = nb + li * Z;
+    if constexpr (Z == 4) {
+        const uint2 v = *reinterpret_cast<const uint2 *>(row);
+        e[0] = v.x;
+        e[1] = v.y;
+    } else if constexpr (Z == 8) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(row);
+        e[0] = v.x;
+        e[1] = v.y;
+        e[2] = v.z;
+        e[3] = v.w;
     } else {
 #pragma unroll
-        for (int d = 0; d < Z; ++d) e[d] = row[d];
+        for (int i = 0; i < Z / 2; ++i) e[i] = reinterpret_cast<const uint32_t *>(row)[i];
     }
 }
+// The shared-window address of entry d.  In a cluster the window of CTA r starts
+// at r << 24 (win, S.win): the 16-bit offset alone would name another CTA's
+// window, which ld.shared must not touch.
+__device__ __forceinline__ uint32_t nb_addr(uint32_t pair, int d, uint32_t win)
+{
+    return __byte_perm(pair, win, (d & 1) ? 0x7632 : 0x7610);
+}
 
-// Sum over the cluster, in rank order, of the ET value at byte offset `off`
-// of every CTA's shared memory (the same result in every CTA).
+// Spin word `off` bytes from the cluster word of each neighbour of li.
+template <int Z>
+__device__ __forceinline__ void nb_words(const CS &S, int li, uint32_t off, uint32_t (&w)[Z])
+{
+    uint32_t e[Z / 2];
+    nb_row<Z>(S.nb, li, e);
+#pragma unroll
+    for (int d = 0; d < Z; ++d) w[d] = sh_ld(nb_addr(e[d >> 1], d, S.win) + off);
+}
+
+// Apply f to the addresses of the copies of own site li's cluster word in the
+// halos of other CTAs (none for an inner site).  The last one has bit 0 set.
+template <typename F>
+__device__ __forceinline__ void for_copies(const CS &S, int li, F f)
+{
+    uint32_t i = S.xoff[li];
+    if (i == 0xffffu) return;
+    uint32_t a;
+    do {
+        a = S.xl[i++];
+        f(a & ~1u);
+    } while (!(a & 1u));
+}
+
+// Store v at word `i` of row `rank` of the [K][n] array at byte offset `off`
+// of every CTA's shared memory.
 template <typename ET>
-__device__ __forceinline__ ET cl_sum(const CS &S, int off)
+__device__ __forceinline__ void cl_share(const CS &S, int off, int n, int i, ET v)
+{
+    uint32_t w;
+    if constexpr (std::is_same<ET, float>::value) w = __float_as_uint(v);
+    else w = (uint32_t)v;
+    const uint32_t a = S.base + off + 4u * (uint32_t)((int)S.rank * n + i);
+    for (uint32_t r = 0; r < S.K; ++r) cl_st(cl_map(a, r), w);
+}
+
+// Sum of entry i over the K rows, in rank order (the same result in every CTA).
+template <typename ET>
+__device__ __forceinline__ ET row_sum(const CS &S, const void *rows, int n, int i)
 {
     ET v = ET(0);
-    for (uint32_t r = 0; r < S.K; ++r) v += cl_ldT<ET>(cl_map(S.base + off, r));
+    for (uint32_t r = 0; r < S.K; ++r) v += ((const ET *)rows)[(int)r * n + i];
     return v;
 }
 
@@ -227,145 +275,172 @@ __device__ __forceinline__ int pos_of(const KParams &P, const CS &S, int li)
 }
 
 // ---------------------------------------------------------------------------
-// Step 1, one 16-bit pass of colour COLOR over word g (see sweep_pass in
-// pt_icm.cu: the same arithmetic, with neighbour words read through the
-// cluster window).
-template <bool GAUSS, int Z, bool DIL>
-__device__ __forceinline__ void cl_sweep_pass(const KParams &P, const CS &S, uint32_t t, uint32_t inst, int g,
+// Step 1, Gaussian couplings: one 16-bit pass of colour COLOR over word g
+// (see gauss_pass in pt_icm.cu).
+template <int Z, bool DIL>
+__device__ __forceinline__ void cl_gauss_pass(const KParams &P, const CS &S, uint32_t t, uint32_t inst, int g,
                                               int COLOR, int H, bool tie)
 {
-    using ET = typename std::conditional<GAUSS, float, int>::type;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nth = blockDim.x;
     const int rbase = 32 * g + 16 * H;
     const int sh0 = 16 * H;
     const int npairs8 = (P.R - rbase + 7) >> 3;
-    const uint32_t goff = (uint32_t)(g * S.nls * 4) - S.dCs;   // neighbour entry -> its spin word g
-    uint32_t *sg = S.s + g * S.nls;
-    ET acc[16];
+    const uint32_t goff = (uint32_t)(g * S.ns * 4) - S.dCs;    // cluster word -> spin word g
+    uint32_t *sg = S.s + g * S.ns;
+    float acc[16];
 #pragma unroll
-    for (int b = 0; b < 16; ++b) acc[b] = ET(0);
+    for (int b = 0; b < 16; ++b) acc[b] = 0.f;
     for (int j = threadIdx.x; j < S.hs; j += nth) {
         const int li = COLOR * S.hs + j;
         const uint32_t sw0 = sg[li];
         const uint32_t sw = sw0 >> sh0;
         const uint32_t site = __ldg(P.pos2site + pos_of(P, S, li));
         uint32_t nw[Z];
-        nb_row<Z>(S.nb, li, nw);
-#pragma unroll
-        for (int d = 0; d < Z; ++d) nw[d] = cl_ld(nw[d] + goff);
+        nb_words<Z>(S, li, goff, nw);
         uint32_t flip = 0;
-        if constexpr (GAUSS) {
-            float J2[Z];
-            float Jsum = 0.f;
+        float J[Z];
+        float Jsum = 0.f;
 #pragma unroll
-            for (int d = 0; d < Z; ++d) {
-                nw[d] >>= sh0;
-                const float J = S.Jd[li * Z + d];
-                Jsum += J;
-                J2[d] = 2.f * J;
-            }
-            const float *b2l = S.b2l + rbase;
+        for (int d = 0; d < Z; ++d) {
+            nw[d] >>= sh0;
+            J[d] = S.Jd[li * Z + d];
+            Jsum += J[d];
+        }
+        const float *b2l = S.b2l + rbase;
 #pragma unroll
-            for (int qq = 0; qq < 2; ++qq) {
-                if (qq < npairs8) {
-                    uint32_t x[4], y[4];
-                    philox10x2(site, t, (uint32_t)(rbase >> 2) + 2 * qq, inst, P.key, x, y);
-                    uint32_t f8 = 0u;
+        for (int qq = 0; qq < 2; ++qq) {
+            if (qq < npairs8) {
+                uint32_t x[4], y[4];
+                philox10x2(site, t, (uint32_t)(rbase >> 2) + 2 * qq, inst, P.key, x, y);
+                uint32_t f8 = 0u;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int b = 8 * qq + i;
-                        float h = Jsum;
+                for (int i = 0; i < 8; ++i) {
+                    const int b = 8 * qq + i;
+                    float h = Jsum;
 #pragma unroll
-                        for (int d = 0; d < Z; ++d)
-                            if ((nw[d] >> b) & 1u) h -= J2[d];
-                        const float sh = ((sw >> b) & 1u) ? -h : h;
-                        const uint32_t xr = i < 4 ? x[i] : y[i - 4];
-                        const uint32_t thr = __float2uint_rz(ex2_approx(fmaf(b2l[b], sh, 32.f)));
-                        bool a;
-                        if constexpr (DIL)   // diluted instance: Delta E = 0 accepted with probability 1/2
-                            a = (sh < 0.f) || (sh == 0.f ? (!tie || xr < 0x80000000u) : (xr < thr));
-                        else
-                            a = (sh <= 0.f) || (xr < thr);
-                        f8 |= (uint32_t)a << i;
-                        acc[b] -= sh;
-                        if (a) acc[b] += 2.f * sh;
-                    }
-                    flip |= f8 << (8 * qq);
+                    for (int d = 0; d < Z; ++d)
+                        if ((nw[d] >> b) & 1u) h = fmaf(J[d], -2.f, h);
+                    const float sh = ((sw >> b) & 1u) ? -h : h;
+                    const uint32_t xr = i < 4 ? x[i] : y[i - 4];
+                    const uint32_t thr = __float2uint_rz(ex2_approx(fmaf(b2l[b], sh, 32.f)));
+                    bool a;
+                    if constexpr (DIL)   // diluted instance: Delta E = 0 accepted with probability 1/2
+                        a = (sh < 0.f) || (sh == 0.f ? (!tie || xr < 0x80000000u) : (xr < thr));
+                    else
+                        a = (sh <= 0.f) || (xr < thr);
+                    f8 |= (uint32_t)a << i;
+                    acc[b] -= sh;
+                    if (a) acc[b] += 2.f * sh;
                 }
-            }
-        } else {
-            uint32_t c0 = 0, c1 = 0, c2 = 0, c3 = 0;   // bit-planes of u = # unsatisfied bonds
-            const uint32_t jb = S.Jb[li];
-            uint32_t u[Z];
-#pragma unroll
-            for (int d = 0; d < Z; ++d) u[d] = sw0 ^ nw[d] ^ (0u - ((jb >> d) & 1u));
-            csa_count<Z>(u, c0, c1, c2, c3);
-            c0 >>= sh0;
-            c1 >>= sh0;
-            c2 >>= sh0;
-            c3 >>= sh0;
-            const int z = (!DIL && P.const_z) ? P.const_z : (int)S.zdeg[li];   // bonds present
-            // always accepted: m = z - 2u <= 0; on a diluted instance only m < 0
-            // (m = 0 takes the threshold entry 2^31, probability 1/2)
-            if constexpr (DIL) flip = ge_bitsliced(c0, c1, c2, c3, tie ? (z >> 1) + 1 : (z + 1) >> 1) & 0xFFFFu;
-            else if constexpr (Z > 7) flip = (c3 | c2) & 0xFFFFu;   // z = 8: u >= 4
-            else flip = ((z <= 4) ? (c2 | c1) : (c2 | (c1 & c0))) & 0xFFFFu;
-            constexpr int TS = thr_stride(Z);
-            const uint32_t *thr = S.thr + rbase * TS;
-#pragma unroll
-            for (int qq = 0; qq < 2; ++qq) {
-                if (qq < npairs8) {
-                    uint32_t x[4], y[4];
-                    philox10x2(site, t, (uint32_t)(rbase >> 2) + 2 * qq, inst, P.key, x, y);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int b = 8 * qq + i;
-                        const int u = (int)(((c0 >> b) & 1u) | (((c1 >> b) & 1u) << 1) | (((c2 >> b) & 1u) << 2) |
-                                            (((c3 >> b) & 1u) << 3));
-                        const int m = z - 2 * u;
-                        const uint32_t xr = i < 4 ? x[i] : y[i - 4];
-                        const uint32_t th = thr[b * TS + (m > 0 ? m : 0)];
-                        flip |= (uint32_t)(xr < th) << b;
-                        acc[b] += ((flip >> b) & 1u) ? m : -m;
-                    }
-                }
+                flip |= f8 << (8 * qq);
             }
         }
-        sg[li] = sw0 ^ (flip << sh0);
+        const uint32_t w = sw0 ^ (flip << sh0);
+        sg[li] = w;
+        for_copies(S, li, [&](uint32_t a) { cl_st(a + goff, w); });
     }
     if (COLOR == 1) {
-        const ET v = transpose_reduce16(acc, lane);
+        const float v = transpose_reduce16(acc, lane);
         const int r = rbase + (lane >> 1);
-        if (!(lane & 1) && r < P.R) ((ET *)S.Epart)[warp * P.R + r] = v;
+        if (!(lane & 1) && r < P.R) ((float *)S.Epart)[warp * P.R + r] = v;
     }
 }
 
-// Step 1 for all replicas; then every CTA's share of the energies, summed
-// over the cluster in rank order.
+// Step 1, +-J couplings: the replica groups [q0, q1) of word g of colour COLOR
+// (see pmj_pass in pt_icm.cu).  When warp groups share out the replicas
+// (`shared`), the flips go into the word by atomic XOR and the caller stores
+// the copies.
+template <int Z, bool DIL>
+__device__ __forceinline__ void cl_pmj_pass(const KParams &P, const CS &S, uint32_t t, uint32_t inst, int g, int COLOR,
+                                            int q0, int q1, int j0, int jstride, bool shared, bool tie)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t goff = (uint32_t)(g * S.ns * 4) - S.dCs;
+    uint32_t *sg = S.s + g * S.ns;
+    const int left = P.R - 32 * g;
+    const uint32_t live = left >= 32 ? kFull : (1u << left) - 1u;
+    const int end = 8 * q1 < left ? 8 * q1 : min(32, (left + 15) & ~15);
+    const uint32_t mine = (kFull >> (32 - end)) & (kFull << (8 * q0));
+    uint32_t pl[kPlanes];
+#pragma unroll
+    for (int i = 0; i < kPlanes; ++i) pl[i] = 0u;
+    for (int j = j0; j < S.hs; j += jstride) {
+        const int li = COLOR * S.hs + j;
+        const uint32_t sw = sg[li];
+        const uint32_t site = __ldg(P.pos2site + pos_of(P, S, li));
+        const uint32_t jb = S.Jb[li];
+        uint32_t u[Z], c[4];
+        nb_words<Z>(S, li, goff, u);
+#pragma unroll
+        for (int d = 0; d < Z; ++d) u[d] ^= sw ^ (0u - ((jb >> d) & 1u));
+        csa_count<Z>(u, c[0], c[1], c[2], c[3]);
+        const int z = (!DIL && Z != 6) ? Z : (!DIL && P.const_z) ? P.const_z : (int)S.zdeg[li];   // bonds present
+        const uint32_t flip = pmj_flips<Z, DIL>(c, z, tie, live, S.thr + 16 * g * kThrRow, site, t, 8u * (uint32_t)g,
+                                                inst, P.key, q0, q1) & mine;
+        if (shared) {
+            atomicXor(sg + li, flip);
+        } else {
+            sg[li] = sw ^ flip;
+            for_copies(S, li, [&](uint32_t a) { cl_st(a + goff, sw ^ flip); });
+        }
+        if (COLOR == 1) pmj_count(pl, c, z, flip, mine & live);
+    }
+    if (COLOR == 1) {
+        const int v = warp_vcount(pl, P.cnt_planes, lane);
+        if (lane < left) ((int *)S.Epart)[warp * P.R + 32 * g + lane] = v;
+    }
+}
+
+// Step 1 for all replicas; this CTA's share of the energies goes into every
+// CTA's row.  The barrier that ends the phase is the caller's.
 template <bool GAUSS, int Z, bool DIL>
 __device__ __forceinline__ void cl_metropolis(const KParams &P, const ClusterLayout &L, const CS &S, uint32_t t,
                                               uint32_t inst, bool tie)
 {
     using ET = typename std::conditional<GAUSS, float, int>::type;
-    const int npass = (P.R + 15) >> 4;
-    const int nwarps = blockDim.x >> 5;
-    for (int it = 0; it < 2 * npass; ++it) {
-        const int color = it >= npass;
-        const int pass = it - color * npass;
-        cl_sweep_pass<GAUSS, Z, DIL>(P, S, t, inst, pass >> 1, color, pass & 1, tie);
-        if (pass == npass - 1) {
-            if (color == 0) cl_sync();            // colour 1 reads colour-0 words of other CTAs
+    const int nth = blockDim.x, nwarps = nth >> 5, tid = threadIdx.x;
+    if constexpr (GAUSS) {
+        const int npass = (P.R + 15) >> 4;
+        for (int it = 0; it < 2 * npass; ++it) {
+            const int color = it >= npass;
+            const int pass = it - color * npass;
+            cl_gauss_pass<Z, DIL>(P, S, t, inst, pass >> 1, color, pass & 1, tie);
+            if (pass == npass - 1) {
+                if (color == 0) cl_sync();            // colour 1 reads the copies of colour 0
+                else __syncthreads();
+            }
+        }
+    } else {
+        const int n8 = (P.R + 7) >> 3;                // groups of 8 replicas
+        const int conc = min(nth / S.hs, n8);         // hs is a multiple of 32
+        const bool split = conc >= 2;
+        const int group = split ? tid / S.hs : 0;
+        const int per = split ? (n8 + conc - 1) / conc : n8;
+        const int lo = group * per, hi = min(lo + per, n8);
+        const int j0 = tid - (split ? group * S.hs : 0), jstride = split ? S.hs : nth;
+        if (split)
+            for (int i = tid; i < nwarps * P.R; i += nth) ((int *)S.Epart)[i] = 0;   // before the barrier below
+        for (int color = 0; color < 2; ++color) {
+            for (int g = lo >> 2; lo < hi && 4 * g < hi; ++g)
+                cl_pmj_pass<Z, DIL>(P, S, t, inst, g, color, max(lo - 4 * g, 0), min(hi - 4 * g, 4), j0, jstride, split,
+                                    tie);
+            if (split) {                              // the words are complete: store the copies
+                __syncthreads();
+                for (int i = tid; i < P.G * S.hs; i += nth) {
+                    const int g = i >= S.hs, li = color * S.hs + i - g * S.hs;
+                    const uint32_t w = S.s[g * S.ns + li], goff = (uint32_t)(g * S.ns * 4) - S.dCs;
+                    for_copies(S, li, [&](uint32_t a) { cl_st(a + goff, w); });
+                }
+            }
+            if (color == 0) cl_sync();
             else __syncthreads();
         }
     }
-    for (int r = threadIdx.x; r < P.R; r += blockDim.x) {
+    for (int r = tid; r < P.R; r += nth) {
         ET e = ET(0);
         for (int w = 0; w < nwarps; ++w) e += ((const ET *)S.Epart)[w * P.R + r];
-        ((ET *)S.Esw)[r] = e;
+        cl_share<ET>(S, L.Esw, P.R, r, e);
     }
-    cl_sync();
-    for (int r = threadIdx.x; r < P.R; r += blockDim.x) ((ET *)S.E)[r] = cl_sum<ET>(S, L.Esw + 4 * r);
-    __syncthreads();
 }
 
 // ---------------------------------------------------------------------------
@@ -446,10 +521,11 @@ __device__ __forceinline__ uint32_t uf_root(const Uf &U, uint32_t x)
 // by one).  `it` is bounded (never reached: each union ends within N climbs
 // and N failed swaps).
 template <int Z, bool REMOTE>
-__device__ __forceinline__ void uf_unions(const Uf &U, const CS &S, uint32_t gm0, uint32_t gm1, int n0, uint32_t mys,
-                                          uint32_t dlab, uint32_t qstride)
+__device__ __forceinline__ void uf_unions(const Uf &U, const CS &S, uint32_t gm0, uint32_t gm1, int n0,
+                                          uint32_t qstride)
 {
-    const int nls = S.nls, hs = S.hs, nth = blockDim.x;
+    const int nls = S.nls, ns = S.ns, hs = S.hs, nth = blockDim.x;
+    const uint32_t cw0 = (uint32_t)__cvta_generic_to_shared(S.C) - S.win;
     int j = (int)threadIdx.x - nth, li = 0, d = Z;
     uint32_t x0 = 0u, x1 = 0u, y0 = 0u, y1 = 0u, ea = 0u, eb = 0u, a = 0u, b = 0u;
     bool more = true, busy = false;
@@ -469,26 +545,25 @@ __device__ __forceinline__ void uf_unions(const Uf &U, const CS &S, uint32_t gm0
                     x0 = (w0 ^ (w0 >> 1)) & gm0;
                     x1 = 0u;
                     if (gm1) {
-                        const uint32_t w1 = S.s[nls + li];
+                        const uint32_t w1 = S.s[ns + li];
                         x1 = (w1 ^ (w1 >> 1)) & gm1;
                     }
                     d = (x0 | x1) ? 0 : Z;
                     ea = U.lab + 4u * (uint32_t)li;
                     continue;
                 }
-                const uint32_t e = S.nb[li * Z + d] - S.dCs;   // the neighbour's spin word 0
+                const int q = (int)((S.nb[li * Z + d] - cw0) >> 2);   // own site or halo entry
                 ++d;
-                const uint32_t o = e - mys;
-                if ((o >= qstride) != REMOTE) continue;
+                if ((q >= nls) != REMOTE) continue;
                 if (x0) {
-                    const uint32_t v = REMOTE ? cl_ld(e) : S.s[o >> 2];
+                    const uint32_t v = S.s[q];
                     y0 = x0 & (v ^ (v >> 1));
                 }
                 if (x1) {
-                    const uint32_t v = REMOTE ? cl_ld(e + qstride) : S.s[nls + (o >> 2)];
+                    const uint32_t v = S.s[ns + q];
                     y1 = x1 & (v ^ (v >> 1));
                 }
-                eb = e + dlab;
+                eb = REMOTE ? S.hlab[q - nls] : U.lab + 4u * (uint32_t)q;
             }
             if (y0 | y1) {
                 uint32_t q;
@@ -555,7 +630,7 @@ __device__ __forceinline__ void uf_mark(const Uf &U, const CS &S, uint32_t gm0, 
                 const uint32_t w0 = S.s[li];
                 x0 = (w0 ^ (w0 >> 1)) & gm0;
                 if (gm1) {
-                    const uint32_t w1 = S.s[nls + li];
+                    const uint32_t w1 = S.s[S.ns + li];
                     x1 = (w1 ^ (w1 >> 1)) & gm1;
                 }
             }
@@ -606,9 +681,7 @@ __device__ __forceinline__ void cl_grow_uf(const KParams &P, const ClusterLayout
     U.lab = cl_map(S.base + L.lab, S.rank);
     U.loc = S.base + (uint32_t)L.lab;
     U.limit = P.N + 1;
-    const uint32_t mys = cl_map(S.base + L.s, S.rank);      // this CTA's spin words in the cluster window
-    const uint32_t dlab = (uint32_t)(L.lab - L.s);          // a site's spin word 0 -> its first label word
-    const uint32_t qstride = 4u * (uint32_t)nls;            // label arrays of consecutive group pairs; word 0 -> 1
+    const uint32_t qstride = 4u * (uint32_t)nls;            // label arrays of consecutive group pairs
     uint32_t rest0 = act0, rest1 = act1;
     int groups = 0;
     while (rest0 | rest1) {
@@ -627,9 +700,9 @@ __device__ __forceinline__ void cl_grow_uf(const KParams &P, const ClusterLayout
         ++groups;
         for (int i = tid; i < ng * nls; i += nth) S.lab[i] = U.lab + 4u * (uint32_t)i;
         __syncthreads();
-        uf_unions<Z, false>(U, S, gm0, gm1, n0, mys, dlab, qstride);
+        uf_unions<Z, false>(U, S, gm0, gm1, n0, qstride);
         cl_sync();                                   // every CTA's own unions are done
-        uf_unions<Z, true>(U, S, gm0, gm1, n0, mys, dlab, qstride);
+        uf_unions<Z, true>(U, S, gm0, gm1, n0, qstride);
         cl_sync();
         if (tid < ng) {                              // the root of the tid-th group pair's seed
             uint32_t m0 = gm0, m1 = gm1;
@@ -645,110 +718,118 @@ __device__ __forceinline__ void cl_grow_uf(const KParams &P, const ClusterLayout
         if (rest0 | rest1) cl_sync();                // walks through these labels end before the reset
     }
     __syncthreads();
+    for (int li = tid; li < nls; li += nth) {        // the marked words into the halos
+        const uint32_t c = S.C[li];
+        if (c) for_copies(S, li, [&](uint32_t a) { cl_st(a, c); });
+    }
+    cl_sync();
     if (S.rank == 0 && tid == 0) {
         S.icmst[0] += (unsigned)(__popc(act0) + __popc(act1));
         S.icmst[1] += 4u * (unsigned)groups;         // passes over the own sites
     }
 }
 
-// Steps 2a and 2b (see cluster_moves in pt_icm.cu).
+// Steps 2a and 2b (see cluster_moves in pt_icm.cu).  S.seed holds the seed
+// draws on entry.
 template <bool GAUSS, int Z>
-__device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const CS &S, uint32_t t, uint32_t inst,
-                                 int slot, bool trace)
+__device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const CS &S, uint32_t t, int slot,
+                                 bool trace)
 {
     using ET = typename std::conditional<GAUSS, float, int>::type;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int tid = threadIdx.x, nth = blockDim.x;
-    const int N = P.N, nicm = P.n_icm, G = P.G, nls = S.nls, hs = S.hs, NWl = L.NWl;
+    const int N = P.N, nicm = P.n_icm, G = P.G, nls = S.nls, ns = S.ns, hs = S.hs, NWl = L.NWl;
     ET *E = (ET *)S.E;
     ET *esum = (ET *)S.esum;
 
-    // (a) overlap masks of the own sites, per-colour-block counts
+    // (a) overlap masks of the own sites and their counts per colour block
+    // (cnt_n: colour 0, cnt_d: colour 1); clear the cluster words
+    const int kp = pair_of_bit(lane);
+    int cnt[2] = {0, 0};
     for (int m = warp; m < NWl; m += nwarps) {
         const int li = 32 * m + lane;
-        const uint32_t w0 = S.s[li];
-        uint32_t x = (w0 ^ (w0 >> 1)) & 0x55555555u;   // bit 2j: pair j; bit 2j + 1: pair 16 + j
-        if (G > 1) {
-            const uint32_t w1 = S.s[nls + li];
-            x |= ((w1 ^ (w1 >> 1)) & 0x55555555u) << 1;
-        }
-        const uint32_t col = warp_transpose32(x, lane);
-        const int k = (lane >> 1) + 16 * (lane & 1);
-        if (k < nicm) S.mask[k * NWl + m] = col;
+        const uint32_t col = warp_transpose32(overlap_word(S.s[li], G > 1 ? S.s[ns + li] : 0u), lane);
+        cnt[32 * m >= hs] += __popc(col);
+        if (kp < nicm) S.mask[kp * NWl + m] = col;
     }
-    for (int i = tid; i < nls; i += nth) S.C[i] = 0u;
+    if (kp < nicm) {
+        if (cnt[0]) atomicAdd(&S.cnt_n[kp], cnt[0]);
+        if (cnt[1]) atomicAdd(&S.cnt_d[kp], cnt[1]);
+    }
+    for (int i = tid; i < ns; i += nth) S.C[i] = 0u;
     if (tid < 2) S.flipw[tid] = 0u;
     if (tid < 32) S.csz[tid] = 0;
     __syncthreads();
-    for (int k = tid; k < nicm; k += nth)
-        for (int c = 0; c < 2; ++c) {
-            int n = 0;
-            for (int m = c * (hs / 32); m < (c + 1) * (hs / 32); ++m) n += __popc(S.mask[k * NWl + m]);
-            S.cntloc[c * 32 + k] = n;
-        }
+    for (int i = tid; i < 2 * nicm; i += nth) {
+        const int c = i >= nicm, k = i - c * nicm;
+        int *v = (c ? S.cnt_d : S.cnt_n) + k;
+        cl_share<int>(S, L.cntloc, 64, 32 * c + k, *v);
+        *v = 0;                                       // as the observables expect it
+    }
     cl_sync();
 
     // (b) per pair, in every CTA alike: n, step 2a, the seed's owner by rank;
     // the owner plants the seed
     for (int k = tid; k < nicm; k += nth) {
-        int n = 0;
-        for (int c = 0; c < 2; ++c)
-            for (uint32_t r = 0; r < S.K; ++r) n += (int)cl_ld(cl_map(S.base + L.cntloc + 4 * (c * 32 + k), r));
+        int n = row_sum<int>(S, S.cntloc, 64, k) + row_sum<int>(S, S.cntloc, 64, 32 + k);
         const int n_pre = n;
         const bool flipped = P.enable_2a && 2 * n > N;
         if (flipped) {
             n = N - n;
             atomicOr(&S.flipw[(2 * k + 1) >> 5], 1u << ((2 * k + 1) & 31));
         }
-        int seed_pos = -1;
+        bool moves = false;
         if (n > 0) {
-            uint32_t x[4];
-            philox10k((uint32_t)k, t, 0u, (1u << 24) | inst, P.key, x);
-            uint32_t rank = (uint32_t)(((uint64_t)x[0] * (uint32_t)n) >> 32);
-            for (int c = 0; c < 2 && seed_pos < 0; ++c)
-                for (uint32_t r = 0; r < S.K; ++r) {
-                    int cnt = (int)cl_ld(cl_map(S.base + L.cntloc + 4 * (c * 32 + k), r));
-                    if (flipped) cnt = hs - cnt;
-                    if (rank < (uint32_t)cnt) {
-                        if (r == S.rank) {             // this CTA owns the seed: find the local site
-                            for (int m = c * (hs / 32); m < (c + 1) * (hs / 32); ++m) {
-                                uint32_t w = S.mask[k * NWl + m];
-                                if (flipped) w = ~w;
-                                const uint32_t pc = (uint32_t)__popc(w);
-                                if (rank < pc) {
-                                    const int li = 32 * m + nth_set_bit(w, rank);
-                                    atomicOr(S.C + ICM_IDX(li, nls, 21), 1u << (2 * (k & 15) + (k >> 4)));
-                                    if (L.ufg) {       // the seed's site address, for the union-find roots
-                                        const uint32_t sa = cl_map(S.base, S.rank) + 4u * (uint32_t)li;
-                                        for (uint32_t r2 = 0; r2 < S.K; ++r2) cl_st(cl_map(S.base + L.sadr + 4 * k, r2), sa);
-                                    }
-                                    if (trace) P.tr_seed[(size_t)slot * P.nT + k] = (int)__ldg(P.pos2site + pos_of(P, S, li));
-                                    break;
+            uint32_t rank = (uint32_t)(((uint64_t)(uint32_t)S.seed[k] * (uint32_t)n) >> 32);
+            const uint32_t inv = flipped ? kFull : 0u;
+            for (int cr = 0; cr < 2 * (int)S.K; ++cr) {
+                const int c = cr >= (int)S.K, r = cr - c * (int)S.K;
+                int cn = S.cntloc[64 * r + 32 * c + k];
+                if (flipped) cn = hs - cn;
+                if (rank < (uint32_t)cn) {
+                    moves = true;
+                    if (r == (int)S.rank) {           // this CTA owns the seed: find the local site
+                        for (int m = c * (hs / 32); m < (c + 1) * (hs / 32); ++m) {
+                            const uint32_t w = S.mask[k * NWl + m] ^ inv;
+                            const uint32_t pc = (uint32_t)__popc(w);
+                            if (rank < pc) {
+                                const int li = 32 * m + nth_set_bit(w, rank);
+                                const uint32_t bit = 1u << (2 * (k & 15) + (k >> 4));
+                                atomicOr(S.C + ICM_IDX(li, nls, 21), bit);
+                                if (L.ufg) {           // the seed's site address, for the union-find roots
+                                    const uint32_t sa = cl_map(S.base, S.rank) + 4u * (uint32_t)li;
+                                    for (uint32_t r2 = 0; r2 < S.K; ++r2) cl_st(cl_map(S.base + L.sadr + 4 * k, r2), sa);
                                 }
-                                rank -= pc;
+                                if (trace) P.tr_seed[(size_t)slot * P.nT + k] = (int)__ldg(P.pos2site + pos_of(P, S, li));
+                                break;
                             }
+                            rank -= pc;
                         }
-                        seed_pos = c * P.half + (int)r * hs;   // block of the seed (the owner records the site)
-                        break;
                     }
-                    rank -= (uint32_t)cnt;
+                    break;
                 }
+                rank -= (uint32_t)cn;
+            }
         }
-        S.seed[k] = seed_pos >= 0;
+        S.seed[k] = moves;
         esum[k] = E[2 * k] + E[2 * k + 1];
         if (trace && S.rank == 0) {
             const size_t o = (size_t)slot * P.nT + k;
             P.tr_n_pre[o] = n_pre;
-            P.tr_flip2a[o] = flipped;
-            if (seed_pos < 0) P.tr_seed[o] = -1;
+            P.tr_flip2a[o] = flipped ? 1 : 0;
+            if (!moves) P.tr_seed[o] = -1;
             P.tr_csize[o] = 0;
             P.tr_eb[o] = (float)(E[2 * k] + E[2 * k + 1]);
             P.tr_ea[o] = (float)(E[2 * k] + E[2 * k + 1]);
         }
     }
-    cl_sync();
+    // The growth below stores the seeds' copies first and runs at least two
+    // rounds, so that they are seen before the rounds can end; the union-find
+    // needs every CTA's seed addresses.
+    if (L.ufg) cl_sync();
+    else __syncthreads();
 
-    // (c) step 2a on the own sites, then the clusters of all pairs at once
+    // (c) step 2a on the own and halo sites, then the clusters of all pairs at once
     uint32_t act0 = 0u, act1 = 0u;
     for (int k = 0; k < nicm; ++k)
         if (S.seed[k]) {
@@ -756,117 +837,105 @@ __device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const
             else act1 |= 1u << (2 * (k - 16));
         }
     const uint32_t f0 = S.flipw[0], f1 = S.flipw[1];
-    for (int li = tid; li < nls; li += nth) {
-        S.s[li] ^= f0;
-        if (G > 1) S.s[nls + li] ^= f1;
-    }
-    if (S.gord) __syncthreads();                     // below a thread reads sites that others reversed
-    if (!(act0 | act1)) {
-        __syncthreads();
-        return;                                      // the same decision in every CTA
-    }
+    if (f0 | f1)
+        for (int li = tid; li < ns; li += nth) {
+            S.s[li] ^= f0;
+            if (G > 1) S.s[ns + li] ^= f1;
+        }
+    __syncthreads();                                 // below a thread reads sites that others reversed
+    if (!(act0 | act1)) return;                      // the same decision in every CTA
     // One cluster word per site holds every pair: bit 2j = pair j, bit 2j + 1
     // = pair 16 + j, so that the domain word is q of the first spin word | q
     // of the second << 1 and a neighbour is one load.
     // Growth in cluster rounds of kScansPerRound in-place scans of the own
-    // sites (6: 2D L=128 and 3D L=16 on 8 x 512 +3.3% and +1.3% against 4,
-    // where a round that grows from 2 to 8 scans lost 2.7% on 3D L=16).
-    // Within a round the CTAs scan without barriers, reading each other's
-    // words as they are.  A warp that grew a site writes the round's
+    // sites, reading the halo words as they are; a border site that grew is
+    // stored into its copies.  A warp that grew a site writes the round's
     // stamp into the stamp word of every CTA of the cluster; after the
     // round's barrier each CTA reads its own word, so all CTAs decide alike.
-    // The growth ends after a round in which nothing grew: every read of that
-    // round saw the state that the previous barrier published, and no site
-    // could grow from it, so it is the fixed point, each seed's component of
-    // q = -1.  Stamps are (t << 16) + round + 1 (at most N < 2^16 rounds), so
-    // words need no reset; a stale equal value could only add one empty round.
+    // The growth ends after a round, the second at the earliest, in which
+    // nothing grew: every read of that round saw the state that the previous
+    // barrier published, and no site could grow from it, so it is the fixed
+    // point, each seed's component of q = -1.  Stamps are (t << 16) + round +
+    // 1 (at most N < 2^16 rounds), so words need no reset; a stale equal value
+    // could only add one empty round.
     constexpr int kScansPerRound = 6;
     const uint32_t actc = act0 | (act1 << 1);
-    // with at most four own sites per thread, each thread keeps their domain
-    // and cluster words in registers across the scans and skips the sites
-    // already absorbed (2D L=128 on 8 x 512: +8%, with 50-100 bytes of
-    // register spills under the 64 registers of the launch bounds).  On 2D
-    // lattices with four sites per thread the host gives each thread a 2 x 2
-    // block of sites, taken around the block (S.gord): a scan then carries
-    // the growth across the block and into the next lane's block (a model of
-    // the in-place scans on this workload's domains: 118 scans per sweep
-    // instead of 155).
+    // with at most four own sites per thread, each thread keeps their
+    // neighbour addresses, domain and cluster words in registers across the
+    // scans.  On 2D lattices with four sites per thread the host gives each
+    // thread a 2 x 2 block of sites, taken around the block (S.gord): a scan
+    // then carries the growth across the block and into the next lane's block
+    // (a model of the in-place scans on this workload's domains: 118 scans per
+    // sweep instead of 155).  With more, the domain words take the place of
+    // the overlap masks, which are dead once the seeds are planted.
     const bool in_regs = nls <= 4 * nth;
-    auto own = [&](int j) { return S.gord ? (int)S.gord[4 * tid + j] : tid + j * nth; };
-    uint32_t dm[4], cw[4];
-    uint32_t todo = 0u;                              // bit j: own site j not yet absorbed
+    uint32_t *dom = S.lab;
+    uint32_t dm[4], cw[4], own2[2], e[4][Z / 2];
     if (!L.ufg && in_regs) {
+        own2[0] = own2[1] = 0u;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int li = own(j);
             dm[j] = cw[j] = 0u;
+#pragma unroll
+            for (int i = 0; i < Z / 2; ++i) e[j][i] = 0u;
             if (tid + j * nth < nls) {
-                const uint32_t w0 = S.s[li], w1 = G > 1 ? S.s[nls + li] : 0u;
-                dm[j] = (((w0 ^ (w0 >> 1)) & 0x55555555u) | (((w1 ^ (w1 >> 1)) & 0x55555555u) << 1)) & actc;
+                const int li = S.gord ? (int)S.gord[4 * tid + j] : tid + j * nth;
+                own2[j >> 1] |= (uint32_t)li << (16 * (j & 1));
+                dm[j] = overlap_word(S.s[li], G > 1 ? S.s[ns + li] : 0u) & actc;
                 cw[j] = S.C[li];
-                if (dm[j] != cw[j]) todo |= 1u << j;
+                nb_row<Z>(S.nb, li, e[j]);
+                if (cw[j]) for_copies(S, li, [&](uint32_t a) { cl_st(a, cw[j]); });
             }
+        }
+    } else if (!L.ufg) {
+        for (int li = tid; li < nls; li += nth) {
+            dom[li] = overlap_word(S.s[li], G > 1 ? S.s[ns + li] : 0u) & actc;
+            const uint32_t c = S.C[li];
+            if (c) for_copies(S, li, [&](uint32_t a) { cl_st(a, c); });
         }
     }
     if (L.ufg) cl_grow_uf<Z>(P, L, S, act0, act1);
     else for (int round = 0;; ++round) {
         int grew = 0;
-        if (in_regs) {
-            for (int scan = 0; scan < kScansPerRound; ++scan) {
-                // the thread's four block sites in one 8-byte load
-                uint2 o = make_uint2(0u, 0u);
-                if (S.gord) o = *reinterpret_cast<const uint2 *>(S.gord + 4 * tid);
+        for (int scan = 0; scan < kScansPerRound; ++scan) {
+            if (in_regs) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    // absorbed sites are skipped, except on 2D lattices, where the
-                    // test costs more than it saves (2D L=128: +3.9% without it;
-                    // 3D L=16: -1.7%)
-                    if constexpr (Z != 4) {
-                        if (!((todo >> j) & 1u)) continue;
-                    } else {
-                        if (tid + j * nth >= nls) continue;
-                    }
-                    const int li = S.gord ? (int)(((j < 2 ? o.x : o.y) >> (16 * (j & 1))) & 0xFFFFu) : tid + j * nth;
+                    if (dm[j] == cw[j]) continue;    // nothing left to absorb
                     uint32_t nb = 0u;
-                    // the site's neighbour row in one 16-byte (Z = 4) or 8-byte loads
-                    // (2D L=128 on 8 x 512: +22% against four 4-byte loads)
-                    uint32_t e[Z];
-                    nb_row<Z>(S.nb, li, e);
 #pragma unroll
-                    for (int d = 0; d < Z; ++d) nb |= cl_ld(e[d]);
+                    for (int d = 0; d < Z; ++d) nb |= sh_ld(nb_addr(e[j][d >> 1], d, S.win));
                     const uint32_t n = cw[j] | (dm[j] & nb);
                     if (n != cw[j]) {
+                        const int li = (int)((own2[j >> 1] >> (16 * (j & 1))) & 0xffffu);
                         S.C[li] = n;
                         cw[j] = n;
                         grew = 1;
-                        if constexpr (Z != 4)
-                            if (n == dm[j]) todo &= ~(1u << j);
+                        for_copies(S, li, [&](uint32_t a) { cl_st(a, n); });
                     }
                 }
-            }
-        } else {
-            for (int scan = 0; scan < kScansPerRound; ++scan)
+            } else {
                 for (int li = tid; li < nls; li += nth) {
-                    const uint32_t w0 = S.s[li], w1 = G > 1 ? S.s[nls + li] : 0u;
-                    const uint32_t dmw = (((w0 ^ (w0 >> 1)) & 0x55555555u) | (((w1 ^ (w1 >> 1)) & 0x55555555u) << 1)) & actc;
-                    const uint32_t c = S.C[li];
-                    if (dmw == c) continue;
-                    uint32_t e[Z], nb = 0u;
-                    nb_row<Z>(S.nb, li, e);
+                    const uint32_t d0 = dom[li], c = S.C[li];
+                    if (d0 == c) continue;
+                    uint32_t w[Z], nb = 0u;
+                    nb_words<Z>(S, li, 0u, w);
 #pragma unroll
-                    for (int d = 0; d < Z; ++d) nb |= cl_ld(e[d]);
-                    const uint32_t n = c | (dmw & nb);
+                    for (int d = 0; d < Z; ++d) nb |= w[d];
+                    const uint32_t n = c | (d0 & nb);
                     if (n != c) {
                         S.C[li] = n;
                         grew = 1;
+                        for_copies(S, li, [&](uint32_t a) { cl_st(a, n); });
                     }
                 }
+            }
         }
         const uint32_t stamp = (t << 16) + (uint32_t)round + 1u;
         if (__any_sync(kFull, grew) && lane == 0)
             for (uint32_t r = 0; r < S.K; ++r) cl_st(cl_map(S.base + L.flags + 4 * (round & 1), r), stamp);
         cl_sync();
-        if ((uint32_t)S.flags[round & 1] != stamp) {
+        if (round > 0 && (uint32_t)S.flags[round & 1] != stamp) {
             if (S.rank == 0 && tid == 0) {
                 S.icmst[0] += (unsigned)(__popc(act0) + __popc(act1));
                 S.icmst[1] += (unsigned)(round + 1) * kScansPerRound;   // scans of the own sites
@@ -875,13 +944,13 @@ __device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const
         }
     }
 
-    // (d) flip the own sites; copy-a energies of the moved pairs
-    for (int li = tid; li < nls; li += nth) {
+    // (d) flip the own and halo sites; copy-a energies of the moved pairs
+    for (int li = tid; li < ns; li += nth) {
         const uint32_t cw = S.C[li];
         const uint32_t c0 = cw & 0x55555555u, c1 = (cw >> 1) & 0x55555555u;
         if (c0) S.s[li] ^= c0 | (c0 << 1);
-        if (c1) S.s[nls + li] ^= c1 | (c1 << 1);
-        if (trace) {
+        if (c1) S.s[ns + li] ^= c1 | (c1 << 1);
+        if (trace && li < nls) {
             for (int w = 0; w < 2; ++w)
                 for (uint32_t b = w ? c1 : c0; b; b &= b - 1u) atomicAdd(&S.csz[16 * w + ((__ffs(b) - 1) >> 1)], 1);
             if (P.tr_cmask) {
@@ -891,36 +960,34 @@ __device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const
             }
         }
     }
-    cl_sync();                                       // flipped words of other CTAs are read below
+    __syncthreads();
     // copy-a energies of the moved pairs (cb = 0); a traced sweep then also
     // recomputes the copy-b energies (cb = 1) and records E_a + E_b of the two
     // recomputed energies, so that the trace tests the conservation of E_a + E_b
     ET *part = (ET *)S.Epart;
     for (int cb = 0; cb < (trace ? 2 : 1); ++cb) {
         if (cb) cl_sync();                           // every CTA has read the copy-a shares
-        for (int g = 0; g < G; ++g) {
-            const uint32_t act = g ? act1 : act0;
-            if (!act) continue;
-            const uint32_t goff = (uint32_t)(g * nls * 4) - S.dCs;   // neighbour entry -> its spin word g
-            const uint32_t *sg = S.s + g * nls;
-            ET acc[16];
+        if constexpr (GAUSS) {
+            for (int g = 0; g < G; ++g) {
+                const uint32_t act = g ? act1 : act0;
+                if (!act) continue;
+                const uint32_t goff = (uint32_t)(g * ns * 4) - S.dCs;   // cluster word -> spin word g
+                const uint32_t *sg = S.s + g * ns;
+                float acc[16];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) acc[j] = ET(0);
-            for (int j = tid; j < hs; j += nth) {
-                const int li = hs + j;               // colour-1 sites: every bond once
-                const uint32_t sw = sg[li] >> cb;
-                uint32_t nw[Z];
-                nb_row<Z>(S.nb, li, nw);
-#pragma unroll
-                for (int d = 0; d < Z; ++d) nw[d] = cl_ld(nw[d] + goff) >> cb;
-                if constexpr (GAUSS) {
-                    float J2[Z];
+                for (int j = 0; j < 16; ++j) acc[j] = 0.f;
+                for (int j = tid; j < hs; j += nth) {
+                    const int li = hs + j;           // colour-1 sites: every bond once
+                    const uint32_t sw = sg[li] >> cb;
+                    uint32_t nw[Z];
+                    nb_words<Z>(S, li, goff, nw);
+                    float J[Z];
                     float Jsum = 0.f;
 #pragma unroll
                     for (int d = 0; d < Z; ++d) {
-                        const float J = S.Jd[li * Z + d];
-                        Jsum += J;
-                        J2[d] = 2.f * J;
+                        nw[d] >>= cb;
+                        J[d] = S.Jd[li * Z + d];
+                        Jsum += J[d];
                     }
 #pragma unroll
                     for (int jj = 0; jj < 16; ++jj) {
@@ -929,42 +996,49 @@ __device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const
                         float h = Jsum;
 #pragma unroll
                         for (int d = 0; d < Z; ++d)
-                            if ((nw[d] >> b) & 1u) h -= J2[d];
+                            if ((nw[d] >> b) & 1u) h = fmaf(J[d], -2.f, h);
                         acc[jj] += ((sw >> b) & 1u) ? h : -h;
                     }
-                } else {
-                    uint32_t c0 = 0, c1 = 0, c2 = 0, c3 = 0;
-                    const uint32_t jb = S.Jb[li];
-                    uint32_t u[Z];
-#pragma unroll
-                    for (int d = 0; d < Z; ++d) u[d] = sw ^ nw[d] ^ (0u - ((jb >> d) & 1u));
-                    csa_count<Z>(u, c0, c1, c2, c3);
-#pragma unroll
-                    for (int jj = 0; jj < 16; ++jj) {
-                        const int b = 2 * jj;
-                        acc[jj] += (int)(((c0 >> b) & 1u) | (((c1 >> b) & 1u) << 1) | (((c2 >> b) & 1u) << 2) |
-                                         (((c3 >> b) & 1u) << 3));
-                    }
                 }
+                const float v = transpose_reduce16(acc, lane);
+                if (!(lane & 1)) part[warp * 32 + 16 * g + (lane >> 1)] = v;
             }
-            const ET v = transpose_reduce16(acc, lane);
-            if (!(lane & 1)) part[warp * 32 + 16 * g + (lane >> 1)] = v;
+        } else {
+            uint32_t pl[kPlanes];
+#pragma unroll
+            for (int i = 0; i < kPlanes; ++i) pl[i] = 0u;
+            const uint32_t o1 = (uint32_t)(ns * 4);
+            for (int j = tid; j < hs; j += nth) {
+                const int li = hs + j;               // colour-1 sites: every bond once
+                const uint32_t y = copy_word(S.s[li], G > 1 ? S.s[ns + li] : 0u, cb);
+                const uint32_t jb = S.Jb[li];
+                uint32_t r[Z / 2], u[Z], c0, c1, c2, c3;
+                nb_row<Z>(S.nb, li, r);
+#pragma unroll
+                for (int d = 0; d < Z; ++d) {
+                    const uint32_t a = nb_addr(r[d >> 1], d, S.win) - S.dCs;
+                    u[d] = y ^ copy_word(sh_ld(a), G > 1 ? sh_ld(a + o1) : 0u, cb) ^ (0u - ((jb >> d) & 1u));
+                }
+                csa_count<Z>(u, c0, c1, c2, c3);
+                vadd4(pl, c0, c1, c2, c3);
+            }
+            part[warp * 32 + kp] = warp_vcount(pl, P.cnt_planes, lane);
         }
         __syncthreads();
         for (int k = tid; k < nicm; k += nth) {
-            ET e = ET(0);
+            ET es = ET(0);
             if (S.seed[k])
-                for (int w = 0; w < nwarps; ++w) e += part[w * 32 + k];
-            ((ET *)S.Epair)[k] = e;
+                for (int w = 0; w < nwarps; ++w) es += part[w * 32 + k];
+            cl_share<ET>(S, L.Epair, 32, k, es);
         }
         cl_sync();
         for (int k = tid; k < nicm; k += nth) {
             if (!S.seed[k]) continue;
-            ET e = cl_sum<ET>(S, L.Epair + 4 * k);
-            if constexpr (!GAUSS) e = 2 * e - (P.diluted ? P.nb_inst[slot] : P.Nb);   // E = 2 U - N_b (bonds present)
+            ET es = row_sum<ET>(S, S.Epair, 32, k);
+            if constexpr (!GAUSS) es = 2 * es - (P.diluted ? P.nb_inst[slot] : P.Nb);   // E = 2 U - N_b (bonds present)
             if (cb == 0) {
-                E[2 * k] = e;
-                E[2 * k + 1] = esum[k] - e;
+                E[2 * k] = es;
+                E[2 * k + 1] = esum[k] - es;
             }
             if (trace && S.rank == 0) {
                 const size_t o = (size_t)slot * P.nT + k;
@@ -973,7 +1047,7 @@ __device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const
                     for (uint32_t r = 0; r < S.K; ++r) cs += (int)cl_ld(cl_map(S.base + L.csz + 4 * k, r));
                     P.tr_csize[o] = cs;
                 } else {
-                    P.tr_ea[o] = (float)(E[2 * k] + e);
+                    P.tr_ea[o] = (float)(E[2 * k] + es);
                 }
             }
         }
@@ -982,15 +1056,12 @@ __device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const
 }
 
 // Step 3 (see pt_pass in pt_icm.cu): the same energies and draws in every
-// CTA give the same decisions; each CTA permutes its own words.
+// CTA give the same decisions; each CTA permutes its own and halo words.
 template <bool GAUSS>
-__device__ void cl_pt_pass(const KParams &P, const CS &S, uint32_t t, uint32_t inst, int slot, bool trace)
+__device__ void cl_pt_pass(const KParams &P, const CS &S, int slot, bool trace)
 {
     using ET = typename std::conditional<GAUSS, float, int>::type;
-    const int nT = P.nT, np = nT - 1, nls = S.nls;
-    for (int i = threadIdx.x; i < 2 * np; i += blockDim.x)
-        pt_draw<GAUSS>(i, np, t, inst, P.key, S.swap_x, P.thr_swap, P.swap_off, P.swap_len, P.dbeta_l2e);
-    __syncthreads();
+    const int np = P.nT - 1, ns = S.ns;
     // every CTA decides alike (the same energies and draws); rank 0 traces
     if (threadIdx.x < 32)
         pt_warp<GAUSS, ET>((ET *)S.E, P.R, np, S.swap_x, P.dbeta_l2e, S.swap_mask,
@@ -999,75 +1070,77 @@ __device__ void cl_pt_pass(const KParams &P, const CS &S, uint32_t t, uint32_t i
     SwapMasks m;
     if (swap_masks(S.swap_mask, m)) {
         const bool two = P.G > 1;
-        for (int li = threadIdx.x; li < nls; li += blockDim.x) {
-            const uint64_t x = (uint64_t)S.s[li] | (two ? (uint64_t)S.s[nls + li] << 32 : 0ull);
+        for (int li = threadIdx.x; li < ns; li += blockDim.x) {
+            const uint64_t x = (uint64_t)S.s[li] | (two ? (uint64_t)S.s[ns + li] << 32 : 0ull);
             const uint64_t y = swap_apply(m, x);
             S.s[li] = (uint32_t)y;
-            if (two) S.s[nls + li] = (uint32_t)(y >> 32);
+            if (two) S.s[ns + li] = (uint32_t)(y >> 32);
         }
     }
-    cl_sync();                                       // the observables read other CTAs' words
+    __syncthreads();
 }
 
-// Observables (see measure in pt_icm.cu): per-CTA counts, summed by rank 0.
-template <bool GAUSS, int Z>
-__device__ void cl_measure(const KParams &P, const ClusterLayout &L, const CS &S, int slot)
+// Observables (see measure in pt_icm.cu): this CTA's counts, stored into rank
+// 0's rows.  The barrier before rank 0 adds them is the one that ends the step.
+template <int Z>
+__device__ __forceinline__ void cl_count(const KParams &P, const ClusterLayout &L, const CS &S, int parity)
+{
+    const int lane = threadIdx.x & 31, nth = blockDim.x;
+    const int nT = P.nT, nls = S.nls, ns = S.ns, hs = S.hs;
+    const bool two = P.G > 1;
+    const uint32_t o1 = (uint32_t)(ns * 4);
+    uint32_t pn[kPlanes], pd[kPlanes];
+#pragma unroll
+    for (int i = 0; i < kPlanes; ++i) pn[i] = pd[i] = 0u;
+    for (int li = threadIdx.x; li < nls; li += nth) {
+        const uint32_t x = overlap_word(S.s[li], two ? S.s[ns + li] : 0u);
+        vadd(pn, x);
+        if (li < hs) continue;
+        uint32_t r[Z / 2], y[Z], c0, c1, c2, c3;   // a padding entry points at the site itself: y = 0
+        nb_row<Z>(S.nb, li, r);
+#pragma unroll
+        for (int d = 0; d < Z; ++d) {
+            const uint32_t a = nb_addr(r[d >> 1], d, S.win) - S.dCs;
+            y[d] = x ^ overlap_word(sh_ld(a), two ? sh_ld(a + o1) : 0u);
+        }
+        csa_count<Z>(y, c0, c1, c2, c3);
+        vadd4(pd, c0, c1, c2, c3);
+    }
+    const int k = pair_of_bit(lane);
+    const int n = warp_vcount(pn, P.cnt_planes, lane), d = warp_vcount(pd, P.cnt_planes, lane);
+    if (k < nT) {
+        atomicAdd(S.cnt_n + k, n);
+        atomicAdd(S.cnt_d + k, d);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2 * nT; i += nth) {
+        const int c = i >= nT, kk = i - c * nT;
+        int *v = (c ? S.cnt_d : S.cnt_n) + kk;
+        cl_st(cl_map(S.base + L.cntobs + 4u * (uint32_t)((parity * (int)S.K + (int)S.rank) * 64 + 32 * c + kk), 0u),
+              (uint32_t)*v);
+        *v = 0;
+    }
+}
+
+// rank 0, after the barrier; the rows alternate between steps, since the next
+// step may count without another barrier
+template <bool GAUSS>
+__device__ __forceinline__ void cl_accumulate(const KParams &P, const CS &S, int slot, int parity)
 {
     using ET = typename std::conditional<GAUSS, float, int>::type;
-    const int lane = threadIdx.x & 31;
-    const int N = P.N, nT = P.nT, nls = S.nls, hs = S.hs;
-    if (threadIdx.x < 32) {
-        S.cnt_n[threadIdx.x] = 0;
-        S.cnt_d[threadIdx.x] = 0;
+    const int N = P.N, nT = P.nT;
+    const int *rows = S.cntobs + parity * (int)S.K * 64;
+    for (int k = threadIdx.x; k < nT; k += blockDim.x) {
+        const long long n = row_sum<int>(S, rows, 64, k), d = row_sum<int>(S, rows, 64, 32 + k);
+        const ET *E = (const ET *)S.E;
+        S.accE[k] += (double)E[2 * k] + (double)E[2 * k + 1];
+        S.acc64[0 * nT + k] += n;
+        S.acc64[1 * nT + k] += (N - 2 * n) * (N - 2 * n);
+        S.acc64[2 * nT + k] += n < N - n ? n : N - n;
+        S.acc64[3 * nT + k] += d;
+        atomicAdd(&P.hist[((size_t)slot * nT + k) * (N + 1) + ICM_IDX(n, N + 1, 22)], 1ull);
     }
-    __syncthreads();
-    for (int g = 0; g < P.G; ++g) {
-        const int npair = min(16, nT - 16 * g);
-        const uint32_t goff = (uint32_t)(g * nls * 4) - S.dCs;   // neighbour entry -> its spin word g
-        const uint32_t *sg = S.s + g * nls;
-        uint32_t pl[kPlanes];   // even bit 2k: q = -1 sites of pair k; odd bit 2k+1: its q_i q_j = -1 bonds
-#pragma unroll
-        for (int i = 0; i < kPlanes; ++i) pl[i] = 0u;
-        for (int li = threadIdx.x; li < nls; li += blockDim.x) {
-            const uint32_t w = sg[li];
-            vadd(pl, (w ^ (w >> 1)) & 0x55555555u);
-        }
-        for (int li = hs + threadIdx.x; li < nls; li += blockDim.x) {
-            const uint32_t w = sg[li];
-            const uint32_t qp = (w ^ (w >> 1)) & 0x55555555u;
-            uint32_t x[Z];                 // a padding entry points at the site itself: x = 0
-            nb_row<Z>(S.nb, li, x);
-#pragma unroll
-            for (int d = 0; d < Z; ++d) {
-                const uint32_t wq = cl_ld(x[d] + goff);
-                x[d] = (qp ^ ((wq ^ (wq >> 1)) & 0x55555555u)) << 1;
-            }
-            uint32_t c0, c1, c2, c3;
-            csa_count<Z>(x, c0, c1, c2, c3);
-            vadd4(pl, c0, c1, c2, c3);
-        }
-        const int v = warp_vsum(pl, lane);   // lane 2k: n of pair k, lane 2k+1: d of pair k
-        if (lane < 2 * npair) atomicAdd(((lane & 1) ? S.cnt_d : S.cnt_n) + 16 * g + (lane >> 1), v);
-    }
-    cl_sync();
-    if (S.rank == 0) {
-        for (int k = threadIdx.x; k < nT; k += blockDim.x) {
-            long long n = 0, d = 0;
-            for (uint32_t r = 0; r < S.K; ++r) {
-                n += (int)cl_ld(cl_map(S.base + L.cnt_n + 4 * k, r));
-                d += (int)cl_ld(cl_map(S.base + L.cnt_d + 4 * k, r));
-            }
-            const ET *E = (const ET *)S.E;
-            S.accE[k] += (double)E[2 * k] + (double)E[2 * k + 1];
-            S.acc64[0 * nT + k] += n;
-            S.acc64[1 * nT + k] += (N - 2 * n) * (N - 2 * n);
-            S.acc64[2 * nT + k] += n < N - n ? n : N - n;
-            S.acc64[3 * nT + k] += d;
-            atomicAdd(&P.hist[((size_t)slot * nT + k) * (N + 1) + ICM_IDX(n, N + 1, 22)], 1ull);
-        }
-        if (threadIdx.x == 0) S.nmeas[0] += 1;
-    }
-    __syncthreads();
+    if (threadIdx.x == 0) S.nmeas[0] += 1;
 }
 
 // ---------------------------------------------------------------------------
@@ -1079,39 +1152,57 @@ __global__ void __launch_bounds__(kMaxThreadsWide, 1) cluster_kernel(const KPara
     extern __shared__ __align__(16) unsigned char smem[];
     const CS S = make_cs(smem, L);
     const int tid = threadIdx.x, nth = blockDim.x;
-    const int N = P.N, R = P.R, nT = P.nT, G = P.G, nls = S.nls, hs = S.hs, half = P.half;
+    const int N = P.N, R = P.R, nT = P.nT, G = P.G, nls = S.nls, ns = S.ns;
 
     if (tid < 2) S.flags[tid] = 0;   // growth round stamps (the same in every CTA at all times)
-    // neighbour table: cluster-window address of each neighbour's cluster word
-    // (of the batch's lattice here; per instance for diluted batches, below)
+    if (tid < 32) {
+        S.cnt_n[tid] = 0;
+        S.cnt_d[tid] = 0;
+    }
+    // neighbour table: the offset of each neighbour's cluster word in the shared
+    // window, own or halo, by the batch's lattice; an instance's absent bonds (diluted
+    // batches) point at the site itself
+    const uint32_t cadr = S.base + (uint32_t)L.C;
+    const uint16_t *tab = P.cl_nb + (size_t)S.rank * nls * Z;
     auto neighbour_table = [&](const uint16_t *nbr, const uint8_t *zdeg) {
         for (int i = tid; i < nls * Z; i += nth) {
-            const int li = i / Z, d = i % Z;
-            const int q = ICM_IDX(nbr[pos_of(P, S, li) * Z + d], N, 20);
-            const int cq = q >= half;
-            const int hq = q - cq * half;
-            const uint32_t rq = (uint32_t)(hq / hs);
-            const int lq = cq * hs + hq % hs;
-            S.nb[i] = cl_map(S.base + L.C, rq) + 4u * (uint32_t)lq;
+            const int li = i / Z, d = i - li * Z;
+            int q = ICM_IDX(tab[i], ns, 20);
+            if constexpr (DIL) {
+                const int p = pos_of(P, S, li);
+                if (nbr[p * Z + d] == p) q = li;
+            }
+            S.nb[i] = (uint16_t)(cadr - S.win + 4u * (uint32_t)q);
         }
         if (!GAUSS && (DIL || !P.const_z))
             for (int li = tid; li < nls; li += nth) S.zdeg[li] = zdeg[pos_of(P, S, li)];
     };
     if constexpr (!DIL) neighbour_table(P.nbr, P.zdeg);
+    for (int li = tid; li < nls; li += nth) S.xoff[li] = P.cl_xoff[S.rank * nls + li];
+    for (int i = tid; i < L.nx; i += nth) {          // copies: (CTA, halo entry, last) -> cluster-window address
+        const uint32_t v = P.cl_xl[S.rank * L.nx + i];
+        S.xl[i] = cl_map(cadr + 4u * ((uint32_t)nls + (v & 0xffffu)), (v >> 16) & 0xffu) | (v >> 31);
+    }
+    if (L.ufg)
+        for (int i = tid; i < L.nh; i += nth) {      // halo entry -> the owner's first label word
+            const uint32_t v = P.cl_hown[S.rank * L.nh + i];
+            S.hlab[i] = cl_map(S.base + L.lab + 4u * (v & 0xffffu), v >> 16);
+        }
+    const uint16_t *hpos = P.cl_hpos + S.rank * L.nh;
     if (L.gord >= 0)
         for (int i = tid; i < nls; i += nth) S.gord[i] = P.cl_order[i];
     if constexpr (GAUSS) {
         for (int r = tid; r < 32 * G; r += nth) S.b2l[r] = r < R ? P.b2l[r] : 0.f;
     } else {
-        constexpr int TS = thr_stride(Z);
-        for (int i = tid; i < 32 * G * TS; i += nth) S.thr[i] = i < R * TS ? P.thr_metro[i] : 0u;
+        load_thr_rows<Z>(S.thr, P.thr_metro, R, G, tid, nth);
     }
 
     for (int slot = (int)cl_id(); slot < P.n_inst; slot += (int)cl_count()) {
         if (P.active && !P.active[slot]) continue;   // the same for every CTA of the cluster
-        for (int i = tid; i < G * nls; i += nth) {
-            const int g = i / nls, li = i % nls;
-            S.s[i] = P.spins[((size_t)slot * G + g) * N + pos_of(P, S, li)];
+        for (int i = tid; i < G * ns; i += nth) {
+            const int g = i >= ns, li = i - g * ns;
+            const int p = li < nls ? pos_of(P, S, li) : (int)hpos[li - nls];
+            if (p != 0xffff) S.s[i] = P.spins[((size_t)slot * G + g) * N + p];   // fewer entries than nh: unused
         }
         if constexpr (GAUSS) {
             for (int i = tid; i < nls * Z; i += nth)
@@ -1164,18 +1255,44 @@ __global__ void __launch_bounds__(kMaxThreadsWide, 1) cluster_kernel(const KPara
                     cm[0] = 0u;
                     cm[1] = 0u;
                 }
-            cl_sync();                               // buffers read remotely in the last step are free again
+            const bool icm = P.icm_every > 0 && t % (uint32_t)P.icm_every == 0 && P.n_icm > 0;
+            const bool pt = P.swap_every > 0 && t % (uint32_t)P.swap_every == 0 && nT > 1;
+            const bool meas = (long long)t >= t_meas;
             if (P.enable_metropolis) cl_metropolis<GAUSS, Z, DIL>(P, L, S, t, inst, tie);
-            if (P.icm_every > 0 && t % (uint32_t)P.icm_every == 0 && P.n_icm > 0)
-                cl_cluster_moves<GAUSS, Z>(P, L, S, t, inst, slot, trace);
-            if (P.swap_every > 0 && t % (uint32_t)P.swap_every == 0 && nT > 1) cl_pt_pass<GAUSS>(P, S, t, inst, slot, trace);
-            else cl_sync();                          // 2a and cluster flips visible to the observables
-            if ((long long)t >= t_meas) cl_measure<GAUSS, Z>(P, L, S, slot);
+            {   // the draws of steps 2b and 3, by the threads that share no energy
+                const int nicm = icm ? P.n_icm : 0, np = nT - 1, n = nicm + (pt ? 2 * np : 0);
+                const int at = ((R + 31) & ~31) < nth ? (R + 31) & ~31 : 0;
+                for (int i = tid < at ? tid + nth - at : tid - at; i < n; i += nth) {
+                    if (i < nicm) {
+                        uint32_t x[4];
+                        philox10k((uint32_t)i, t, 0u, (1u << 24) | inst, P.key, x);
+                        S.seed[i] = (int)x[0];
+                    } else {
+                        pt_draw<GAUSS>(i - nicm, np, t, inst, P.key, S.swap_x, P.thr_swap, P.swap_off, P.swap_len,
+                                       P.dbeta_l2e);
+                    }
+                }
+            }
+            if (P.enable_metropolis) {
+                cl_sync();
+                for (int r = tid; r < R; r += nth) {
+                    ET e = row_sum<ET>(S, S.Esw, R, r);
+                    if constexpr (!GAUSS) e = 2 * e - (DIL ? P.nb_inst[slot] : P.Nb);   // E = 2 U - (bonds present)
+                    ((ET *)S.E)[r] = e;
+                }
+            }
+            __syncthreads();
+            if (icm) cl_cluster_moves<GAUSS, Z>(P, L, S, t, slot, trace);
+            if (pt) cl_pt_pass<GAUSS>(P, S, slot, trace);
+            if (meas) cl_count<Z>(P, L, S, (int)(step & 1u));
+            cl_sync();               // ends the step: no CTA reads this step's words any more
+            if (meas && S.rank == 0) cl_accumulate<GAUSS>(P, S, slot, (int)(step & 1u));
         }
+        __syncthreads();
 
         for (int i = tid; i < G * nls; i += nth) {
-            const int g = i / nls, li = i % nls;
-            P.spins[((size_t)slot * G + g) * N + pos_of(P, S, li)] = S.s[i];
+            const int g = i >= nls, li = i - g * nls;
+            P.spins[((size_t)slot * G + g) * N + pos_of(P, S, li)] = S.s[g * ns + li];
         }
         if (S.rank == 0) {
             for (int r = tid; r < R; r += nth) {
@@ -1246,7 +1363,7 @@ int align_up16(int v) { return (v + 15) / 16 * 16; }
 }  // namespace
 
 ClusterLayout cluster_layout(int N, int Z, int R, int G, int nT, int K, int nwarps, bool gauss, int ufg,
-                             bool order)
+                             bool order, int nh, int nx)
 {
     ClusterLayout L{};
     L.K = K;
@@ -1254,6 +1371,9 @@ ClusterLayout cluster_layout(int N, int Z, int R, int G, int nT, int K, int nwar
     L.hs = (N / 2) / K;
     L.nls = 2 * L.hs;
     L.NWl = L.nls / 32;
+    L.nh = nh;
+    L.nx = nx;
+    L.ns = L.nls + nh;
     int o = 0;
     auto take = [&](int bytes) {
         o = align_up16(o);
@@ -1261,25 +1381,30 @@ ClusterLayout cluster_layout(int N, int Z, int R, int G, int nT, int K, int nwar
         o += bytes;
         return at;
     };
-    const int nls = L.nls;
-    L.s = take(G * nls * 4);
-    L.C = take(nls * 4);
-    L.nb = take(nls * Z * 4);
+    const int nls = L.nls, ns = L.ns;
+    L.C = take(ns * 4);            // first: its addresses fit the 16 bits of the neighbour table
+    L.s = take(G * ns * 4);
+    L.nb = take(nls * Z * 2);
+    L.xoff = take(nls * 2);
+    L.xl = take(nx * 4);
+    L.hlab = ufg ? take(nh * 4) : 0;
     L.coup = take(gauss ? nls * Z * 4 : nls);
     L.zdeg = take(nls);
     L.E = take(R * 4);
     L.Epart = take(nwarps * (R > 32 ? R : 32) * 4);
-    L.Esw = take(R * 4);
-    L.Epair = take(32 * 4);
-    L.rtab = take(gauss ? G * 32 * 4 : G * 32 * thr_stride(Z) * 4);
-    // the overlap masks are dead once the seeds are planted: the union-find
-    // labels take their place (one pair's labels are as large as the masks)
+    L.Esw = take(K * R * 4);
+    L.Epair = take(K * 32 * 4);
+    L.rtab = take(gauss ? G * 32 * 4 : G * 16 * 8 * 4);
+    // the overlap masks are dead once the seeds are planted: the domain words
+    // or the union-find labels take their place (one pair's labels are as
+    // large as the masks)
     L.lab = take((ufg > 1 ? ufg : 1) * nls * 4);
     L.mask = L.lab;
     L.sadr = take(32 * 4);
     L.sroot = take(kMaxUfGroup * 4);
     L.gord = order ? take(nls * 2) : -1;
-    L.cntloc = take(2 * 32 * 4);
+    L.cntloc = take(K * 64 * 4);
+    L.cntobs = take(2 * K * 64 * 4);
     L.flags = take(2 * 4);
     L.seed = take(32 * 4);
     L.esum = take(32 * 4);

@@ -274,6 +274,7 @@ struct icm_batch {
     int64_t launches = 0;
     std::vector<std::pair<void *, size_t>> allocs;   // device blocks and their sizes
     std::vector<uint16_t> h_pos2site;  // [N] site of each colour-major position
+    std::vector<uint16_t> h_nbr;       // [N][Z] neighbour positions of the lattice
     // staging buffers for loads and reads
     void *raw_coup = nullptr;     // [n_inst][Nb] int8 or float
     int8_t *raw_spins = nullptr;  // [n_inst][R][N]
@@ -290,6 +291,9 @@ struct icm_batch {
     int cluster_k = 0;
     int cl_growth = -1;               // cluster growth: -1 = by the library (scans), 0 = scans, 1 = union-find
     uint16_t *d_cl_order = nullptr;   // [N] growth order of the cluster layout's own sites (KParams::cl_order)
+    uint16_t *d_cl_tab = nullptr;     // ClusterTables of cl_tab_k CTAs, cl_tab_size 16-bit entries in all
+    size_t cl_tab_size = 0;
+    int cl_tab_k = 0, cl_nh = 0, cl_nx = 0;
     icm::ClusterLayout cl{};
     int n_clusters = 0;
     // wide (global-resident) layout: per-CTA scratch, grown on demand (in allocs)
@@ -556,6 +560,61 @@ bool host_tables(int lattice, int L, HostTables &t)
         }
     }
     return true;
+}
+
+// See ClusterTables.  A CTA's halo entries are numbered in ascending position;
+// nh and nx are the most that any CTA has.
+void cluster_tables(const uint16_t *nbr, int N, int Z, int K, ClusterTables &t)
+{
+    const int half = N / 2, hs = half / K, nls = 2 * hs;
+    std::vector<uint8_t> owner(N);
+    std::vector<uint16_t> local(N);
+    for (int c = 0, p = 0; c < 2; ++c)
+        for (int r = 0; r < K; ++r)
+            for (int i = 0; i < hs; ++i, ++p) {
+                owner[p] = (uint8_t)r;
+                local[p] = (uint16_t)(c * hs + i);
+            }
+    // which CTAs hold a copy of a position (K <= 8), then its entry in each halo
+    std::vector<uint8_t> holds(N, 0);
+    for (int p = 0; p < N; ++p)
+        for (int d = 0; d < Z; ++d) {
+            const int q = nbr[(size_t)p * Z + d];
+            if (owner[q] != owner[p]) holds[q] |= (uint8_t)(1u << owner[p]);
+        }
+    std::vector<int> nh(K, 0), nx(K, 0);
+    std::vector<uint16_t> entry((size_t)N * K, 0);
+    for (int p = 0; p < N; ++p)
+        for (int r = 0; holds[p] >> r; ++r)
+            if ((holds[p] >> r) & 1) {
+                entry[(size_t)p * K + r] = (uint16_t)nh[r]++;
+                ++nx[owner[p]];
+            }
+    t.nh = *std::max_element(nh.begin(), nh.end());
+    t.nx = *std::max_element(nx.begin(), nx.end());
+    t.nb.resize((size_t)N * Z);
+    t.hpos.assign((size_t)K * t.nh, 0xffff);
+    t.xoff.assign(N, 0xffff);
+    t.xl.assign((size_t)K * t.nx, 0);
+    t.hown.assign((size_t)K * t.nh, 0);
+    std::vector<int> used(K, 0);
+    for (int p = 0; p < N; ++p) {
+        const int r = owner[p], li = local[p];
+        uint16_t *row = t.nb.data() + ((size_t)r * nls + li) * Z;
+        for (int d = 0; d < Z; ++d) {
+            const int q = nbr[(size_t)p * Z + d];
+            row[d] = owner[q] == r ? local[q] : (uint16_t)(nls + entry[(size_t)q * K + r]);
+        }
+        if (!holds[p]) continue;
+        t.xoff[(size_t)r * nls + li] = (uint16_t)used[r];
+        for (int c = 0; holds[p] >> c; ++c) {
+            if (!((holds[p] >> c) & 1)) continue;
+            const uint32_t e = entry[(size_t)p * K + c], last = (holds[p] >> (c + 1)) ? 0u : 1u;
+            t.xl[(size_t)r * t.nx + used[r]++] = (last << 31) | ((uint32_t)c << 16) | e;
+            t.hpos[(size_t)c * t.nh + e] = (uint16_t)p;
+            t.hown[(size_t)c * t.nh + e] = ((uint32_t)r << 16) | (uint32_t)li;
+        }
+    }
 }
 
 }  // namespace icm
@@ -847,6 +906,7 @@ icm_status icm_batch_create(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t di
     if (e == cudaSuccess) e = UP(d_nbr, nbr);
     if (e == cudaSuccess) e = UP(d_pos2site, pos2site);
     b->h_pos2site = pos2site;
+    b->h_nbr = nbr;
     if (e == cudaSuccess) e = UP(d_zdeg, zdeg);
     if (e == cudaSuccess) e = UP(b->edge_bond, edge_bond);
     if (e == cudaSuccess) e = UP(d_id, ids);
@@ -1334,6 +1394,45 @@ static icm_status apply_threads(icm_batch *b, int threads)
     return ICM_OK;
 }
 
+// The cluster layout's tables of the batch's lattice and K CTAs, on the device.
+static icm_status upload_cluster_tables(icm_batch *b, int K)
+{
+    icm::KParams &P = b->kp;
+    if (b->cl_tab_k != K) {
+        icm::ClusterTables t;
+        icm::cluster_tables(b->h_nbr.data(), P.N, P.Z, K, t);
+        // 32-bit tables first, then the 16-bit ones
+        std::vector<uint16_t> all;
+        auto put = [&](const void *p, size_t bytes) {
+            all.insert(all.end(), (const uint16_t *)p, (const uint16_t *)p + bytes / 2);
+        };
+        put(t.xl.data(), t.xl.size() * 4);
+        put(t.hown.data(), t.hown.size() * 4);
+        put(t.nb.data(), t.nb.size() * 2);
+        put(t.hpos.data(), t.hpos.size() * 2);
+        put(t.xoff.data(), t.xoff.size() * 2);
+        if (all.size() > b->cl_tab_size) {
+            uint16_t *q = nullptr;
+            if (icm_status st = dalloc(b, &q, all.size())) return st;
+            b->d_cl_tab = q;
+            b->cl_tab_size = all.size();
+        }
+        ICM_CUDA(b->ctx, cudaMemcpyAsync(b->d_cl_tab, all.data(), all.size() * 2, cudaMemcpyHostToDevice,
+                                         b->ctx->stream));
+        ICM_CUDA(b->ctx, cudaStreamSynchronize(b->ctx->stream));   // the host tables are read by the copy
+        b->cl_tab_k = K;
+        b->cl_nh = t.nh;
+        b->cl_nx = t.nx;
+    }
+    const size_t n = (size_t)P.N, nh = (size_t)K * b->cl_nh, nx = (size_t)K * b->cl_nx;
+    P.cl_xl = (const uint32_t *)b->d_cl_tab;
+    P.cl_hown = P.cl_xl + nx;
+    P.cl_nb = (const uint16_t *)(P.cl_hown + nh);
+    P.cl_hpos = P.cl_nb + n * P.Z;
+    P.cl_xoff = P.cl_hpos + nh;
+    return ICM_OK;
+}
+
 // One instance per thread-block cluster of K CTAs (K = 2, 4, 8) of `threads`
 // threads each; see cluster_icm.cu.  K = 0 returns to one CTA per instance.
 static icm_status apply_cluster(icm_batch *b, int K, int threads)
@@ -1385,7 +1484,12 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
                                          b->ctx->stream));
         ICM_CUDA(b->ctx, cudaStreamSynchronize(b->ctx->stream));   // the host table is read by the copy
     }
-    icm::ClusterLayout L = icm::cluster_layout(P.N, P.Z, P.R, P.G, P.nT, K, threads / 32, b->gauss, ufg1, order);
+    if (icm_status st = upload_cluster_tables(b, K)) return st;
+    const int nh = b->cl_nh, nx = b->cl_nx;
+    icm::ClusterLayout L = icm::cluster_layout(P.N, P.Z, P.R, P.G, P.nT, K, threads / 32, b->gauss, ufg1, order, nh, nx);
+    // the neighbour table holds shared-memory offsets in 16 bits (a slice
+    // whose words reach past them exceeds the shared memory anyway)
+    if (4 * L.ns > 65536 - 4096) return fail(b->ctx, ICM_ERR_UNSUPPORTED, "cluster slice exceeds shared memory");
     if (L.total > b->ctx->max_smem_optin) return fail(b->ctx, ICM_ERR_UNSUPPORTED, "cluster slice exceeds shared memory");
     int clusters = 0;
     cudaError_t e = icm::cluster_occupancy(b->gauss, P.Z, P.diluted != 0, K, threads, L.total, &clusters);
@@ -1393,7 +1497,7 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
     if (clusters < 1) return fail(b->ctx, ICM_ERR_UNSUPPORTED, "cluster does not fit");
     for (int g = 2; ufg1 && g <= icm::kMaxUfGroup && g <= (P.n_icm > 1 ? P.n_icm : 1); ++g) {
         const icm::ClusterLayout Lg = icm::cluster_layout(P.N, P.Z, P.R, P.G, P.nT, K, threads / 32, b->gauss, g,
-                                                          order);
+                                                          order, nh, nx);
         int cg = 0;
         if (Lg.total > b->ctx->max_smem_optin ||
             icm::cluster_occupancy(b->gauss, P.Z, P.diluted != 0, K, threads, Lg.total, &cg) != cudaSuccess ||

@@ -126,6 +126,9 @@ struct KParams {
     // thread-block-cluster layout of 2D lattices: the own site that thread t
     // of a CTA grows as its j-th, at [4 t + j] (2 x 2 blocks of sites), or null
     const uint16_t *cl_order;     // [nls]
+    // thread-block-cluster layout: ClusterTables of the lattice and K
+    const uint16_t *cl_nb, *cl_hpos, *cl_xoff;
+    const uint32_t *cl_xl, *cl_hown;
     SmemLayout sm;
 };
 
@@ -162,37 +165,45 @@ SmemLayout smem_layout(int N, int Z, int R, int G, int nT, int n_icm, int nwarps
 
 // Thread-block-cluster layout (cluster_icm.cu): one instance per cluster of
 // K CTAs.  CTA r owns the positions [c half + r hs, c half + (r+1) hs) of
-// each colour c (hs = half / K), stored as local index li = c hs + i; every
-// per-site array has stride 4 bytes per local site, so the cluster-window
-// address of a neighbour's spin word also locates its other words.  Byte
-// offsets into each CTA's dynamic shared memory:
+// each colour c (hs = half / K), stored as local index li = c hs + i; the
+// local indices nls .. ns-1 are its halo, copies of the sites of other CTAs
+// that border its own (cluster_tables).  The spin and cluster words have
+// stride 4 bytes per local site, so the address of a neighbour's cluster word
+// also locates its spin words.  Byte offsets into each CTA's dynamic shared
+// memory:
 struct ClusterLayout {
     int K, hs, nls, NWl;   // CTAs, own sites per colour, own sites (2 hs), mask words (nls / 32)
-    int s;          // uint32 [G][nls]   spin words
-    int C;          // uint32 [nls]      cluster word: bit 2j = pair j, bit 2j + 1 = pair 16 + j
-    int nb;         // uint32 [nls][Z]   cluster-window address of the neighbour's cluster word C
+    int nh, nx, ns;        // halo entries, copies of own sites in other halos, nls + nh
+    int C;          // uint32 [ns]       cluster word: bit 2j = pair j, bit 2j + 1 = pair 16 + j
+    int s;          // uint32 [G][ns]    spin words
+    int nb;         // uint16 [nls][Z]   offset of the neighbour's cluster word C in the shared window
+    int xoff;       // uint16 [nls]      first entry of the site's copies in xl, 0xffff = none
+    int xl;         // uint32 [nx]       cluster-window address of a copy's cluster word, bit 0 = the site's last
+    int hlab;       // uint32 [nh]       cluster-window address of the halo site's first label word (union-find)
     int coup;       // float [nls][Z] (Gaussian) or uint8 [nls] sign bits (+-J)
     int zdeg;       // uint8 [nls]
     int E;          // float or int32 [R]       energies (the same in every CTA)
     int Epart;      // float or int32 [nwarps][max(R, 32)]
-    int Esw;        // float or int32 [R]       this CTA's share of the sweep energies (read remotely)
-    int Epair;      // float or int32 [32]      this CTA's share of the copy-a energies (read remotely)
+    int Esw;        // float or int32 [K][R]    every CTA's share of the sweep energies (written remotely)
+    int Epair;      // float or int32 [K][32]   every CTA's share of the copy-a energies (written remotely)
     int rtab;       // thresholds (+-J) or -2 beta log2(e) (Gaussian), as in SmemLayout
     int mask;       // uint32 [32][NWl]         overlap masks of the ICM pairs (in the lab region)
     int lab;        // uint32 [max(ufg, 1)][nls] union-find parents: the cluster-window address of the
-                    //                          parent's label word (a root holds its own address)
+                    //                          parent's label word (a root holds its own address);
+                    //                          growth by scans: the domain words
     int ufg;        // pairs per union-find group; 0 = growth by in-place scans (no labels)
     int sadr;       // uint32 [32]              cluster-window address of each pair's seed site (written remotely)
     int sroot;      // uint32 [8]               root of each group pair's seed
     int gord;       // uint16 [nls]             KParams::cl_order in shared memory, or -1 (site tid + j nth)
-    int cntloc;     // int32 [2][32]            q = -1 sites per colour block and pair (read remotely)
+    int cntloc;     // int32 [K][2][32]         every CTA's q = -1 sites per colour block and pair (written remotely)
+    int cntobs;     // int32 [2][K][2][32]      every CTA's observable counts, by step parity (written remotely, rank 0)
     int flags;      // uint32 [2]               growth-round stamps, by round parity (written remotely)
-    int seed;       // int32 [32]               1 = the pair moves
+    int seed;       // int32 [32]               seed draws, then 1 = the pair moves
     int esum;       // float or int32 [32]
     int flipw;      // uint32 [2]
     int csz;        // int32 [32]               this CTA's cluster sites per pair (read remotely)
     int swap_x, swap_mask;                      // as in SmemLayout
-    int cnt_n, cnt_d;   // int32 [32]           this CTA's observable counts (read remotely)
+    int cnt_n, cnt_d;   // int32 [32]           this CTA's counts
     int accE, acc64, nmeas;                     // observables (rank 0)
     int icmst;      // uint64 [2]               cluster moves and growth scans of this instance (rank 0)
     int total;
@@ -200,7 +211,17 @@ struct ClusterLayout {
 // ufg: pairs per union-find group (1..kMaxUfGroup), or 0 for growth by scans.
 constexpr int kMaxUfGroup = 8;
 ClusterLayout cluster_layout(int N, int Z, int R, int G, int nT, int K, int nwarps, bool gauss, int ufg,
-                             bool order);
+                             bool order, int nh, int nx);
+// Host-built tables of the layout for one lattice and K, every CTA's in turn:
+// the neighbours' local indices, the positions of its halo entries (0xffff =
+// unused), the first copy of each own site, the copies ((last << 31) | CTA
+// << 16 | halo entry) and the halo entries' owners (CTA << 16 | local index).
+struct ClusterTables {
+    int nh = 0, nx = 0;
+    std::vector<uint16_t> nb, hpos, xoff;   // [K][nls][Z], [K][nh], [K][nls]
+    std::vector<uint32_t> xl, hown;         // [K][nx], [K][nh]
+};
+void cluster_tables(const uint16_t *nbr, int N, int Z, int K, ClusterTables &t);
 cudaError_t launch_cluster(const KParams &P, const ClusterLayout &CL, bool gauss, int threads, int n_clusters,
                            uint32_t n_sweeps, cudaStream_t st);
 cudaError_t cluster_occupancy(bool gauss, int Z, bool dil, int K, int threads, int smem, int *clusters);
