@@ -440,6 +440,7 @@ icm_status refresh_dilution(icm_batch *b, int first, int count)
     const bool was_diluted = P.diluted != 0;
     P.diluted = diluted ? 1 : 0;
     P.const_z = diluted ? 0 : b->uniform_z;
+    P.row_kind = diluted ? 0 : icm::row_kind_of(b->lattice == ICM_SQUARE2D, b->L);
     if (b->cluster_k && diluted != was_diluted) {
         // the cluster layout switches to its kernels with per-instance tables
         // (or back): the clusters that fit are counted again
@@ -833,6 +834,9 @@ icm_status icm_batch_create(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t di
     P.N = N; P.Nb = g.Nb; P.nT = n_T; P.R = R; P.G = G; P.Z = Z; P.n_inst = n_inst; P.n_icm = n_icm;
     P.half = half; P.NW = (N + 31) / 32; P.const_z = uniform ? Z : 0;
     b->uniform_z = P.const_z;
+    P.L = L;
+    P.row_kind = icm::row_kind_of(lattice == ICM_SQUARE2D, L);
+    P.row_words = P.row_kind ? icm::row_words_of(P.row_kind, L) : 0;
     P.seed_lo = (uint32_t)(seed & 0xffffffffu);
     P.seed_hi = (uint32_t)(seed >> 32);
     for (int i = 0; i < 10; ++i) {                 // Philox round keys (Weyl sequence of the seed)

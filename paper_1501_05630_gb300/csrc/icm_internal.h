@@ -27,6 +27,22 @@ __host__ __device__
 #endif
 constexpr int mask_stride(int NW) { return NW | 1; }
 
+// Row forms of the cluster moves on undiluted 2D lattices (row_growth.cuh), by
+// the lattice's size; 0: the word-per-site form (other lattices, absent bonds,
+// L above 128 or not divisible into lanes of four rows).
+constexpr int kRows8 = 1, kRows16 = 2, kRows32 = 3, kRows64 = 4, kRows128 = 5;
+inline int row_kind_of(bool square2d, int L)
+{
+    if (!square2d) return 0;
+    return L <= 8 ? kRows8 : L <= 16 ? kRows16 : L <= 32 ? kRows32 : L <= 64 ? kRows64
+                                                        : L <= 128 && L % 4 == 0 ? kRows128 : 0;
+}
+// words of one pair's rows
+inline int row_words_of(int kind, int L)
+{
+    return kind == kRows8 ? (L + 3) / 4 : kind == kRows16 ? L / 2 : kind == kRows32 ? L : kind == kRows64 ? 2 * L : 4 * L;
+}
+
 // Bit-planes for the counts of a thread that takes `sites` sites, `half_sites`
 // of them of colour 1 with Z bonds each (at most kPlanes: the launch-shape
 // checks bound both counts by 255).
@@ -74,6 +90,8 @@ struct KParams {
     int diluted;                  // 1: some instance has absent bonds (J = 0): per-instance tables below
     int scratch_words;            // wide layout: uint32 words of scratch per CTA (cluster words, masks)
     uint32_t *scratch;            // wide layout: [grid][scratch_words]
+    int row_kind, row_words;      // row form of the cluster moves and words per pair (row_kind 0: none)
+    int L;                        // lattice size
     int cnt_planes;               // bit-planes that hold a thread's counts of sites and bonds
     // geometry, shared by all instances of the batch
     const uint16_t *nbr;          // [N][Z]

@@ -84,6 +84,8 @@ namespace icm {
 
 namespace {
 
+#include "row_growth.cuh"
+
 struct Sm {
     uint32_t *s;
     uint16_t *nbr;
@@ -480,30 +482,20 @@ __device__ __forceinline__ void pair_energies(const KParams &P, const Sm &S, con
     }
 }
 
-// ---------------------------------------------------------------------------
-// Steps 2a and 2b at every ICM temperature k < n_icm.
-//  (a) overlap masks of all pairs by a warp bit-matrix transpose (bit 2k of s ^ (s >> 1));
-//  (b) one thread per pair: n, the step-2a decision, the seed by rank;
-//  (c) copy-1 reversal of the flagged pairs, then the clusters of all pairs
-//      at once: C_p (bit 2k = site p in pair k's cluster, bit 2k + 1 the same
-//      for pair 16 + k) grows by
-//      C_p |= domain_p & OR(C of the neighbours) in rounds until a round
-//      changes nothing -- the fixed point is each seed's connected component
-//      of {q = -1};
-//  (d) flip in both copies (bits 2k, 2k + 1 of the spin word of the pair), then E_a from
-//      the spins and E_b = (E_a + E_b)_before - E_a (the move is isoenergetic).
-//      A traced sweep also recomputes E_b from the spins and records
-//      E_a + E_b of the two recomputed energies, so that the trace tests the
-//      conservation of E_a + E_b instead of restating it.
+// The overlap words of the sites grown word by word: steps (a) to (d) below for
+// lattices without the row form.  Returns the growth rounds; act0/act1: the
+// pairs that moved.
 template <bool GAUSS, int Z, bool WIDE>
-__device__ void cluster_moves(const KParams &P, const Sm &S, const Team &T, int slot, bool trace)
+__device__ __forceinline__ int site_moves(const KParams &P, const Sm &S, const Team &T, int slot, bool trace,
+                                          uint32_t &act0, uint32_t &act1)
 {
     using ET = typename std::conditional<GAUSS, float, int>::type;
     const int lane = threadIdx.x & 31, warp = T.tid >> 5, nwarps = T.nth >> 5;
     const int tid = T.tid, nth = T.nth;
     const int N = P.N, NW = P.NW, NS = mask_stride(P.NW), nicm = P.n_icm, G = P.G;
-    ET *E = (ET *)S.E;
+    const ET *E = (const ET *)S.E;
     ET *esum = (ET *)S.icm_esum_raw;
+
     ICM_SUB_INIT();
 
     // (a) masks and their counts; clear the cluster words
@@ -581,7 +573,7 @@ __device__ void cluster_moves(const KParams &P, const Sm &S, const Team &T, int 
     // pair 16 + j (the bit of pair j's copy a in the first spin word, and the
     // one below pair 16 + j's copy a in the second), so that the domain word
     // is q of the first word | q of the second word << 1.
-    uint32_t act0 = 0u, act1 = 0u;
+    act0 = act1 = 0u;
     for (int k = 0; k < nicm; ++k)
         if (S.icm_seed[k] >= 0) {
             if (k < 16) act0 |= 1u << (2 * k);
@@ -705,6 +697,158 @@ __device__ void cluster_moves(const KParams &P, const Sm &S, const Team &T, int 
             }
         }
     }
+    return rounds;
+}
+
+// Steps (a) to (d) in the row form (row_growth.cuh): the masks hold rows of
+// sites, a pair's count, reversal, seed and component are one warp's (or a few
+// lanes') work in registers, and both copies flip by XOR after the transpose
+// back to site words.  2D L=64 x 40 in wide CTAs: 1.83 to 0.99 ms per 16 sweeps
+// against the scans of site_moves; one 2D L=8 instance: 639 to 602 us per 64.
+template <int KIND>
+__device__ __forceinline__ int rows_pairs(const KParams &P, const Sm &S, const Team &T, int slot, bool trace, uint32_t *rows,
+                                          int RS)
+{
+    using Sh = RowShape<KIND>;
+    const int lane = threadIdx.x & 31, ul = lane & (Sh::U - 1), per = 32 / Sh::U;
+    int rounds = 0;
+    for (int k0 = (T.tid >> 5) * per; k0 < P.n_icm; k0 += (T.nth >> 5) * per) {
+        const int k = k0 + lane / Sh::U;
+        const bool have = k < P.n_icm;
+        uint32_t w[Sh::NW];
+        uint32_t *r = rows + k * RS + ul * Sh::NW;
+        const bool mine = have && ul * Sh::NW < P.row_words;
+#pragma unroll
+        for (int i = 0; i < Sh::NW; ++i) w[i] = mine ? r[i] : 0u;
+        const RowMove mv = rows_move<KIND>(w, have, have ? (uint32_t)S.icm_seed[k] : 0u, P.enable_2a != 0, P.L, lane);
+        rounds = max(rounds, mv.rounds);
+        if (mine)
+#pragma unroll
+            for (int i = 0; i < Sh::NW; ++i) r[i] = w[i];
+        __syncwarp();
+        if (have && ul == 0) {
+            S.icm_seed[k] = mv.seed;
+            if (mv.flipped) atomicOr(&S.flipw[(2 * k + 1) >> 5], 1u << ((2 * k + 1) & 31));
+            if (trace) {
+                const size_t o = (size_t)slot * P.nT + k;
+                P.tr_n_pre[o] = mv.n_pre;
+                P.tr_flip2a[o] = mv.flipped ? 1 : 0;
+                P.tr_seed[o] = mv.seed;
+                P.tr_csize[o] = 0;
+            }
+        }
+    }
+    return rounds;
+}
+
+template <bool GAUSS>
+__device__ __forceinline__ int row_moves(const KParams &P, const Sm &S, const Team &T, int slot, bool trace, uint32_t *rows,
+                                         uint32_t &act0, uint32_t &act1)
+{
+    using ET = typename std::conditional<GAUSS, float, int>::type;
+    const int lane = threadIdx.x & 31, warp = T.tid >> 5, nwarps = T.nth >> 5;
+    const int tid = T.tid, nth = T.nth;
+    const int N = P.N, L = P.L, nicm = P.n_icm, kind = P.row_kind, half = P.half, words = P.row_words;
+    const int RS = words | 1;
+    const bool two = P.G > 1;
+    const ET *E = (const ET *)S.E;
+    ET *esum = (ET *)S.icm_esum_raw;
+    // position of lane's site of word j, or -1
+    auto pos_of = [&](int j) {
+        int x, y;
+        row_site(kind, j, lane, x, y);
+        return x < L && y < L ? ((x + y) & 1) * half + ((y * L + x) >> 1) : -1;
+    };
+    const int kp = pair_of_bit(lane);
+    for (int j = warp; j < words; j += nwarps) {
+        const int p = pos_of(j);
+        const uint32_t x = p >= 0 ? overlap_word(S.s[ICM_IDX(p, N, 9)], two ? S.s[N + p] : 0u) : 0u;
+        const uint32_t col = warp_transpose32(x, lane);
+        if (kp < nicm) rows[kp * RS + j] = col;
+    }
+    if (tid < 2) S.flipw[tid] = 0u;
+    int *most = (int *)S.swap_mask;              // free until step 3
+    if (tid == 0) *most = 0;
+    for (int k = tid; k < nicm; k += nth) {
+        esum[k] = E[2 * k] + E[2 * k + 1];
+        if (trace) P.tr_eb[(size_t)slot * P.nT + k] = P.tr_ea[(size_t)slot * P.nT + k] = (float)(E[2 * k] + E[2 * k + 1]);
+    }
+    team_sync(T);
+    int rounds = 0;
+    switch (kind) {
+    case kRows8: rounds = rows_pairs<kRows8>(P, S, T, slot, trace, rows, RS); break;
+    case kRows16: rounds = rows_pairs<kRows16>(P, S, T, slot, trace, rows, RS); break;
+    case kRows32: rounds = rows_pairs<kRows32>(P, S, T, slot, trace, rows, RS); break;
+    case kRows64: rounds = rows_pairs<kRows64>(P, S, T, slot, trace, rows, RS); break;
+    default: rounds = rows_pairs<kRows128>(P, S, T, slot, trace, rows, RS); break;
+    }
+    if (lane == 0 && rounds) atomicMax(most, rounds);
+    team_sync(T);
+    act0 = act1 = 0u;
+    for (int k = 0; k < nicm; ++k)
+        if (S.icm_seed[k] >= 0) {
+            if (k < 16) act0 |= 1u << (2 * k);
+            else act1 |= 1u << (2 * (k - 16));
+        }
+    const uint32_t f0 = S.flipw[0], f1 = S.flipw[1];
+    rounds = *most;
+    if ((act0 | act1 | f0 | f1) == 0u) return rounds;
+    for (int j = warp; j < words; j += nwarps) {
+        const uint32_t c = warp_transpose32(kp < nicm ? rows[kp * RS + j] : 0u, lane);   // this lane's site
+        const int p = pos_of(j);
+        if (p < 0) continue;
+        const uint32_t e0 = c & 0x55555555u, e1 = (c >> 1) & 0x55555555u;
+        S.s[ICM_IDX(p, N, 9)] ^= f0 ^ (e0 | (e0 << 1));
+        if (two) S.s[N + p] ^= f1 ^ (e1 | (e1 << 1));
+        if (trace) {
+            for (uint32_t b = c; b; b &= b - 1u) atomicAdd(&S.cnt_d[pair_of_bit(__ffs(b) - 1)], 1);
+            if (P.tr_cmask) {
+                P.tr_cmask[(size_t)slot * 2 * N + 2 * p] = e0;
+                P.tr_cmask[(size_t)slot * 2 * N + 2 * p + 1] = e1;
+            }
+        }
+    }
+    return rounds;
+}
+
+// ---------------------------------------------------------------------------
+// Steps 2a and 2b at every ICM temperature k < n_icm.
+//  (a) overlap masks of all pairs by a warp bit-matrix transpose (bit 2k of s ^ (s >> 1));
+//  (b) one thread per pair: n, the step-2a decision, the seed by rank;
+//  (c) copy-1 reversal of the flagged pairs, then the clusters of all pairs
+//      at once: C_p (bit 2k = site p in pair k's cluster, bit 2k + 1 the same
+//      for pair 16 + k) grows by
+//      C_p |= domain_p & OR(C of the neighbours) in rounds until a round
+//      changes nothing -- the fixed point is each seed's connected component
+//      of {q = -1};
+//  (d) flip in both copies (bits 2k, 2k + 1 of the spin word of the pair), then E_a from
+//      the spins and E_b = (E_a + E_b)_before - E_a (the move is isoenergetic).
+//      A traced sweep also recomputes E_b from the spins and records
+//      E_a + E_b of the two recomputed energies, so that the trace tests the
+//      conservation of E_a + E_b instead of restating it.
+template <bool GAUSS, int Z, bool WIDE, bool DIL>
+__device__ void cluster_moves(const KParams &P, const Sm &S, const Team &T, int slot, bool trace)
+{
+    using ET = typename std::conditional<GAUSS, float, int>::type;
+    const int nwarps = T.nth >> 5, tid = T.tid, nth = T.nth;
+    const int N = P.N, nicm = P.n_icm;
+    ET *E = (ET *)S.E;
+    ET *esum = (ET *)S.icm_esum_raw;
+    ICM_SUB_INIT();
+
+    uint32_t act0 = 0u, act1 = 0u;
+    int rounds = 0;
+    bool by_rows = false;
+    if constexpr (Z == 4 && !DIL) by_rows = P.row_kind != 0;
+    if (by_rows) {
+        // the rows take the place of the masks and cluster words (the scratch in
+        // the wide layout): nicm (row_words | 1) words fit there for every L
+        if constexpr (Z == 4 && !DIL)
+            rounds = row_moves<GAUSS>(P, S, T, slot, trace, WIDE ? S.C : S.mask, act0, act1);
+    } else {
+        rounds = site_moves<GAUSS, Z, WIDE>(P, S, T, slot, trace, act0, act1);
+    }
+    const uint32_t actc = act0 | (act1 << 1);
 #ifdef ICM_PHASE_TIMERS
     if (tid == 0) atomicAdd(&g_icm_phase_cycles[11], (unsigned long long)rounds);
 #endif
@@ -717,7 +861,7 @@ __device__ void cluster_moves(const KParams &P, const Sm &S, const Team &T, int 
         team_sync(T);
         return;
     }
-    if (trace) {
+    if (trace && !by_rows) {
         // cluster sizes: counted once per cluster site; the cluster words as
         // [N][2] words, bit 2(k & 15) of word k >> 4 = site in pair k's cluster
         for (int p = tid; p < N; p += nth) {
@@ -1000,7 +1144,7 @@ __device__ __forceinline__ void run_instance(const KParams &P, const uint32_t (&
         step_draws<GAUSS>(P, key, S, T, t, inst, free_at < nth ? free_at : 0, icm, pt);
         team_sync(T);
         PHASE_MARK(0);
-        if (icm) cluster_moves<GAUSS, Z, WIDE>(P, S, T, slot, trace);   // steps 2a, 2b
+        if (icm) cluster_moves<GAUSS, Z, WIDE, DIL>(P, S, T, slot, trace);   // steps 2a, 2b
         PHASE_MARK(1);
         if (pt) pt_pass<GAUSS, WIDE>(P, S, T, slot, trace);              // step 3
         PHASE_MARK(2);

@@ -26,3 +26,14 @@ pytestmark = pytest.mark.gpu
 ])
 def test_sweep_edges(icm, kind, L, nT, n_inst, threads):
     _compare_sweeps(icm, kind, L, nT, 0.2, 2.0, 1.2, n_inst, 24, 0xE0 + L + nT, threads=threads)
+
+
+@pytest.mark.parametrize("L,nT,n_inst,threads", [
+    (2, 4, 2, None), (10, 20, 2, None), (14, 7, 1, 64), (16, 32, 1, None), (18, 6, 2, None), (30, 17, 1, 128),
+    (32, 5, 1, None), (34, 6, 1, None), (50, 18, 1, 256), (64, 4, 1, None), (68, 3, 1, None), (70, 3, 1, None),
+    (100, 2, 1, None),
+])
+def test_row_shapes(icm, L, nT, n_inst, threads):
+    """Every row shape of the 2D cluster moves (70: none, word per site), more and
+    fewer pairs than the team's warps take at once, shared-memory and wide CTAs."""
+    _compare_sweeps(icm, O.SQUARE2D, L, nT, 0.2, 1.5, 1.2, n_inst, 8, 0xF0 + L, threads=threads)
