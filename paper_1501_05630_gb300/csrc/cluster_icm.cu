@@ -36,10 +36,13 @@
 #include "icm_internal.h"
 #include "icm_device.cuh"
 
+#include <algorithm>
 #include <type_traits>
 
 namespace icm {
 namespace {
+
+#include "row_growth.cuh"
 
 __device__ __forceinline__ uint32_t cl_rank()
 {
@@ -129,6 +132,7 @@ struct CS {
     uint32_t *thr;
     float *b2l;
     uint32_t *mask, *lab, *sadr, *sroot;
+    uint32_t *rowm, *rowc, *rowi;
     uint16_t *gord;
     int *cntloc, *cntobs, *flags, *seed, *csz, *cnt_n, *cnt_d;   // cntloc [K][2][32], cntobs [2][K][2][32]
     uint32_t *flipw;
@@ -165,6 +169,9 @@ __device__ __forceinline__ CS make_cs(unsigned char *smem, const ClusterLayout &
     S.b2l = (float *)(smem + L.rtab);
     S.mask = (uint32_t *)(smem + L.mask);
     S.lab = (uint32_t *)(smem + L.lab);
+    S.rowm = (uint32_t *)(smem + L.rowm);
+    S.rowc = (uint32_t *)(smem + L.rowc);
+    S.rowi = (uint32_t *)(smem + L.rowi);
     S.sadr = (uint32_t *)(smem + L.sadr);
     S.sroot = (uint32_t *)(smem + L.sroot);
     S.gord = L.gord >= 0 ? (uint16_t *)(smem + L.gord) : nullptr;
@@ -729,17 +736,156 @@ __device__ __forceinline__ void cl_grow_uf(const KParams &P, const ClusterLayout
     }
 }
 
-// Steps 2a and 2b (see cluster_moves in pt_icm.cu).  S.seed holds the seed
-// draws on entry.
+// Steps 2a and 2b in the row form (row_growth.cuh): every CTA stores its rows of
+// a pair into the CTA that takes the pair (k mod K), whose warp counts,
+// reverses, seeds and grows it on its own and stores the cluster's rows back
+// into the CTAs that hold them or their halo copies.  Two cluster barriers,
+// where the scans took one each round of six.  2D L=128 x 20 on 8 x 1024:
+// CLROWFIG.
+template <int KIND>
+__device__ __forceinline__ void cl_rows_pairs(const KParams &P, const ClusterLayout &L, const CS &S, int slot, bool trace)
+{
+    using Sh = RowShape<KIND>;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int ul = lane & (Sh::U - 1), per = 32 / Sh::U, K = (int)S.K, pairs = (P.n_icm + K - 1) / K;
+    const int stride = L.rw + 2 * L.rh;
+    for (int s0 = warp * per; s0 < pairs; s0 += nwarps * per) {
+        const int s = s0 + lane / Sh::U, k = s * K + (int)S.rank;
+        const bool have = s < pairs && k < P.n_icm;
+        const bool mine = have && ul * Sh::NW < L.rs;
+        uint32_t w[Sh::NW];
+#pragma unroll
+        for (int i = 0; i < Sh::NW; ++i) w[i] = mine ? S.rowm[s * L.rs + ul * Sh::NW + i] : 0u;
+        const RowMove mv = rows_move<KIND>(w, have, have ? (uint32_t)S.seed[k] : 0u, P.enable_2a != 0, P.L, lane);
+        if (mine)
+#pragma unroll
+            for (int i = 0; i < Sh::NW; ++i) {
+                const int j = ul * Sh::NW + i, r = j / L.rw, jl = j - r * L.rw;   // CTA of the row, word in its rows
+                const uint32_t at = S.base + (uint32_t)L.rowc + 4u * (uint32_t)(k * stride);
+                cl_st(cl_map(at + 4u * (uint32_t)jl, (uint32_t)r), w[i]);
+                if (jl < L.rh)                     // the first rows follow the CTA before
+                    cl_st(cl_map(at + 4u * (uint32_t)(L.rw + L.rh + jl), (uint32_t)((r + K - 1) & (K - 1))), w[i]);
+                if (jl >= L.rw - L.rh)             // the last ones precede the CTA after
+                    cl_st(cl_map(at + 4u * (uint32_t)(L.rw + jl - (L.rw - L.rh)), (uint32_t)((r + 1) & (K - 1))), w[i]);
+            }
+        int size = 0;
+        if (trace) {
+#pragma unroll
+            for (int i = 0; i < Sh::NW; ++i) size += __popc(w[i]);
+#pragma unroll
+            for (int o = Sh::U / 2; o >= 1; o >>= 1) size += __shfl_xor_sync(kFull, size, o);
+        }
+        if (have && ul == 0) {
+            const uint32_t info = (uint32_t)(mv.seed >= 0) | ((uint32_t)mv.flipped << 1) | ((uint32_t)mv.rounds << 2);
+            for (int r = 0; r < K; ++r) cl_st(cl_map(S.base + (uint32_t)L.rowi + 4u * (uint32_t)k, (uint32_t)r), info);
+            if (trace) {
+                const size_t o = (size_t)slot * P.nT + k;
+                P.tr_n_pre[o] = mv.n_pre;
+                P.tr_flip2a[o] = mv.flipped ? 1 : 0;
+                P.tr_seed[o] = mv.seed;
+                P.tr_csize[o] = size;
+            }
+        }
+    }
+}
+
+template <bool GAUSS>
+__device__ __forceinline__ void cl_row_moves(const KParams &P, const ClusterLayout &L, const CS &S, int slot, bool trace,
+                                             uint32_t &act0, uint32_t &act1)
+{
+    using ET = typename std::conditional<GAUSS, float, int>::type;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int tid = threadIdx.x, nth = blockDim.x;
+    const int Lx = P.L, nicm = P.n_icm, kind = P.row_kind, K = (int)S.K, rank = (int)S.rank;
+    const int ns = S.ns, hs = S.hs, rows = Lx / K, y0 = rank * rows;
+    const bool two = P.G > 1;
+    const ET *E = (const ET *)S.E;
+    ET *esum = (ET *)S.esum;
+    const int kp = pair_of_bit(lane);
+    // local index of lane's site of the pair's word j of this CTA's rows, or -1
+    auto own_of = [&](int j) {
+        int x, y;
+        row_site(kind, rank * L.rw + j, lane, x, y);
+        return x < Lx ? ((x + y) & 1) * hs + (((y - y0) * Lx + x) >> 1) : -1;
+    };
+    for (int j = warp; j < L.rw; j += nwarps) {
+        const int li = own_of(j);
+        const uint32_t x = li >= 0 ? overlap_word(S.s[li], two ? S.s[ns + li] : 0u) : 0u;
+        const uint32_t col = warp_transpose32(x, lane);
+        if (kp < nicm) {
+            const int s = kp / K;
+            cl_st(cl_map(S.base + (uint32_t)L.rowm + 4u * (uint32_t)(s * L.rs + rank * L.rw + j), (uint32_t)(kp - s * K)), col);
+        }
+    }
+    for (int k = tid; k < nicm; k += nth) {
+        esum[k] = E[2 * k] + E[2 * k + 1];
+        if (trace && rank == 0)
+            P.tr_eb[(size_t)slot * P.nT + k] = P.tr_ea[(size_t)slot * P.nT + k] = (float)(E[2 * k] + E[2 * k + 1]);
+    }
+    cl_sync();
+    switch (kind) {
+    case kRows16: cl_rows_pairs<kRows16>(P, L, S, slot, trace); break;
+    case kRows32: cl_rows_pairs<kRows32>(P, L, S, slot, trace); break;
+    case kRows64: cl_rows_pairs<kRows64>(P, L, S, slot, trace); break;
+    default: cl_rows_pairs<kRows128>(P, L, S, slot, trace); break;
+    }
+    cl_sync();
+    uint32_t f0 = 0u, f1 = 0u, rounds = 0u;
+    act0 = act1 = 0u;
+    for (int k = 0; k < nicm; ++k) {
+        const uint32_t v = S.rowi[k];
+        const uint32_t bit = 1u << (2 * (k & 15));
+        if (v & 1u) (k < 16 ? act0 : act1) |= bit;
+        if (v & 2u) (k < 16 ? f0 : f1) |= bit << 1;
+        rounds = max(rounds, v >> 2);
+        if (tid == 0) S.seed[k] = (int)(v & 1u);
+    }
+    if (rank == 0 && tid == 0) {
+        S.icmst[0] += (unsigned)(__popc(act0) + __popc(act1));
+        S.icmst[1] += rounds;
+    }
+    // flip the own sites, then the two halo rows (entries by colour, row, x)
+    const int stride = L.rw + 2 * L.rh;
+    const int ya = (y0 + Lx - 1) % Lx, yb = (y0 + rows) % Lx;
+    for (int j = warp; j < stride; j += nwarps) {
+        const uint32_t c = warp_transpose32(kp < nicm ? S.rowc[kp * stride + j] : 0u, lane);
+        int li;
+        if (j < L.rw) {
+            li = own_of(j);
+        } else {
+            // the row before in the last row of its words, the row after in the first of its own
+            const bool after = j >= L.rw + L.rh;
+            const int jh = j - L.rw - (after ? L.rh : 0);
+            int x, y;
+            row_site(kind, jh, lane, x, y);
+            const int want = !after && kind == kRows16 ? 1 : 0;
+            y = y == want && x < Lx ? (after ? yb : ya) : -1;
+            const bool upper = after ? yb > ya : ya > yb;      // the larger of the two rows
+            li = y < 0 ? -1 : S.nls + ((x + y) & 1) * Lx + (upper ? Lx / 2 : 0) + (x >> 1);
+        }
+        if (li < 0) continue;
+        const uint32_t e0 = c & 0x55555555u, e1 = (c >> 1) & 0x55555555u;
+        S.s[li] ^= f0 ^ (e0 | (e0 << 1));
+        if (two) S.s[ns + li] ^= f1 ^ (e1 | (e1 << 1));
+        if (trace && P.tr_cmask && li < S.nls) {
+            uint32_t *cm = P.tr_cmask + ((size_t)slot * P.N + pos_of(P, S, li)) * 2;
+            cm[0] = e0;
+            cm[1] = e1;
+        }
+    }
+    __syncthreads();
+}
+
+// Steps 2a and 2b word by word (see site_moves in pt_icm.cu), or by union-find.
 template <bool GAUSS, int Z>
-__device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const CS &S, uint32_t t, int slot,
-                                 bool trace)
+__device__ __forceinline__ void cl_site_moves(const KParams &P, const ClusterLayout &L, const CS &S, uint32_t t, int slot,
+                                              bool trace, uint32_t &act0, uint32_t &act1)
 {
     using ET = typename std::conditional<GAUSS, float, int>::type;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int tid = threadIdx.x, nth = blockDim.x;
     const int N = P.N, nicm = P.n_icm, G = P.G, nls = S.nls, ns = S.ns, hs = S.hs, NWl = L.NWl;
-    ET *E = (ET *)S.E;
+    const ET *E = (const ET *)S.E;
     ET *esum = (ET *)S.esum;
 
     // (a) overlap masks of the own sites and their counts per colour block
@@ -830,7 +976,7 @@ __device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const
     else __syncthreads();
 
     // (c) step 2a on the own and halo sites, then the clusters of all pairs at once
-    uint32_t act0 = 0u, act1 = 0u;
+    act0 = act1 = 0u;
     for (int k = 0; k < nicm; ++k)
         if (S.seed[k]) {
             if (k < 16) act0 |= 1u << (2 * k);
@@ -961,6 +1107,30 @@ __device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const
         }
     }
     __syncthreads();
+}
+
+// Steps 2a and 2b (see cluster_moves in pt_icm.cu).  S.seed holds the seed
+// draws on entry.
+template <bool GAUSS, int Z, bool DIL>
+__device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const CS &S, uint32_t t, int slot,
+                                 bool trace)
+{
+    using ET = typename std::conditional<GAUSS, float, int>::type;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int tid = threadIdx.x, nth = blockDim.x;
+    const int nicm = P.n_icm, G = P.G, ns = S.ns, hs = S.hs;
+    const int kp = pair_of_bit(lane);
+    ET *E = (ET *)S.E;
+    const ET *esum = (const ET *)S.esum;
+    uint32_t act0 = 0u, act1 = 0u;
+    bool by_rows = false;
+    if constexpr (Z == 4 && !DIL) by_rows = L.rw > 0;
+    if (by_rows) {
+        if constexpr (Z == 4 && !DIL) cl_row_moves<GAUSS>(P, L, S, slot, trace, act0, act1);
+    } else {
+        cl_site_moves<GAUSS, Z>(P, L, S, t, slot, trace, act0, act1);
+    }
+    if (!(act0 | act1)) return;                      // the same decision in every CTA
     // copy-a energies of the moved pairs (cb = 0); a traced sweep then also
     // recomputes the copy-b energies (cb = 1) and records E_a + E_b of the two
     // recomputed energies, so that the trace tests the conservation of E_a + E_b
@@ -1043,6 +1213,7 @@ __device__ void cl_cluster_moves(const KParams &P, const ClusterLayout &L, const
             if (trace && S.rank == 0) {
                 const size_t o = (size_t)slot * P.nT + k;
                 if (cb == 0) {
+                    if (by_rows) continue;           // counted by the pair's warp
                     int cs = 0;
                     for (uint32_t r = 0; r < S.K; ++r) cs += (int)cl_ld(cl_map(S.base + L.csz + 4 * k, r));
                     P.tr_csize[o] = cs;
@@ -1282,7 +1453,7 @@ __global__ void __launch_bounds__(kMaxThreadsWide, 1) cluster_kernel(const KPara
                 }
             }
             __syncthreads();
-            if (icm) cl_cluster_moves<GAUSS, Z>(P, L, S, t, slot, trace);
+            if (icm) cl_cluster_moves<GAUSS, Z, DIL>(P, L, S, t, slot, trace);
             if (pt) cl_pt_pass<GAUSS>(P, S, slot, trace);
             if (meas) cl_count<Z>(P, L, S, (int)(step & 1u));
             cl_sync();               // ends the step: no CTA reads this step's words any more
@@ -1363,7 +1534,7 @@ int align_up16(int v) { return (v + 15) / 16 * 16; }
 }  // namespace
 
 ClusterLayout cluster_layout(int N, int Z, int R, int G, int nT, int K, int nwarps, bool gauss, int ufg,
-                             bool order, int nh, int nx)
+                             bool order, int nh, int nx, int row_kind, int Lx)
 {
     ClusterLayout L{};
     L.K = K;
@@ -1382,7 +1553,17 @@ ClusterLayout cluster_layout(int N, int Z, int R, int G, int nT, int K, int nwar
         return at;
     };
     const int nls = L.nls, ns = L.ns;
-    L.C = take(ns * 4);            // first: its addresses fit the 16 bits of the neighbour table
+    if (row_kind) {
+        L.rs = row_words_of(row_kind, Lx);
+        L.rw = L.rs / K;
+        L.rh = L.rs / Lx > 1 ? L.rs / Lx : 1;       // words of a row (or the word that holds it)
+    }
+    // in the row form the pairs' clusters take the place of the cluster words and
+    // the pairs' rows that of the masks
+    const int c_bytes = std::max(ns * 4, row_kind ? nT * (L.rw + 2 * L.rh) * 4 : 0);
+    const int m_bytes = std::max((ufg > 1 ? ufg : 1) * nls * 4, row_kind ? (nT + K - 1) / K * L.rs * 4 : 0);
+    L.C = take(c_bytes);           // first: its addresses fit the 16 bits of the neighbour table
+    L.rowc = L.C;
     L.s = take(G * ns * 4);
     L.nb = take(nls * Z * 2);
     L.xoff = take(nls * 2);
@@ -1398,8 +1579,9 @@ ClusterLayout cluster_layout(int N, int Z, int R, int G, int nT, int K, int nwar
     // the overlap masks are dead once the seeds are planted: the domain words
     // or the union-find labels take their place (one pair's labels are as
     // large as the masks)
-    L.lab = take((ufg > 1 ? ufg : 1) * nls * 4);
-    L.mask = L.lab;
+    L.lab = take(m_bytes);
+    L.mask = L.rowm = L.lab;
+    L.rowi = take(32 * 4);
     L.sadr = take(32 * 4);
     L.sroot = take(kMaxUfGroup * 4);
     L.gord = order ? take(nls * 2) : -1;

@@ -1490,7 +1490,9 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
     }
     if (icm_status st = upload_cluster_tables(b, K)) return st;
     const int nh = b->cl_nh, nx = b->cl_nx;
-    icm::ClusterLayout L = icm::cluster_layout(P.N, P.Z, P.R, P.G, P.nT, K, threads / 32, b->gauss, ufg1, order, nh, nx);
+    const int rows = ufg1 ? 0 : icm::cluster_row_kind(P.row_kind, b->L, K);
+    icm::ClusterLayout L = icm::cluster_layout(P.N, P.Z, P.R, P.G, P.nT, K, threads / 32, b->gauss, ufg1, order, nh, nx,
+                                               rows, b->L);
     // the neighbour table holds shared-memory offsets in 16 bits (a slice
     // whose words reach past them exceeds the shared memory anyway)
     if (4 * L.ns > 65536 - 4096) return fail(b->ctx, ICM_ERR_UNSUPPORTED, "cluster slice exceeds shared memory");
@@ -1501,7 +1503,7 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
     if (clusters < 1) return fail(b->ctx, ICM_ERR_UNSUPPORTED, "cluster does not fit");
     for (int g = 2; ufg1 && g <= icm::kMaxUfGroup && g <= (P.n_icm > 1 ? P.n_icm : 1); ++g) {
         const icm::ClusterLayout Lg = icm::cluster_layout(P.N, P.Z, P.R, P.G, P.nT, K, threads / 32, b->gauss, g,
-                                                          order, nh, nx);
+                                                          order, nh, nx, 0, b->L);
         int cg = 0;
         if (Lg.total > b->ctx->max_smem_optin ||
             icm::cluster_occupancy(b->gauss, P.Z, P.diluted != 0, K, threads, Lg.total, &cg) != cudaSuccess ||

@@ -37,6 +37,12 @@ inline int row_kind_of(bool square2d, int L)
     return L <= 8 ? kRows8 : L <= 16 ? kRows16 : L <= 32 ? kRows32 : L <= 64 ? kRows64
                                                         : L <= 128 && L % 4 == 0 ? kRows128 : 0;
 }
+// the row form on K CTAs, each with L / K whole rows in whole words
+inline int cluster_row_kind(int kind, int L, int K)
+{
+    const int per = kind == kRows8 ? 4 : kind == kRows16 ? 2 : 1;   // rows of a word
+    return kind && L % K == 0 && (L / K) % per == 0 ? kind : 0;
+}
 // words of one pair's rows
 inline int row_words_of(int kind, int L)
 {
@@ -209,6 +215,14 @@ struct ClusterLayout {
     int lab;        // uint32 [max(ufg, 1)][nls] union-find parents: the cluster-window address of the
                     //                          parent's label word (a root holds its own address);
                     //                          growth by scans: the domain words
+    // row form (undiluted 2D lattices whose CTAs hold whole row words): words of
+    // this CTA's rows of a pair, the two halo rows' words, row words of a pair's
+    // slot (0: word-per-site form)
+    int rw, rh, rs;
+    int rowm;       // uint32 [pairs of this CTA][rs]   whole pairs, every CTA's rows (written remotely, lab region)
+    int rowc;       // uint32 [nT][rw + 2 rh]           clusters: own rows, the row before, the row after (written
+                    //                                  remotely, C region)
+    int rowi;       // uint32 [32]              per pair: moves | flipped << 1 | rounds << 2 (written remotely)
     int ufg;        // pairs per union-find group; 0 = growth by in-place scans (no labels)
     int sadr;       // uint32 [32]              cluster-window address of each pair's seed site (written remotely)
     int sroot;      // uint32 [8]               root of each group pair's seed
@@ -229,7 +243,7 @@ struct ClusterLayout {
 // ufg: pairs per union-find group (1..kMaxUfGroup), or 0 for growth by scans.
 constexpr int kMaxUfGroup = 8;
 ClusterLayout cluster_layout(int N, int Z, int R, int G, int nT, int K, int nwarps, bool gauss, int ufg,
-                             bool order, int nh, int nx);
+                             bool order, int nh, int nx, int row_kind, int L);
 // Host-built tables of the layout for one lattice and K, every CTA's in turn:
 // the neighbours' local indices, the positions of its halo entries (0xffff =
 // unused), the first copy of each own site, the copies ((last << 31) | CTA
