@@ -753,28 +753,22 @@ __device__ __forceinline__ void cl_rows_pairs(const KParams &P, const ClusterLay
         const int s = s0 + lane / Sh::U, k = s * K + (int)S.rank;
         const bool have = s < pairs && k < P.n_icm;
         const bool mine = have && ul * Sh::NW < L.rs;
-        uint32_t w[Sh::NW];
-#pragma unroll
-        for (int i = 0; i < Sh::NW; ++i) w[i] = mine ? S.rowm[s * L.rs + ul * Sh::NW + i] : 0u;
-        const RowMove mv = rows_move<KIND>(w, have, have ? (uint32_t)S.seed[k] : 0u, P.enable_2a != 0, P.L, lane);
+        uint32_t *row = S.rowm + s * L.rs + ul * Sh::NW;
+        const RowMove mv = rows_move<KIND>(row, have, mine, have ? (uint32_t)S.seed[k] : 0u, P.enable_2a != 0, P.L);
         if (mine)
-#pragma unroll
+#pragma unroll 1
             for (int i = 0; i < Sh::NW; ++i) {
                 const int j = ul * Sh::NW + i, r = j / L.rw, jl = j - r * L.rw;   // CTA of the row, word in its rows
-                const uint32_t at = S.base + (uint32_t)L.rowc + 4u * (uint32_t)(k * stride);
-                cl_st(cl_map(at + 4u * (uint32_t)jl, (uint32_t)r), w[i]);
+                const uint32_t at = S.base + (uint32_t)L.rowc + 4u * (uint32_t)(k * stride), w = row[i];
+                cl_st(cl_map(at + 4u * (uint32_t)jl, (uint32_t)r), w);
                 if (jl < L.rh)                     // the first rows follow the CTA before
-                    cl_st(cl_map(at + 4u * (uint32_t)(L.rw + L.rh + jl), (uint32_t)((r + K - 1) & (K - 1))), w[i]);
+                    cl_st(cl_map(at + 4u * (uint32_t)(L.rw + L.rh + jl), (uint32_t)((r + K - 1) & (K - 1))), w);
                 if (jl >= L.rw - L.rh)             // the last ones precede the CTA after
-                    cl_st(cl_map(at + 4u * (uint32_t)(L.rw + jl - (L.rw - L.rh)), (uint32_t)((r + 1) & (K - 1))), w[i]);
+                    cl_st(cl_map(at + 4u * (uint32_t)(L.rw + jl - (L.rw - L.rh)), (uint32_t)((r + 1) & (K - 1))), w);
             }
-        int size = 0;
-        if (trace) {
-#pragma unroll
-            for (int i = 0; i < Sh::NW; ++i) size += __popc(w[i]);
-#pragma unroll
+        int size = mv.size;
+        if (trace)
             for (int o = Sh::U / 2; o >= 1; o >>= 1) size += __shfl_xor_sync(kFull, size, o);
-        }
         if (have && ul == 0) {
             const uint32_t info = (uint32_t)(mv.seed >= 0) | ((uint32_t)mv.flipped << 1) | ((uint32_t)mv.rounds << 2);
             for (int r = 0; r < K; ++r) cl_st(cl_map(S.base + (uint32_t)L.rowi + 4u * (uint32_t)k, (uint32_t)r), info);
@@ -830,16 +824,13 @@ __device__ __forceinline__ void cl_row_moves(const KParams &P, const ClusterLayo
     default: cl_rows_pairs<kRows128>(P, L, S, slot, trace); break;
     }
     cl_sync();
-    uint32_t f0 = 0u, f1 = 0u, rounds = 0u;
-    act0 = act1 = 0u;
-    for (int k = 0; k < nicm; ++k) {
-        const uint32_t v = S.rowi[k];
-        const uint32_t bit = 1u << (2 * (k & 15));
-        if (v & 1u) (k < 16 ? act0 : act1) |= bit;
-        if (v & 2u) (k < 16 ? f0 : f1) |= bit << 1;
-        rounds = max(rounds, v >> 2);
-        if (tid == 0) S.seed[k] = (int)(v & 1u);
-    }
+    const uint32_t info = lane < nicm ? S.rowi[lane] : 0u;
+    const uint32_t act = __ballot_sync(kFull, info & 1u), fl = __ballot_sync(kFull, info & 2u);
+    const uint32_t rounds = __reduce_max_sync(kFull, info >> 2);
+    if (tid < nicm) S.seed[tid] = (int)(info & 1u);
+    act0 = spread16(act & 0xFFFFu);
+    act1 = spread16(act >> 16);
+    const uint32_t f0 = spread16(fl & 0xFFFFu) << 1, f1 = spread16(fl >> 16) << 1;
     if (rank == 0 && tid == 0) {
         S.icmst[0] += (unsigned)(__popc(act0) + __popc(act1));
         S.icmst[1] += rounds;

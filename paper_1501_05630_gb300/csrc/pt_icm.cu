@@ -715,16 +715,9 @@ __device__ __forceinline__ int rows_pairs(const KParams &P, const Sm &S, const T
     for (int k0 = (T.tid >> 5) * per; k0 < P.n_icm; k0 += (T.nth >> 5) * per) {
         const int k = k0 + lane / Sh::U;
         const bool have = k < P.n_icm;
-        uint32_t w[Sh::NW];
-        uint32_t *r = rows + k * RS + ul * Sh::NW;
-        const bool mine = have && ul * Sh::NW < P.row_words;
-#pragma unroll
-        for (int i = 0; i < Sh::NW; ++i) w[i] = mine ? r[i] : 0u;
-        const RowMove mv = rows_move<KIND>(w, have, have ? (uint32_t)S.icm_seed[k] : 0u, P.enable_2a != 0, P.L, lane);
+        const RowMove mv = rows_move<KIND>(rows + k * RS + ul * Sh::NW, have, have && ul * Sh::NW < P.row_words,
+                                           have ? (uint32_t)S.icm_seed[k] : 0u, P.enable_2a != 0, P.L);
         rounds = max(rounds, mv.rounds);
-        if (mine)
-#pragma unroll
-            for (int i = 0; i < Sh::NW; ++i) r[i] = w[i];
         __syncwarp();
         if (have && ul == 0) {
             S.icm_seed[k] = mv.seed;
@@ -784,12 +777,9 @@ __device__ __forceinline__ int row_moves(const KParams &P, const Sm &S, const Te
     }
     if (lane == 0 && rounds) atomicMax(most, rounds);
     team_sync(T);
-    act0 = act1 = 0u;
-    for (int k = 0; k < nicm; ++k)
-        if (S.icm_seed[k] >= 0) {
-            if (k < 16) act0 |= 1u << (2 * k);
-            else act1 |= 1u << (2 * (k - 16));
-        }
+    const uint32_t act = __ballot_sync(kFull, lane < nicm && S.icm_seed[lane] >= 0);
+    act0 = spread16(act & 0xFFFFu);
+    act1 = spread16(act >> 16);
     const uint32_t f0 = S.flipw[0], f1 = S.flipw[1];
     rounds = *most;
     if ((act0 | act1 | f0 | f1) == 0u) return rounds;

@@ -6,10 +6,9 @@
 // The word-per-site form grows all pairs at once, but only one or two bonds per
 // scan, and a 2D cluster is 130-300 bonds deep (L = 64, 128).  Here a pair's
 // q = -1 sites are rows of bits held in the registers of one warp (or of 2 or
-// 8 lanes for small L): a step along a row is a shift of whole words, the run
-// to the right of a member is filled by one addition (the carry runs through
-// the ones of the domain), a step between rows of a lane is an AND-OR of
-// registers, and between lanes a shuffle.  No shared memory and no barrier is
+// 8 lanes for small L): a step along a row is a shift of whole words, a step
+// between rows of a lane is an AND-OR of registers, and between lanes a
+// shuffle.  No shared memory and no barrier is
 // touched until the component is complete.  Measured against the word-per-site
 // scans: see cluster_moves (pt_icm.cu) and cl_cluster_moves (cluster_icm.cu).
 //
@@ -73,7 +72,12 @@ __device__ __forceinline__ int grow_packed(uint32_t m, uint32_t &c, int L, int l
     return rounds;
 }
 
-// As above with rows of W words, RPL rows per lane (lane l holds rows RPL l ..).
+// As above with rows of W words, RPL rows per lane (lane l holds rows RPL l ..):
+// down and up through the lane's rows, each row with one bond to either side
+// as it is passed.  Bound by the latency of that chain (a warp has a pair, and
+// few warps share an SM sub-partition).  Filling runs by additions or taking
+// more steps per row needs fewer passes (17 against 25 on 128 x 128 sites at
+// 0.57) but a longer chain for each.
 template <int KIND>
 __device__ __forceinline__ int grow_rows(const uint32_t (&m)[RowShape<KIND>::NW], uint32_t (&c)[RowShape<KIND>::NW],
                                          int L, int lane, int nl)
@@ -83,35 +87,28 @@ __device__ __forceinline__ int grow_rows(const uint32_t (&m)[RowShape<KIND>::NW]
     const int bl = (L - 1) & 31;
     const bool last3 = W == 4 && ((L - 1) >> 5) == 3;      // a row's last word: 3 or 2 (W = 4), 1 (W = 2)
     auto row_end = [&](const uint32_t *w) { return W == 2 ? w[1] : last3 ? w[W - 1] : w[W - 2]; };
-    auto close = [&](int r) {
+    // one bond along row r, both ways: first to higher x, then to lower x
+    auto along = [&](int r, bool wrap_up) {
         uint32_t *cr = c + r * W;
         const uint32_t *mr = m + r * W;
-        cr[0] |= mr[0] & ((row_end(cr) >> bl) & 1u);
-        // to the right: m + c carries from every member to the end of its run
+        if (wrap_up) cr[0] |= mr[0] & ((row_end(cr) >> bl) & 1u);
         uint32_t t[W];
-        if constexpr (W == 2) {
-            asm("add.cc.u32 %0, %2, %4;\n\taddc.u32 %1, %3, %5;"
-                : "=&r"(t[0]), "=r"(t[1]) : "r"(mr[0]), "r"(mr[1]), "r"(cr[0]), "r"(cr[1]));
-        } else {
-            asm("add.cc.u32 %0, %4, %8;\n\taddc.cc.u32 %1, %5, %9;\n\taddc.cc.u32 %2, %6, %10;\n\taddc.u32 %3, %7, %11;"
-                : "=&r"(t[0]), "=&r"(t[1]), "=&r"(t[W - 2]), "=r"(t[W - 1])
-                : "r"(mr[0]), "r"(mr[1]), "r"(mr[W - 2]), "r"(mr[W - 1]), "r"(cr[0]), "r"(cr[1]), "r"(cr[W - 2]),
-                  "r"(cr[W - 1]));
+#pragma unroll
+        for (int j = 0; j < W; ++j) t[j] = j ? __funnelshift_l(cr[j - 1], cr[j], 1) : cr[0] << 1;
+#pragma unroll
+        for (int j = 0; j < W; ++j) cr[j] |= mr[j] & t[j];
+        if (!wrap_up) {
+            const uint32_t wrap = (cr[0] & 1u) << bl;
+            if constexpr (W == 2) cr[1] |= mr[1] & wrap;
+            else {
+                cr[W - 1] |= mr[W - 1] & (last3 ? wrap : 0u);
+                cr[W - 2] |= mr[W - 2] & (last3 ? 0u : wrap);
+            }
         }
 #pragma unroll
-        for (int j = 0; j < W; ++j) cr[j] |= mr[j] & ~t[j];
-        // to the left: two steps, from the row's end
-        const uint32_t wrap = (cr[0] & 1u) << bl;
-        if constexpr (W == 2) cr[1] |= mr[1] & wrap;
-        else {
-            cr[W - 1] |= mr[W - 1] & (last3 ? wrap : 0u);
-            cr[W - 2] |= mr[W - 2] & (last3 ? 0u : wrap);
-        }
+        for (int j = 0; j < W; ++j) t[j] = __funnelshift_r(cr[j], j + 1 < W ? cr[j + 1] : 0u, 1);
 #pragma unroll
-        for (int s = 0; s < 2; ++s)
-#pragma unroll
-            for (int j = W - 1; j >= 0; --j)
-                cr[j] |= mr[j] & __funnelshift_r(cr[j], j + 1 < W ? cr[j + 1] : 0u, 1);
+        for (int j = 0; j < W; ++j) cr[j] |= mr[j] & t[j];
     };
     int rounds = 0;
     for (;;) {
@@ -124,7 +121,7 @@ __device__ __forceinline__ int grow_rows(const uint32_t (&m)[RowShape<KIND>::NW]
             for (int r = 0; r < RPL; ++r) {
 #pragma unroll
                 for (int j = 0; j < W; ++j) c[r * W + j] |= m[r * W + j] & (r ? c[(r - 1) * W + j] : n[j]);
-                close(r);
+                along(r, true);
             }
 #pragma unroll
             for (int j = 0; j < W; ++j) n[j] = __shfl_sync(kFull, c[j], nxt);
@@ -132,7 +129,7 @@ __device__ __forceinline__ int grow_rows(const uint32_t (&m)[RowShape<KIND>::NW]
             for (int r = RPL - 1; r >= 0; --r) {
 #pragma unroll
                 for (int j = 0; j < W; ++j) c[r * W + j] |= m[r * W + j] & (r < RPL - 1 ? c[(r + 1) * W + j] : n[j]);
-                close(r);
+                along(r, false);
             }
         }
         rounds += 2;
@@ -162,18 +159,25 @@ __device__ __forceinline__ int grow_rows(const uint32_t (&m)[RowShape<KIND>::NW]
 }
 
 struct RowMove {
-    int n_pre, n, seed, rounds;   // q = -1 sites before and after step 2a; seed site, -1: none
+    int n_pre, seed, rounds;      // q = -1 sites before step 2a; seed site, -1: none; growth rounds
+    int size;                     // this lane's share of the cluster's sites
     bool flipped;
 };
 
-// Steps 2a and 2b of the pair whose q = -1 bits are w (before step 2a): w
-// becomes its cluster (0 when it has none).  Every lane of the warp calls;
-// lanes without a pair pass have = false.
+// Steps 2a and 2b of the pair whose q = -1 bits are the words at row (this
+// lane's, before step 2a; `mine`: the lane has words): they become its cluster
+// (0 when it has none).  Every lane of the warp calls; lanes without a pair
+// pass have = false.  Not inlined: the rows take half of the 64 registers of
+// the wide kernels, and next to the caller's values they were spilled inside
+// the growth loop (2D L=128 on 8 x 512: 47 of 105 us per sweep).
 template <int KIND>
-__device__ __forceinline__ RowMove rows_move(uint32_t (&w)[RowShape<KIND>::NW], bool have, uint32_t draw, bool enable_2a,
-                                             int L, int lane)
+__device__ __noinline__ RowMove rows_move(uint32_t *row, bool have, bool mine, uint32_t draw, bool enable_2a, int L)
 {
     using S = RowShape<KIND>;
+    const int lane = threadIdx.x & 31;
+    uint32_t w[S::NW];
+#pragma unroll
+    for (int k = 0; k < S::NW; ++k) w[k] = mine ? row[k] : 0u;
     constexpr int U = S::U, W = S::W, NW = S::NW, FB = S::FB;
     const int ul = lane & (U - 1), half = L * L / 2;
     const int nl = S::W > 1 ? L / S::RPL : (L + 32 / FB - 1) / (32 / FB);
@@ -186,7 +190,6 @@ __device__ __forceinline__ RowMove rows_move(uint32_t (&w)[RowShape<KIND>::NW], 
     int n = 0, n0 = 0;
 #pragma unroll
     for (int k = 0; k < NW; ++k) {
-        if (!have) w[k] = 0u;
         n += __popc(w[k]);
         n0 += __popc(w[k] & col0(k));
     }
@@ -217,7 +220,6 @@ __device__ __forceinline__ RowMove rows_move(uint32_t (&w)[RowShape<KIND>::NW], 
             w[k] = ~w[k] & valid;
         }
     }
-    mv.n = n;
     // the seed: the rank-th site in (colour, site) order
     uint32_t rank = __umulhi(draw, (uint32_t)n);
     const bool second = rank >= (uint32_t)n0;
@@ -263,7 +265,11 @@ __device__ __forceinline__ RowMove rows_move(uint32_t (&w)[RowShape<KIND>::NW], 
     mv.seed = seed;
     if constexpr (W == 1) mv.rounds = grow_packed<KIND>(w[0], c[0], L, lane, ul, nl);
     else mv.rounds = grow_rows<KIND>(w, c, L, lane, nl);
+    mv.size = 0;
 #pragma unroll
-    for (int k = 0; k < NW; ++k) w[k] = c[k];
+    for (int k = 0; k < NW; ++k) {
+        if (mine) row[k] = c[k];
+        mv.size += __popc(c[k]);
+    }
     return mv;
 }
