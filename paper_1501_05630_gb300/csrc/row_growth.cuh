@@ -73,11 +73,13 @@ __device__ __forceinline__ int grow_packed(uint32_t m, uint32_t &c, int L, int l
 }
 
 // As above with rows of W words, RPL rows per lane (lane l holds rows RPL l ..):
-// down and up through the lane's rows, each row with one bond to either side
-// as it is passed.  Bound by the latency of that chain (a warp has a pair, and
-// few warps share an SM sub-partition).  Filling runs by additions or taking
-// more steps per row needs fewer passes (17 against 25 on 128 x 128 sites at
-// 0.57) but a longer chain for each.
+// down through the lane's rows, each filling its runs to higher x, and up
+// again, each with two bonds to lower x.  A warp has a pair and few warps share
+// an SM sub-partition: bound by the ALU instructions of a pass, so the test for
+// completion and the rows' periodic seam come once in three passes.  Passes and
+// word operations per row on 128 x 128 sites at 0.57: this form 25 x 32, one
+// bond either way in both directions 25 x 40, runs and two bonds in both 17 x
+// 64.
 template <int KIND>
 __device__ __forceinline__ int grow_rows(const uint32_t (&m)[RowShape<KIND>::NW], uint32_t (&c)[RowShape<KIND>::NW],
                                          int L, int lane, int nl)
@@ -87,33 +89,53 @@ __device__ __forceinline__ int grow_rows(const uint32_t (&m)[RowShape<KIND>::NW]
     const int bl = (L - 1) & 31;
     const bool last3 = W == 4 && ((L - 1) >> 5) == 3;      // a row's last word: 3 or 2 (W = 4), 1 (W = 2)
     auto row_end = [&](const uint32_t *w) { return W == 2 ? w[1] : last3 ? w[W - 1] : w[W - 2]; };
-    // one bond along row r, both ways: first to higher x, then to lower x
-    auto along = [&](int r, bool wrap_up) {
+    // across the seam of the periodic row, both ways
+    auto seam = [&](int r) {
         uint32_t *cr = c + r * W;
         const uint32_t *mr = m + r * W;
-        if (wrap_up) cr[0] |= mr[0] & ((row_end(cr) >> bl) & 1u);
+        const uint32_t wrap = (cr[0] & 1u) << bl;
+        cr[0] |= mr[0] & ((row_end(cr) >> bl) & 1u);
+        if constexpr (W == 2) cr[1] |= mr[1] & wrap;
+        else {
+            cr[W - 1] |= mr[W - 1] & (last3 ? wrap : 0u);
+            cr[W - 2] |= mr[W - 2] & (last3 ? 0u : wrap);
+        }
+    };
+    // to higher x: m + c carries from every member through the ones of the domain
+    // to the end of its run
+    auto run = [&](int r) {
+        uint32_t *cr = c + r * W;
+        const uint32_t *mr = m + r * W;
         uint32_t t[W];
-#pragma unroll
-        for (int j = 0; j < W; ++j) t[j] = j ? __funnelshift_l(cr[j - 1], cr[j], 1) : cr[0] << 1;
-#pragma unroll
-        for (int j = 0; j < W; ++j) cr[j] |= mr[j] & t[j];
-        if (!wrap_up) {
-            const uint32_t wrap = (cr[0] & 1u) << bl;
-            if constexpr (W == 2) cr[1] |= mr[1] & wrap;
-            else {
-                cr[W - 1] |= mr[W - 1] & (last3 ? wrap : 0u);
-                cr[W - 2] |= mr[W - 2] & (last3 ? 0u : wrap);
-            }
+        if constexpr (W == 2) {
+            asm("add.cc.u32 %0, %2, %4;\n\taddc.u32 %1, %3, %5;"
+                : "=&r"(t[0]), "=r"(t[1]) : "r"(mr[0]), "r"(mr[1]), "r"(cr[0]), "r"(cr[1]));
+        } else {
+            asm("add.cc.u32 %0, %4, %8;\n\taddc.cc.u32 %1, %5, %9;\n\taddc.cc.u32 %2, %6, %10;\n\taddc.u32 %3, %7, %11;"
+                : "=&r"(t[0]), "=&r"(t[1]), "=&r"(t[W - 2]), "=r"(t[W - 1])
+                : "r"(mr[0]), "r"(mr[1]), "r"(mr[W - 2]), "r"(mr[W - 1]), "r"(cr[0]), "r"(cr[1]), "r"(cr[W - 2]),
+                  "r"(cr[W - 1]));
         }
 #pragma unroll
-        for (int j = 0; j < W; ++j) t[j] = __funnelshift_r(cr[j], j + 1 < W ? cr[j + 1] : 0u, 1);
+        for (int j = 0; j < W; ++j) cr[j] |= mr[j] & ~t[j];
+    };
+    // to lower x: two bonds
+    auto back = [&](int r) {
+        uint32_t *cr = c + r * W;
+        const uint32_t *mr = m + r * W;
 #pragma unroll
-        for (int j = 0; j < W; ++j) cr[j] |= mr[j] & t[j];
+        for (int s = 0; s < 2; ++s) {
+            uint32_t t[W];
+#pragma unroll
+            for (int j = 0; j < W; ++j) t[j] = __funnelshift_r(cr[j], j + 1 < W ? cr[j + 1] : 0u, 1);
+#pragma unroll
+            for (int j = 0; j < W; ++j) cr[j] |= mr[j] & t[j];
+        }
     };
     int rounds = 0;
     for (;;) {
 #pragma unroll 1
-        for (int it = 0; it < 2; ++it) {
+        for (int it = 0; it < 3; ++it) {
             uint32_t n[W];
 #pragma unroll
             for (int j = 0; j < W; ++j) n[j] = __shfl_sync(kFull, c[(RPL - 1) * W + j], prv);
@@ -121,7 +143,7 @@ __device__ __forceinline__ int grow_rows(const uint32_t (&m)[RowShape<KIND>::NW]
             for (int r = 0; r < RPL; ++r) {
 #pragma unroll
                 for (int j = 0; j < W; ++j) c[r * W + j] |= m[r * W + j] & (r ? c[(r - 1) * W + j] : n[j]);
-                along(r, true);
+                run(r);
             }
 #pragma unroll
             for (int j = 0; j < W; ++j) n[j] = __shfl_sync(kFull, c[j], nxt);
@@ -129,10 +151,12 @@ __device__ __forceinline__ int grow_rows(const uint32_t (&m)[RowShape<KIND>::NW]
             for (int r = RPL - 1; r >= 0; --r) {
 #pragma unroll
                 for (int j = 0; j < W; ++j) c[r * W + j] |= m[r * W + j] & (r < RPL - 1 ? c[(r + 1) * W + j] : n[j]);
-                along(r, false);
+                back(r);
             }
         }
-        rounds += 2;
+        rounds += 3;
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) seam(r);
         // complete when no site of the domain outside has a neighbour inside
         uint32_t open = 0u;
         uint32_t up[W], dn[W];

@@ -111,30 +111,44 @@ def sim(kind,L,neg,draw,en2a):
         RPL=W
         bl=(L-1)&31
         last=(L-1)>>5
-        def along(u, r, wrap_up):
-            cr = c[u][r * W:(r + 1) * W]
-            mr = w[u][r * W:(r + 1) * W]
-            if wrap_up:
-                cr[0] |= mr[0] & ((cr[last] >> bl) & 1)
-            t = [((cr[j] << 1) | (cr[j - 1] >> 31 if j else 0)) & M for j in range(W)]
-            cr = [cr[j] | (mr[j] & t[j]) for j in range(W)]
-            if not wrap_up:
-                cr[last] |= mr[last] & (((cr[0] & 1) << bl) & M)
-            t = [fsr(cr[j], cr[j + 1] if j + 1 < W else 0) for j in range(W)]
-            c[u][r * W:(r + 1) * W] = [cr[j] | (mr[j] & t[j]) for j in range(W)]
+        def row(words, r):
+            return words[r * W:(r + 1) * W]
+
+        def run(u, r):
+            cr, mr = row(c[u], r), row(w[u], r)
+            t = sum(mr[j] << (32 * j) for j in range(W)) + sum(cr[j] << (32 * j) for j in range(W))
+            c[u][r * W:(r + 1) * W] = [cr[j] | (mr[j] & ~(t >> (32 * j)) & M) for j in range(W)]
+
+        def back(u, r):
+            for _ in range(2):
+                cr, mr = row(c[u], r), row(w[u], r)
+                t = [fsr(cr[j], cr[j + 1] if j + 1 < W else 0) for j in range(W)]
+                c[u][r * W:(r + 1) * W] = [cr[j] | (mr[j] & t[j]) for j in range(W)]
+
+        def seam(u, r):
+            cr, mr = row(c[u], r), row(w[u], r)
+            wrap = ((cr[0] & 1) << bl) & M
+            cr[0] |= mr[0] & ((cr[last] >> bl) & 1)
+            cr[last] |= mr[last] & wrap
+            c[u][r * W:(r + 1) * W] = cr
 
         while True:
-            for it in range(2):
-                nn=[c[(nl-1 if u==0 else u-1)][(RPL-1)*W:] for u in range(U)]
+            for it in range(3):
+                nn = [row(c[nl - 1 if u == 0 else u - 1], RPL - 1) for u in range(U)]
                 for u in range(U):
                     for r in range(RPL):
-                        for j in range(W): c[u][r*W+j]|=w[u][r*W+j]&(c[u][(r-1)*W+j] if r else nn[u][j])
-                        along(u, r, True)
-                nn=[c[(0 if u>=nl-1 else u+1)][:W] for u in range(U)]
+                        for j in range(W):
+                            c[u][r * W + j] |= w[u][r * W + j] & (c[u][(r - 1) * W + j] if r else nn[u][j])
+                        run(u, r)
+                nn = [row(c[0 if u >= nl - 1 else u + 1], 0) for u in range(U)]
                 for u in range(U):
-                    for r in range(RPL-1,-1,-1):
-                        for j in range(W): c[u][r*W+j]|=w[u][r*W+j]&(c[u][(r+1)*W+j] if r<RPL-1 else nn[u][j])
-                        along(u, r, False)
+                    for r in range(RPL - 1, -1, -1):
+                        for j in range(W):
+                            c[u][r * W + j] |= w[u][r * W + j] & (c[u][(r + 1) * W + j] if r < RPL - 1 else nn[u][j])
+                        back(u, r)
+            for u in range(U):
+                for r in range(RPL):
+                    seam(u, r)
             op=0
             for u in range(U):
                 dn=c[(nl-1 if u==0 else u-1)][(RPL-1)*W:]
