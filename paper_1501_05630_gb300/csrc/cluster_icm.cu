@@ -39,6 +39,26 @@
 #include <algorithm>
 #include <type_traits>
 
+// The file is compiled three times so that the kernels build in parallel:
+// ICM_PART 0 = layout and dispatch (the default), 1 = kernels for +-J couplings,
+// 2 = Gaussian (cluster_pmj.cu and cluster_gauss.cu define the macro and include
+// this file).
+#ifndef ICM_PART
+#define ICM_PART 0
+#endif
+
+namespace icm {
+cudaError_t launch_cluster_pmj(const KParams &P, const ClusterLayout &L, int threads, int n_clusters, uint32_t n_sweeps,
+                               cudaStream_t st);
+cudaError_t launch_cluster_gauss(const KParams &P, const ClusterLayout &L, int threads, int n_clusters,
+                                 uint32_t n_sweeps, cudaStream_t st);
+cudaError_t cluster_occupancy_pmj(int Z, bool dil, bool lean, int K, int threads, int smem, int *clusters);
+cudaError_t cluster_occupancy_gauss(int Z, bool dil, bool lean, int K, int threads, int smem, int *clusters);
+int debug_check_cluster_pmj(unsigned int *out, int reset);
+int debug_check_cluster_gauss(unsigned int *out, int reset);
+}  // namespace icm
+
+#if ICM_PART != 0
 namespace icm {
 namespace {
 
@@ -313,12 +333,14 @@ __device__ __forceinline__ void cl_gauss_pass(const KParams &P, const CS &S, uin
             J[d] = S.Jd[li * Z + d];
             Jsum += J[d];
         }
-        const float *b2l = S.b2l + rbase;
+        const float *b2l = S.b2l + (rbase >> 1);
 #pragma unroll
         for (int qq = 0; qq < 2; ++qq) {
             if (qq < npairs8) {
                 uint32_t x[4], y[4];
                 philox10x2(site, t, (uint32_t)(rbase >> 2) + 2 * qq, inst, P.key, x, y);
+                const float4 bl4 = *reinterpret_cast<const float4 *>(b2l + 4 * qq);   // four temperatures
+                const float bl[4] = {bl4.x, bl4.y, bl4.z, bl4.w};
                 uint32_t f8 = 0u;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
@@ -327,17 +349,19 @@ __device__ __forceinline__ void cl_gauss_pass(const KParams &P, const CS &S, uin
 #pragma unroll
                     for (int d = 0; d < Z; ++d)
                         if ((nw[d] >> b) & 1u) h = fmaf(J[d], -2.f, h);
-                    const float sh = ((sw >> b) & 1u) ? -h : h;
+                    const float sh = neg_if(h, sw & (1u << b));
                     const uint32_t xr = i < 4 ? x[i] : y[i - 4];
-                    const uint32_t thr = __float2uint_rz(ex2_approx(fmaf(b2l[b], sh, 32.f)));
+                    const uint32_t thr = __float2uint_rz(ex2_approx(fmaf(bl[i >> 1], sh, 32.f)));
                     bool a;
                     if constexpr (DIL)   // diluted instance: Delta E = 0 accepted with probability 1/2
                         a = (sh < 0.f) || (sh == 0.f ? (!tie || xr < 0x80000000u) : (xr < thr));
                     else
                         a = (sh <= 0.f) || (xr < thr);
-                    f8 |= (uint32_t)a << i;
                     acc[b] -= sh;
-                    if (a) acc[b] += 2.f * sh;
+                    if (a) {
+                        f8 |= 1u << i;
+                        acc[b] += 2.f * sh;
+                    }
                 }
                 flip |= f8 << (8 * qq);
             }
@@ -1306,9 +1330,14 @@ __device__ __forceinline__ void cl_accumulate(const KParams &P, const CS &S, int
 }
 
 // ---------------------------------------------------------------------------
-template <bool GAUSS, int Z, bool DIL>
-__global__ void __launch_bounds__(kMaxThreadsWide, 1) cluster_kernel(const KParams P, const ClusterLayout L,
-                                                                    uint32_t n_sweeps)
+// MAXT: the widest CTA of the variant, which sets its registers a thread: 64
+// (1024) or 128 (512).  At 64 the kernel spills; at 128 fewer CTAs share an SM.
+// 3D Gaussian L=16 on 8 x 256, us per sweep: 20 instances 52.8 (64 registers) and
+// 42.9 (128), one 43.1 and 34.4, but 72 instances, more than the clusters
+// resident at 128 registers, 87.6 and 92.3.  So the host takes 128 where every
+// instance is resident with them (ClusterLayout::lean).
+template <bool GAUSS, int Z, bool DIL, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) cluster_kernel(const KParams P, const ClusterLayout L, uint32_t n_sweeps)
 {
     using ET = typename std::conditional<GAUSS, float, int>::type;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1354,7 +1383,7 @@ __global__ void __launch_bounds__(kMaxThreadsWide, 1) cluster_kernel(const KPara
     if (L.gord >= 0)
         for (int i = tid; i < nls; i += nth) S.gord[i] = P.cl_order[i];
     if constexpr (GAUSS) {
-        for (int r = tid; r < 32 * G; r += nth) S.b2l[r] = r < R ? P.b2l[r] : 0.f;
+        for (int k = tid; k < 16 * G; k += nth) S.b2l[k] = k < nT ? P.b2l[2 * k] : 0.f;
     } else {
         load_thr_rows<Z>(S.thr, P.thr_metro, R, G, tid, nth);
     }
@@ -1478,11 +1507,11 @@ __global__ void __launch_bounds__(kMaxThreadsWide, 1) cluster_kernel(const KPara
     }
 }
 
-template <bool GAUSS, int Z, bool DIL>
+template <bool GAUSS, int Z, bool DIL, int MAXT>
 cudaError_t launch_cluster_t(const KParams &P, const ClusterLayout &L, int threads, int n_clusters, uint32_t n_sweeps,
                              cudaStream_t st)
 {
-    auto kern = cluster_kernel<GAUSS, Z, DIL>;
+    auto kern = cluster_kernel<GAUSS, Z, DIL, MAXT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -1500,10 +1529,10 @@ cudaError_t launch_cluster_t(const KParams &P, const ClusterLayout &L, int threa
     return cudaLaunchKernelEx(&cfg, kern, P, L, n_sweeps);
 }
 
-template <bool GAUSS, int Z, bool DIL>
+template <bool GAUSS, int Z, bool DIL, int MAXT>
 cudaError_t cluster_occupancy_t(int K, int threads, int smem, int *clusters)
 {
-    auto kern = cluster_kernel<GAUSS, Z, DIL>;
+    auto kern = cluster_kernel<GAUSS, Z, DIL, MAXT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -1520,8 +1549,97 @@ cudaError_t cluster_occupancy_t(int K, int threads, int smem, int *clusters)
     return cudaOccupancyMaxActiveClusters(clusters, kern, &cfg);
 }
 
-int align_up16(int v) { return (v + 15) / 16 * 16; }
 
+constexpr bool kPartGauss = ICM_PART == 2;
+
+template <int Z, bool DIL>
+cudaError_t launch_part_zd(const KParams &P, const ClusterLayout &L, int threads, int n_clusters, uint32_t n_sweeps,
+                           cudaStream_t st)
+{
+    return L.lean ? launch_cluster_t<kPartGauss, Z, DIL, kLeanThreads>(P, L, threads, n_clusters, n_sweeps, st)
+                  : launch_cluster_t<kPartGauss, Z, DIL, kMaxThreadsWide>(P, L, threads, n_clusters, n_sweeps, st);
+}
+
+template <int Z>
+cudaError_t launch_part_z(const KParams &P, const ClusterLayout &L, int threads, int n_clusters, uint32_t n_sweeps,
+                          cudaStream_t st)
+{
+    return P.diluted ? launch_part_zd<Z, true>(P, L, threads, n_clusters, n_sweeps, st)
+                     : launch_part_zd<Z, false>(P, L, threads, n_clusters, n_sweeps, st);
+}
+
+cudaError_t launch_part(const KParams &P, const ClusterLayout &L, int threads, int n_clusters, uint32_t n_sweeps,
+                        cudaStream_t st)
+{
+    switch (P.Z) {
+    case 4: return launch_part_z<4>(P, L, threads, n_clusters, n_sweeps, st);
+    case 6: return launch_part_z<6>(P, L, threads, n_clusters, n_sweeps, st);
+    case 8: return launch_part_z<8>(P, L, threads, n_clusters, n_sweeps, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+template <int Z>
+cudaError_t occupancy_part_z(bool dil, bool lean, int K, int threads, int smem, int *clusters)
+{
+    if (lean)
+        return dil ? cluster_occupancy_t<kPartGauss, Z, true, kLeanThreads>(K, threads, smem, clusters)
+                   : cluster_occupancy_t<kPartGauss, Z, false, kLeanThreads>(K, threads, smem, clusters);
+    return dil ? cluster_occupancy_t<kPartGauss, Z, true, kMaxThreadsWide>(K, threads, smem, clusters)
+               : cluster_occupancy_t<kPartGauss, Z, false, kMaxThreadsWide>(K, threads, smem, clusters);
+}
+
+cudaError_t occupancy_part(int Z, bool dil, bool lean, int K, int threads, int smem, int *clusters)
+{
+    switch (Z) {
+    case 4: return occupancy_part_z<4>(dil, lean, K, threads, smem, clusters);
+    case 6: return occupancy_part_z<6>(dil, lean, K, threads, smem, clusters);
+    case 8: return occupancy_part_z<8>(dil, lean, K, threads, smem, clusters);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+int check_part(unsigned int *out, int reset)
+{
+#ifdef ICM_CHECKED
+    if (cudaMemcpyFromSymbol(out, g_icm_check, sizeof(unsigned int) * 4) != cudaSuccess) return -4;
+    if (reset) {
+        unsigned int z[4] = {};
+        if (cudaMemcpyToSymbol(g_icm_check, z, sizeof(z)) != cudaSuccess) return -4;
+    }
+    return 0;
+#else
+    (void)out;
+    (void)reset;
+    return -7;
+#endif
+}
+
+}  // namespace
+
+#if ICM_PART == 1
+#define ICM_CL_NAME(f) f##_pmj
+#else
+#define ICM_CL_NAME(f) f##_gauss
+#endif
+cudaError_t ICM_CL_NAME(launch_cluster)(const KParams &P, const ClusterLayout &L, int threads, int n_clusters,
+                                        uint32_t n_sweeps, cudaStream_t st)
+{
+    return launch_part(P, L, threads, n_clusters, n_sweeps, st);
+}
+cudaError_t ICM_CL_NAME(cluster_occupancy)(int Z, bool dil, bool lean, int K, int threads, int smem, int *clusters)
+{
+    return occupancy_part(Z, dil, lean, K, threads, smem, clusters);
+}
+int ICM_CL_NAME(debug_check_cluster)(unsigned int *out, int reset) { return check_part(out, reset); }
+
+}  // namespace icm
+
+#else  // ICM_PART == 0
+
+namespace icm {
+namespace {
+int align_up16(int v) { return (v + 15) / 16 * 16; }
 }  // namespace
 
 ClusterLayout cluster_layout(int N, int Z, int R, int G, int nT, int K, int nwarps, bool gauss, int ufg,
@@ -1598,40 +1716,34 @@ ClusterLayout cluster_layout(int N, int Z, int R, int G, int nT, int K, int nwar
 cudaError_t launch_cluster(const KParams &P, const ClusterLayout &L, bool gauss, int threads, int n_clusters,
                            uint32_t n_sweeps, cudaStream_t st)
 {
-    if (threads > kMaxThreadsWide || L.K < 1 || L.hs % 32) return cudaErrorInvalidValue;
+    if (threads > (L.lean ? kLeanThreads : kMaxThreadsWide) || L.K < 1 || L.hs % 32) return cudaErrorInvalidValue;
     if (P.diluted && (!P.nbr_inst || !P.zdeg_inst || !P.nb_inst)) return cudaErrorInvalidValue;
-#define ICM_LAUNCH_CL(G_, Z_)                                                                          \
-    (P.diluted ? launch_cluster_t<G_, Z_, true>(P, L, threads, n_clusters, n_sweeps, st)               \
-               : launch_cluster_t<G_, Z_, false>(P, L, threads, n_clusters, n_sweeps, st))
-    if (gauss) return P.Z == 4 ? ICM_LAUNCH_CL(true, 4) : P.Z == 6 ? ICM_LAUNCH_CL(true, 6) : ICM_LAUNCH_CL(true, 8);
-    return P.Z == 4 ? ICM_LAUNCH_CL(false, 4) : P.Z == 6 ? ICM_LAUNCH_CL(false, 6) : ICM_LAUNCH_CL(false, 8);
-#undef ICM_LAUNCH_CL
+    return gauss ? launch_cluster_gauss(P, L, threads, n_clusters, n_sweeps, st)
+                 : launch_cluster_pmj(P, L, threads, n_clusters, n_sweeps, st);
 }
 
-cudaError_t cluster_occupancy(bool gauss, int Z, bool dil, int K, int threads, int smem, int *clusters)
+cudaError_t cluster_occupancy(bool gauss, int Z, bool dil, bool lean, int K, int threads, int smem, int *clusters)
 {
-    if (Z != 4 && Z != 6 && Z != 8) return cudaErrorInvalidValue;
-#define ICM_OCC_CL(G_, Z_)                                                                             \
-    (dil ? cluster_occupancy_t<G_, Z_, true>(K, threads, smem, clusters)                                \
-         : cluster_occupancy_t<G_, Z_, false>(K, threads, smem, clusters))
-    if (gauss) return Z == 4 ? ICM_OCC_CL(true, 4) : Z == 6 ? ICM_OCC_CL(true, 6) : ICM_OCC_CL(true, 8);
-    return Z == 4 ? ICM_OCC_CL(false, 4) : Z == 6 ? ICM_OCC_CL(false, 6) : ICM_OCC_CL(false, 8);
-#undef ICM_OCC_CL
+    return gauss ? cluster_occupancy_gauss(Z, dil, lean, K, threads, smem, clusters)
+                 : cluster_occupancy_pmj(Z, dil, lean, K, threads, smem, clusters);
 }
 
 }  // namespace icm
 
 #ifdef ICM_CHECKED
-// Checked builds: the check word of the thread-block-cluster kernels (guarded
-// neighbour positions, seed sites and histogram bins; site codes 20-22), read
+// Checked builds: the check words of the thread-block-cluster kernels (guarded
+// neighbour positions, seed sites and histogram bins; site codes 20-23), read
 // like icm_debug_check reads those of the fused kernels.
 extern "C" int icm_debug_check_cluster(unsigned int *out, int reset)
 {
-    if (cudaMemcpyFromSymbol(out, icm::g_icm_check, sizeof(unsigned int) * 4) != cudaSuccess) return -4;
-    if (reset) {
-        unsigned int z[4] = {};
-        if (cudaMemcpyToSymbol(icm::g_icm_check, z, sizeof(z)) != cudaSuccess) return -4;
-    }
+    unsigned int a[4], b[4];
+    int rc = icm::debug_check_cluster_pmj(a, reset);
+    if (!rc) rc = icm::debug_check_cluster_gauss(b, reset);
+    if (rc) return rc;
+    out[0] = a[0] + b[0];
+    for (int i = 1; i < 4; ++i) out[i] = a[0] ? a[i] : b[i];
     return 0;
 }
 #endif
+
+#endif  // ICM_PART

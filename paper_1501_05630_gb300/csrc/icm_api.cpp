@@ -1498,7 +1498,7 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
     if (4 * L.ns > 65536 - 4096) return fail(b->ctx, ICM_ERR_UNSUPPORTED, "cluster slice exceeds shared memory");
     if (L.total > b->ctx->max_smem_optin) return fail(b->ctx, ICM_ERR_UNSUPPORTED, "cluster slice exceeds shared memory");
     int clusters = 0;
-    cudaError_t e = icm::cluster_occupancy(b->gauss, P.Z, P.diluted != 0, K, threads, L.total, &clusters);
+    cudaError_t e = icm::cluster_occupancy(b->gauss, P.Z, P.diluted != 0, false, K, threads, L.total, &clusters);
     if (e != cudaSuccess) return cuda_fail(b->ctx, e, "cluster occupancy");
     if (clusters < 1) return fail(b->ctx, ICM_ERR_UNSUPPORTED, "cluster does not fit");
     for (int g = 2; ufg1 && g <= icm::kMaxUfGroup && g <= (P.n_icm > 1 ? P.n_icm : 1); ++g) {
@@ -1506,11 +1506,19 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
                                                           order, nh, nx, 0, b->L);
         int cg = 0;
         if (Lg.total > b->ctx->max_smem_optin ||
-            icm::cluster_occupancy(b->gauss, P.Z, P.diluted != 0, K, threads, Lg.total, &cg) != cudaSuccess ||
+            icm::cluster_occupancy(b->gauss, P.Z, P.diluted != 0, false, K, threads, Lg.total, &cg) != cudaSuccess ||
             cg < clusters)
             break;
         L = Lg;
     }
+    // 128 registers a thread where that keeps every instance resident
+    int lean = 0;
+    if (threads <= icm::kLeanThreads &&
+        icm::cluster_occupancy(b->gauss, P.Z, P.diluted != 0, true, K, threads, L.total, &lean) != cudaSuccess) {
+        (void)cudaGetLastError();
+        lean = 0;
+    }
+    L.lean = lean >= b->n_inst ? 1 : 0;
     b->cluster_k = K;
     b->cl = L;
     P.cl_order = order ? b->d_cl_order : nullptr;

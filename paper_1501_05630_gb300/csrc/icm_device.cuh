@@ -84,6 +84,14 @@ __device__ __forceinline__ float ex2_approx(float x)
     return y;
 }
 
+// c ? -h : h, as one predicated negation (the compiler's select takes two
+// instructions on the busier ALU pipe).
+__device__ __forceinline__ float neg_if(float h, uint32_t c)
+{
+    asm("{.reg .pred q; setp.ne.u32 q, %1, 0; @q neg.f32 %0, %0;}" : "+f"(h) : "r"(c));
+    return h;
+}
+
 // ---------------------------------------------------------------------------
 // Step 3 (the PT pass).  For each copy c the swaps (k, k+1), k = 0 .. np-1, are
 // decided in ascending k; an accepted swap moves the configuration at k up to

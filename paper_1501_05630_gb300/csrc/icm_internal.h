@@ -70,7 +70,7 @@ struct SmemLayout {
     int coup;       // float [N][Z] (Gaussian) or uint8 [N] bit d = (J < 0) (+-J)
     int E;          // float or int32 [R]
     int Epart;      // float or int32 [nwarps][max(R, 32)]
-    int rtab;       // uint32 [16 G][8] threshold rows (+-J) or float [32 G] -2 beta log2(e) (Gaussian)
+    int rtab;       // uint32 [16 G][8] threshold rows (+-J) or float [16 G] -2 beta log2(e) (Gaussian)
     int icm_mask;   // uint32 [n_icm][mask_stride(NW)] overlap masks per ICM pair
     int icm_C;      // uint32 [N]        cluster bits of every pair (bit 2k: pair k, bit 2k + 1: pair 16 + k)
     int swap_x;     // uint32 [2][32]
@@ -196,6 +196,7 @@ SmemLayout smem_layout(int N, int Z, int R, int G, int nT, int n_icm, int nwarps
 // also locates its spin words.  Byte offsets into each CTA's dynamic shared
 // memory:
 struct ClusterLayout {
+    int lean;              // 1: the variant with 128 registers a thread (CTAs up to kLeanThreads)
     int K, hs, nls, NWl;   // CTAs, own sites per colour, own sites (2 hs), mask words (nls / 32)
     int nh, nx, ns;        // halo entries, copies of own sites in other halos, nls + nh
     int C;          // uint32 [ns]       cluster word: bit 2j = pair j, bit 2j + 1 = pair 16 + j
@@ -240,6 +241,7 @@ struct ClusterLayout {
     int icmst;      // uint64 [2]               cluster moves and growth scans of this instance (rank 0)
     int total;
 };
+constexpr int kLeanThreads = 512;
 // ufg: pairs per union-find group (1..kMaxUfGroup), or 0 for growth by scans.
 constexpr int kMaxUfGroup = 8;
 ClusterLayout cluster_layout(int N, int Z, int R, int G, int nT, int K, int nwarps, bool gauss, int ufg,
@@ -256,7 +258,7 @@ struct ClusterTables {
 void cluster_tables(const uint16_t *nbr, int N, int Z, int K, ClusterTables &t);
 cudaError_t launch_cluster(const KParams &P, const ClusterLayout &CL, bool gauss, int threads, int n_clusters,
                            uint32_t n_sweeps, cudaStream_t st);
-cudaError_t cluster_occupancy(bool gauss, int Z, bool dil, int K, int threads, int smem, int *clusters);
+cudaError_t cluster_occupancy(bool gauss, int Z, bool dil, bool lean, int K, int threads, int smem, int *clusters);
 int fused_threads(int N);
 int fused_threads_wide(int N);
 // uint32 words of per-CTA scratch of the wide layout (the cluster words and the

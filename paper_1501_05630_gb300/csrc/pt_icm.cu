@@ -242,15 +242,21 @@ __device__ __forceinline__ void gauss_pass(const KParams &P, const uint32_t (&ke
 #pragma unroll
         for (int d = 0; d < Z; ++d) {
             nw[d] = sg[ICM_IDX(q[d], N, 1)] >> sh0;
-            J[d] = S.Jd[ICM_IDX(p * Z + d, N * Z, 2)];
+            if (!(d & 1)) {                             // rows of Z floats, Z even
+                const float2 v = *reinterpret_cast<const float2 *>(S.Jd + ICM_IDX(p * Z + d, N * Z, 2));
+                J[d] = v.x;
+                J[d + 1] = v.y;
+            }
             Jsum += J[d];
         }
-        const float *b2l = S.b2l + rbase;
+        const float *b2l = S.b2l + (rbase >> 1);
 #pragma unroll
         for (int qq = 0; qq < 2; ++qq) {
             if (qq < npairs8) {
                 uint32_t x[4], y[4];
                 philox10x2(site, t, (uint32_t)(rbase >> 2) + 2 * qq, inst, key, x, y);
+                const float4 bl4 = *reinterpret_cast<const float4 *>(b2l + 4 * qq);   // four temperatures
+                const float bl[4] = {bl4.x, bl4.y, bl4.z, bl4.w};
                 uint32_t f8 = 0u;                           // this group's accepted bits
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
@@ -263,9 +269,9 @@ __device__ __forceinline__ void gauss_pass(const KParams &P, const uint32_t (&ke
                     // compared as rz(x) < 2^(32 + b2l sh) in fp32 (b2l = -2 beta log2 e):
                     // for sh <= 0 the right side is >= 2^32 > rz(x), so Delta E <= 0 is
                     // always accepted
-                    const float sh = ((sw >> b) & 1u) ? -h : h;
+                    const float sh = neg_if(h, sw & (1u << b));
                     const uint32_t xr = i < 4 ? x[i] : y[i - 4];
-                    const float lim = ex2_approx(fmaf(b2l[b], sh, 32.f));
+                    const float lim = ex2_approx(fmaf(bl[i >> 1], sh, 32.f));
                     bool a;
                     if constexpr (DIL) {
                         // diluted instance: Delta E = 0 (a site without bonds) is
@@ -274,9 +280,11 @@ __device__ __forceinline__ void gauss_pass(const KParams &P, const uint32_t (&ke
                     } else {
                         a = __uint2float_rz(xr) < lim;
                     }
-                    f8 |= (uint32_t)a << i;
                     acc[b] -= sh;                           // e = -s'h: -sh, or +sh after a flip
-                    if (a) acc[b] += 2.f * sh;
+                    if (a) {
+                        f8 |= 1u << i;
+                        acc[b] += 2.f * sh;
+                    }
                 }
                 flip |= f8 << (8 * qq);
             }
@@ -1032,7 +1040,7 @@ __device__ __forceinline__ void load_tables(const KParams &P, Sm &S, const Team 
         }
     }
     if constexpr (GAUSS) {
-        for (int r = tid; r < 32 * G; r += nth) S.b2l[r] = r < R ? P.b2l[r] : 0.f;
+        for (int k = tid; k < 16 * G; k += nth) S.b2l[k] = k < nT ? P.b2l[2 * k] : 0.f;
     } else {
         load_thr_rows<Z>(S.thr, P.thr_metro, R, G, tid, nth);
     }
