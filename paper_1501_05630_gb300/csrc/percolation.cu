@@ -1,8 +1,13 @@
 // percolation.cu -- site percolation on the supported lattices (the paper's
 // Supplemental Material: largest-cluster statistics and the Binder ratio of
-// the chimera lattice).  One CTA per mask: a lock-free union-find in shared
-// memory (roots hook to the smaller index with atomicCAS, finds halve paths),
-// then a count per root and a block maximum.
+// the chimera lattice).  One CTA per mask.  Every bond joins the two colours,
+// so only colour-0 sites are nodes of the union-find: an occupied colour-1 site
+// hangs under its first occupied neighbour for good and links that one with
+// its other occupied neighbours (lock-free: roots hook to the smaller index
+// with atomicCAS, finds halve paths); then sites are counted per root.  Bound
+// by the latency of the finds; per site the masks take a bit, the parents and
+// counts together 4 bytes, so several CTAs share an SM.  20000 masks of chimera
+// C_32 at p = 0.387: 14.1 to 6.3 ms against all sites as nodes with 8 bytes.
 #include "icmpt.h"
 
 #include <string>
@@ -70,39 +75,81 @@ __device__ __forceinline__ bool occupied(const uint8_t *masks, const uint16_t *p
     return c0 < thr;
 }
 
+// Bytes of a CTA's shared memory: parents (int) and 16-bit counts of the
+// colour-0 sites, the link of every colour-1 site (16 bits), occupancy bits.
+__host__ __device__ inline int percolation_smem(int N) { return 2 * N + N + N + (N + 31) / 32 * 4; }
+
+constexpr uint32_t kNone = 0xffffu, kAlone = 0xfffeu;   // links: empty site, occupied site without neighbours
+
 template <int Z>
 __global__ void __launch_bounds__(256) largest_cluster_kernel(const uint8_t *__restrict__ masks, int n_masks, int N,
                                                               const uint16_t *__restrict__ nbr,
                                                               const uint16_t *__restrict__ pos2site, uint32_t thr,
                                                               uint32_t k0, uint32_t k1, int32_t *__restrict__ smax)
 {
-    extern __shared__ int sh[];
-    int *parent = sh;                  // [N], -1 = empty
-    int *count = sh + N;               // [N]
+    extern __shared__ __align__(16) int sh[];
+    const int half = N >> 1, lane = threadIdx.x & 31;
+    int *parent = sh;                                       // [half]
+    uint32_t *count = (uint32_t *)(sh + half);              // two colour-0 sites to a word, [half / 2]
+    uint16_t *link = (uint16_t *)(count + (half >> 1));     // [half]
+    uint32_t *occ = (uint32_t *)(link + half);              // [(N + 31) / 32]
     __shared__ int best;
+    auto occupied_at = [&](int p) { return (occ[p >> 5] >> (p & 31)) & 1u; };
+    // both 16-bit halves of a count stay below 2^16: a cluster has at most N sites
+    auto add = [&](int root, int n) { atomicAdd(&count[root >> 1], (uint32_t)n << (16 * (root & 1))); };
     for (long long m = blockIdx.x; m < n_masks; m += gridDim.x) {
-        for (int p = threadIdx.x; p < N; p += blockDim.x) {
-            parent[p] = occupied(masks, pos2site, N, m, p, thr, k0, k1) ? p : -1;
-            count[p] = 0;
+        for (int p0 = threadIdx.x - lane; p0 < N; p0 += blockDim.x) {
+            const int p = p0 + lane;
+            const uint32_t w = __ballot_sync(0xffffffffu, p < N && occupied(masks, pos2site, N, m, p < N ? p : 0, thr, k0, k1));
+            if (lane == 0) occ[p0 >> 5] = w;
         }
+        for (int p = threadIdx.x; p < half; p += blockDim.x) parent[p] = p;
+        for (int i = threadIdx.x; i < half >> 1; i += blockDim.x) count[i] = 0u;
         if (threadIdx.x == 0) best = 0;
         __syncthreads();
-        for (int p = threadIdx.x; p < N; p += blockDim.x) {
-            if (parent[p] < 0) continue;
+        for (int j = threadIdx.x; j < half; j += blockDim.x) {
+            const int p = half + j;
+            uint32_t first = kNone;
+            if (occupied_at(p)) {
+                first = kAlone;
+                const uint32_t *row = (const uint32_t *)(nbr + p * Z);
+                uint32_t q2[Z / 2];
 #pragma unroll
-            for (int d = 0; d < Z; ++d) {
-                const int q = nbr[p * Z + d];
-                if (q > p && ((volatile int *)parent)[q] >= 0) unite(parent, p, q);
+                for (int i = 0; i < Z / 2; ++i) q2[i] = __ldg(row + i);
+#pragma unroll
+                for (int d = 0; d < Z; ++d) {
+                    const int q = (int)((d & 1) ? q2[d >> 1] >> 16 : q2[d >> 1] & 0xffffu);
+                    if (q >= half || !occupied_at(q)) continue;   // padding names the site itself
+                    if (first == kAlone) first = (uint32_t)q;
+                    else unite(parent, (int)first, q);
+                }
             }
+            link[j] = (uint16_t)first;
         }
         __syncthreads();
-        for (int p = threadIdx.x; p < N; p += blockDim.x)
-            if (parent[p] >= 0) atomicAdd(&count[find_root(parent, p)], 1);
+        // a thread adds runs of sites with the same root in one atomic
+        int mx = 0, root = -1, n = 0;
+        auto one = [&](int q) {
+            const int r = find_root(parent, q);
+            if (r != root) {
+                if (n) add(root, n);
+                root = r;
+                n = 0;
+            }
+            ++n;
+        };
+        for (int p = threadIdx.x; p < half; p += blockDim.x) {
+            if (occupied_at(p)) one(p);
+            const uint32_t f = link[p];
+            if (f == kAlone) mx = 1;
+            else if (f != kNone) one((int)f);
+        }
+        if (n) add(root, n);
         __syncthreads();
-        int mx = 0;
-        for (int p = threadIdx.x; p < N; p += blockDim.x) mx = max(mx, count[p]);
+        for (int i = threadIdx.x; i < half >> 1; i += blockDim.x)
+            mx = max(mx, (int)max(count[i] & 0xffffu, count[i] >> 16));
         for (int o = 16; o >= 1; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if ((threadIdx.x & 31) == 0) atomicMax(&best, mx);
+        if (lane == 0) atomicMax(&best, mx);
         __syncthreads();
         if (threadIdx.x == 0) smax[m] = best;
         __syncthreads();
@@ -124,11 +171,11 @@ icm_status percolation(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t n_masks
         return ICM_ERR_ARG;
     }
     const int N = tab.N, Z = tab.Z;
-    const size_t smem = (size_t)N * 8;
-    if (smem > 200 * 1024) {
+    if ((size_t)N * 8 > 200 * 1024) {        // also keeps the 16-bit links and counts in range
         icm::set_ctx_error(ctx, "icm_percolation: lattice too large for one CTA");
         return ICM_ERR_UNSUPPORTED;
     }
+    const size_t smem = (size_t)percolation_smem(N);
     cudaStream_t st = icm::ctx_stream(ctx);
     const bool dev = (flags & ICM_DEVICE_PTR) != 0;
     uint16_t *d_nbr = nullptr, *d_p2s = nullptr;
