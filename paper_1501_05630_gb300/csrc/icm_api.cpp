@@ -845,7 +845,7 @@ icm_status icm_batch_create(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t di
         bool wide = sm0.total > ctx->max_smem_optin;
         int c0 = 0;
         if (!wide && N / 2 > icm::kMaxThreads &&
-            icm::fused_occupancy(b->gauss, Z, false, threads, sm0.total, &c0) == cudaSuccess && c0 <= 2)
+            icm::fused_occupancy(b->gauss, Z, icm::kLayoutShared, threads, sm0.total, &c0) == cudaSuccess && c0 <= 2)
             wide = true;
         (void)cudaGetLastError();
         if (wide) threads = icm::fused_threads_wide(N);
@@ -1399,16 +1399,32 @@ static icm_status apply_threads(icm_batch *b, int threads)
     const int half = P.N / 2;
     if (((half + threads - 1) / threads) * P.Z >= 256 || (P.N + threads - 1) / threads >= 256)
         return fail(b->ctx, ICM_ERR_UNSUPPORTED, "too many sites per thread for the observable counters");
-    const bool wide = threads > icm::kMaxThreads;
-    const icm::SmemLayout sm = icm::smem_layout(P.N, P.Z, P.R, P.G, P.nT, b->n_icm, threads / 32, b->gauss, wide);
+    int layout = threads > icm::kMaxThreads ? icm::kLayoutWide : icm::kLayoutShared;
+    icm::SmemLayout sm = icm::smem_layout(P.N, P.Z, P.R, P.G, P.nT, b->n_icm, threads / 32, b->gauss,
+                                          layout == icm::kLayoutWide);
     if (sm.total > b->ctx->max_smem_optin)
         return fail(b->ctx, ICM_ERR_UNSUPPORTED, "instance needs " + std::to_string(sm.total) +
                                                      " bytes of shared memory at this width; widths above 128 "
                                                      "threads keep it in global memory");
     int ctas = 0;
-    cudaError_t e = icm::fused_occupancy(b->gauss, P.Z, wide, threads, sm.total, &ctas);
+    cudaError_t e = icm::fused_occupancy(b->gauss, P.Z, layout, threads, sm.total, &ctas);
     if (e != cudaSuccess) return cuda_fail(b->ctx, e, "occupancy");
     if (ctas < 1) return fail(b->ctx, ICM_ERR_UNSUPPORTED, "kernel does not fit");
+    if (layout == icm::kLayoutWide) {
+        // a wide CTA whose instance fits its shared memory keeps it there, where
+        // that leaves as many CTAs on an SM as the instances can use
+        const icm::SmemLayout big = icm::smem_layout(P.N, P.Z, P.R, P.G, P.nT, b->n_icm, threads / 32, b->gauss, false);
+        const int sms = b->ctx->num_sms, use = std::min(ctas, (b->n_inst + sms - 1) / sms);
+        int cb = 0;
+        if (big.total <= b->ctx->max_smem_optin &&
+            icm::fused_occupancy(b->gauss, P.Z, icm::kLayoutBig, threads, big.total, &cb) == cudaSuccess && cb >= use) {
+            layout = icm::kLayoutBig;
+            sm = big;
+            ctas = cb;
+        }
+        (void)cudaGetLastError();
+    }
+    const bool wide = layout == icm::kLayoutWide;
     const int slots = b->ctx->num_sms * ctas;
     const int grid = b->n_inst < slots ? b->n_inst : slots;
     const int words = icm::wide_scratch_words(P.N);
@@ -1424,7 +1440,7 @@ static icm_status apply_threads(icm_batch *b, int threads)
     b->cluster_k = 0;
     b->n_clusters = 0;
     P.sm = sm;
-    P.wide = wide ? 1 : 0;
+    P.wide = layout;
     P.scratch = wide ? b->scratch : nullptr;
     P.scratch_words = wide ? words : 0;
     P.cnt_planes = icm::count_planes((P.N + threads - 1) / threads, (half + threads - 1) / threads, P.Z);

@@ -11,6 +11,9 @@ constexpr int kMaxZ = 8;          // largest degree of the supported graphs (4D 
 constexpr int kMaxR = 64;         // replicas per instance (2 N_T, N_T <= 32)
 constexpr int kMaxThreads = 128;  // threads per CTA of the fused kernel, shared-memory layout
 constexpr int kMaxThreadsWide = 1024;  // threads per CTA of the fused kernel, global-resident layout
+// One-CTA layouts: the instance in shared memory with CTAs up to kMaxThreads;
+// in global memory with wider CTAs; in shared memory with wider CTAs.
+constexpr int kLayoutShared = 0, kLayoutWide = 1, kLayoutBig = 2;
 constexpr int kPlanes = 8;        // bit-planes of the vertical counters (counts < 256 per thread)
 
 // Entries per replica of the +-J Metropolis threshold table, indexed by
@@ -92,7 +95,7 @@ struct SmemLayout {
 struct KParams {
     int N, Nb, nT, R, G, Z, n_inst, n_icm, half, NW;
     int const_z;                  // degree when uniform (lattices), 0 = per-site table
-    int wide;                     // 1: global-resident layout (instances too large for shared memory)
+    int wide;                     // kLayoutShared, kLayoutWide or kLayoutBig
     int diluted;                  // 1: some instance has absent bonds (J = 0): per-instance tables below
     int scratch_words;            // wide layout: uint32 words of scratch per CTA (cluster words, masks)
     uint32_t *scratch;            // wide layout: [grid][scratch_words]
@@ -266,7 +269,7 @@ int fused_threads_wide(int N);
 int wide_scratch_words(int N);
 
 // Host-callable launchers (pt_icm.cu).  Return a cudaError_t.
-cudaError_t fused_occupancy(bool gauss, int Z, bool wide, int threads, int smem, int *ctas_per_sm);
+cudaError_t fused_occupancy(bool gauss, int Z, int layout, int threads, int smem, int *ctas_per_sm);
 cudaError_t launch_fused(const KParams &P, bool gauss, int threads, int grid, uint32_t n_sweeps,
                          cudaStream_t st);
 // Spins int8 [n_inst][R][N] by site <-> packed words [n_inst][G][N] by position

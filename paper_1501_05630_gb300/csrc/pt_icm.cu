@@ -53,8 +53,8 @@ cudaError_t launch_team_pmj(const TeamParams &TP, int Z, int grid, int smem, uin
 cudaError_t launch_team_gauss(const TeamParams &TP, int Z, int grid, int smem, uint32_t n_sweeps, cudaStream_t st);
 cudaError_t team_occupancy_pmj(int Z, int smem, int *ctas);
 cudaError_t team_occupancy_gauss(int Z, int smem, int *ctas);
-cudaError_t fused_occupancy_pmj(int Z, bool wide, int threads, int smem, int *ctas);
-cudaError_t fused_occupancy_gauss(int Z, bool wide, int threads, int smem, int *ctas);
+cudaError_t fused_occupancy_pmj(int Z, int layout, int threads, int smem, int *ctas);
+cudaError_t fused_occupancy_gauss(int Z, int layout, int threads, int smem, int *ctas);
 int debug_phase_cycles_pmj(unsigned long long *out, int reset);
 int debug_phase_cycles_gauss(unsigned long long *out, int reset);
 int debug_check_pmj(unsigned int *out, int reset);
@@ -1217,6 +1217,14 @@ __global__ void __launch_bounds__(kMaxThreadsWide, 1) fused_wide_kernel(const KP
     fused_body<GAUSS, Z, true, DIL>(P, n_sweeps);
 }
 
+// A wide CTA with its instance in shared memory: the words that the wide layout
+// reads through L1 and writes through to L2 stay on the SM.  BIGFIG
+template <bool GAUSS, int Z, bool DIL>
+__global__ void __launch_bounds__(kMaxThreadsWide, 1) fused_big_kernel(const KParams P, uint32_t n_sweeps)
+{
+    fused_body<GAUSS, Z, false, DIL>(P, n_sweeps);
+}
+
 // The shared group kernel (see TeamParams): each persistent CTA takes the
 // next work item (a global counter) whenever it is free, so the tiles, in
 // descending order of work, balance over the CTAs; a tile's teams run their
@@ -1511,10 +1519,11 @@ inline int grid_for(size_t n, int threads)
 template <bool GAUSS, int Z, bool DIL>
 cudaError_t launch_fused_t(const KParams &P, int threads, int grid, uint32_t n_sweeps, cudaStream_t st)
 {
-    if (P.wide && (threads > kMaxThreadsWide || !P.scratch)) return cudaErrorInvalidValue;
-    if (!P.wide && threads > kMaxThreads) return cudaErrorInvalidValue;
+    if (threads > (P.wide == kLayoutShared ? kMaxThreads : kMaxThreadsWide)) return cudaErrorInvalidValue;
+    if (P.wide == kLayoutWide && !P.scratch) return cudaErrorInvalidValue;
     if (DIL && (!P.nbr_inst || !P.zdeg_inst || !P.nb_inst)) return cudaErrorInvalidValue;
-    auto kern = P.wide ? fused_wide_kernel<GAUSS, Z, DIL> : fused_kernel<GAUSS, Z, DIL>;
+    auto kern = P.wide == kLayoutWide ? fused_wide_kernel<GAUSS, Z, DIL>
+                : P.wide == kLayoutBig ? fused_big_kernel<GAUSS, Z, DIL> : fused_kernel<GAUSS, Z, DIL>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, P.sm.total);
     if (e != cudaSuccess) return e;
     kern<<<grid, threads, P.sm.total, st>>>(P, n_sweeps);
@@ -1522,10 +1531,11 @@ cudaError_t launch_fused_t(const KParams &P, int threads, int grid, uint32_t n_s
 }
 
 template <bool GAUSS, int Z>
-cudaError_t occupancy_t(bool wide, int threads, int smem, int *ctas)
+cudaError_t occupancy_t(int layout, int threads, int smem, int *ctas)
 {
     // the diluted variants have the same register budget (launch bounds) and layout
-    auto kern = wide ? fused_wide_kernel<GAUSS, Z, false> : fused_kernel<GAUSS, Z, false>;
+    auto kern = layout == kLayoutWide ? fused_wide_kernel<GAUSS, Z, false>
+                : layout == kLayoutBig ? fused_big_kernel<GAUSS, Z, false> : fused_kernel<GAUSS, Z, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, kern, threads, smem);
@@ -1603,9 +1613,9 @@ int wide_scratch_words(int N)
     return (2 * N + 32 * NW + 3) / 4 * 4;   // N cluster words, 32 rows of mask_stride(NW) <= N + 32 NW words in all
 }
 
-cudaError_t fused_occupancy(bool gauss, int Z, bool wide, int threads, int smem, int *ctas)
+cudaError_t fused_occupancy(bool gauss, int Z, int layout, int threads, int smem, int *ctas)
 {
-    return gauss ? fused_occupancy_gauss(Z, wide, threads, smem, ctas) : fused_occupancy_pmj(Z, wide, threads, smem, ctas);
+    return gauss ? fused_occupancy_gauss(Z, layout, threads, smem, ctas) : fused_occupancy_pmj(Z, layout, threads, smem, ctas);
 }
 
 cudaError_t launch_fused(const KParams &P, bool gauss, int threads, int grid, uint32_t n_sweeps, cudaStream_t st)
@@ -1748,12 +1758,12 @@ cudaError_t team_occupancy_part(int Z, int smem, int *ctas)
     }
 }
 
-cudaError_t occupancy_part(int Z, bool wide, int threads, int smem, int *ctas)
+cudaError_t occupancy_part(int Z, int layout, int threads, int smem, int *ctas)
 {
     switch (Z) {
-    case 4: return occupancy_t<kPartGauss, 4>(wide, threads, smem, ctas);
-    case 6: return occupancy_t<kPartGauss, 6>(wide, threads, smem, ctas);
-    case 8: return occupancy_t<kPartGauss, 8>(wide, threads, smem, ctas);
+    case 4: return occupancy_t<kPartGauss, 4>(layout, threads, smem, ctas);
+    case 6: return occupancy_t<kPartGauss, 6>(layout, threads, smem, ctas);
+    case 8: return occupancy_t<kPartGauss, 8>(layout, threads, smem, ctas);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -1796,9 +1806,9 @@ cudaError_t launch_fused_pmj(const KParams &P, int threads, int grid, uint32_t n
 {
     return launch_part(P, threads, grid, n_sweeps, st);
 }
-cudaError_t fused_occupancy_pmj(int Z, bool wide, int threads, int smem, int *ctas)
+cudaError_t fused_occupancy_pmj(int Z, int layout, int threads, int smem, int *ctas)
 {
-    return occupancy_part(Z, wide, threads, smem, ctas);
+    return occupancy_part(Z, layout, threads, smem, ctas);
 }
 cudaError_t launch_team_pmj(const TeamParams &TP, int Z, int grid, int smem, uint32_t n_sweeps, cudaStream_t st)
 {
@@ -1812,9 +1822,9 @@ cudaError_t launch_fused_gauss(const KParams &P, int threads, int grid, uint32_t
 {
     return launch_part(P, threads, grid, n_sweeps, st);
 }
-cudaError_t fused_occupancy_gauss(int Z, bool wide, int threads, int smem, int *ctas)
+cudaError_t fused_occupancy_gauss(int Z, int layout, int threads, int smem, int *ctas)
 {
-    return occupancy_part(Z, wide, threads, smem, ctas);
+    return occupancy_part(Z, layout, threads, smem, ctas);
 }
 cudaError_t launch_team_gauss(const TeamParams &TP, int Z, int grid, int smem, uint32_t n_sweeps, cudaStream_t st)
 {
