@@ -338,6 +338,7 @@ struct icm_batch {
     long long *d_tmeas = nullptr;     // [n_inst]
     std::vector<uint8_t> h_active;
     std::vector<long long> h_tmeas;
+    bool large = false;               // too large for several instances of 128 threads on an SM
     int groups = 0;                   // live groups whose graphs launch this batch's kernels
 };
 
@@ -435,6 +436,42 @@ bool on_device(const icm_ctx *ctx, const void *p, uint32_t flags)
         return false;
     }
     return a.type == cudaMemoryTypeDevice && a.device == ctx->device;
+}
+
+// CTA width of a +-J batch with few instances, whose launches are bound by the
+// latency of a sweep, not by throughput (+-J results do not depend on the width;
+// Gaussian sums do, so those keep theirs).  `threads`: the width for many
+// instances, at most 128 in shared memory.  About one site of a colour per
+// thread is best while an SM has one instance; two or three share its issue
+// slots.  Measured with 24 temperatures, us per sweep, by instances per SM:
+//   2D L=8 (32 sites of a colour), 32 / 128 threads: 15.5 / 9.6 (1), 15.4 / 11.3
+//     (3), 15.2 / 12.2 (4); 1000 instances (7) 12.7 / 15.5 with 16 temperatures
+//   chimera C_12 (576), 128 / 288 / 576: 65.2 / 35.4 / 30.9 (1), 72.0 / 50.5 /
+//     61.2 (2), 82.0 / 66.7 / 90.9 (3), 94.8 / 103.5 (4)
+//   2D L=32 (512), 128 / 256 / 512 / 1024: 40.7 / 27.0 / 22.7 / 24.1 (1), 45.7 /
+//     35.0 / 35.5 (2), 53.4 / 46.7 / 69.7 (3)
+// Instances of 65 to 287 sites of a colour keep 128 threads, the width that a
+// batch of such instances reports by default (chimera C_8, 128 / 256: 24.6 / 18.9
+// alone on an SM, 27.5 / 24.4 with two, 31.3 / 32.2 with three).
+int roomy_threads(const icm_ctx *ctx, int N, int Z, int R, int G, int n_T, int n_icm, int n_inst, int threads)
+{
+    const int per_sm = (n_inst + ctx->num_sms - 1) / ctx->num_sms;
+    const int half = N / 2, gthr = (half + 31) / 32 * 32, n8 = (R + 7) / 8;
+    int t = threads;
+    if (gthr <= 64) {                        // a warp group per 8 replicas
+        if (per_sm <= 4) t = gthr * std::min(n8, 128 / gthr);
+    } else if (gthr >= 288 && per_sm <= 3) { // whole sites: the fewest per thread at this many threads
+        const int most = per_sm == 1 ? icm::kMaxThreadsWide : 288, parts = (half + most - 1) / most;
+        t = ((half + parts - 1) / parts + 31) / 32 * 32;
+    }
+    if (t <= threads) return threads;
+    const int layout = t > icm::kMaxThreads ? icm::kLayoutBig : icm::kLayoutShared;
+    const icm::SmemLayout sm = icm::smem_layout(N, Z, R, G, n_T, n_icm, t / 32, false, false);
+    int ctas = 0;
+    const bool fits = sm.total <= ctx->max_smem_optin &&
+                      icm::fused_occupancy(false, Z, layout, t, sm.total, &ctas) == cudaSuccess && ctas >= per_sm;
+    (void)cudaGetLastError();
+    return fits ? t : threads;
 }
 
 // One launch of n_sweeps simulation steps of the batch, in its layout.
@@ -552,6 +589,7 @@ void set_ctx_error(icm_ctx *ctx, const std::string &msg)
 }
 cudaStream_t ctx_stream(const icm_ctx *ctx) { return ctx->stream; }
 int ctx_device(const icm_ctx *ctx) { return ctx->device; }
+bool batch_large(const icm_batch *b) { return b->large; }
 // device memory of the context (its allocator and budget) for the other
 // translation units; the status is ICM_OK, ICM_ERR_BUDGET or ICM_ERR_OOM
 icm_status ctx_device_alloc(icm_ctx *ctx, void **p, size_t bytes) { return ctx_alloc(ctx, p, bytes); }
@@ -833,7 +871,7 @@ icm_status icm_batch_create(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t di
     int n_icm = 0;
     while (n_icm < n_T && T[n_icm] <= T_icm) ++n_icm;
     int threads = icm::fused_threads(N);
-    if (n_inst < ctx->num_sms) {
+    if (b->gauss && n_inst < ctx->num_sms) {
         // few instances: each CTA alone on its SM is latency-bound, so a tiny
         // instance gets a warp group per 16-bit pass (the passes run at once)
         const int gthr = (N / 2 + 31) / 32 * 32, npass = (R + 15) / 16;
@@ -849,7 +887,9 @@ icm_status icm_batch_create(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t di
             wide = true;
         (void)cudaGetLastError();
         if (wide) threads = icm::fused_threads_wide(N);
+        b->large = wide;
     }
+    if (!b->gauss) threads = roomy_threads(ctx, N, Z, R, G, n_T, n_icm, n_inst, threads);
     b->n_icm = n_icm;
     const int half = N / 2;
 

@@ -20,6 +20,10 @@
 
 #include <cuda_runtime.h>
 
+namespace icm {
+bool batch_large(const icm_batch *b);   // icm_api.cpp
+}  // namespace icm
+
 namespace {
 
 struct Request {
@@ -177,7 +181,7 @@ icm_status create_class(icm_server *s, const Request &r, ShapeClass **out)
         int32_t th = 0, cps = 0, grid = 0, smem = 0;
         int64_t launches = 0;
         st = icm_batch_info(c->batch, &th, &cps, &grid, &smem, &launches);
-        if (st == ICM_OK && th > 128 && icm_batch_set_cluster(c->batch, 8, c->N >= 8192 ? 512 : 256) != ICM_OK &&
+        if (st == ICM_OK && icm::batch_large(c->batch) && icm_batch_set_cluster(c->batch, 8, c->N >= 8192 ? 512 : 256) != ICM_OK &&
             icm_batch_set_cluster(c->batch, 4, 512) != ICM_OK)
             st = icm_batch_set_cluster(c->batch, 0, th);          // keep the one-CTA layout
     }
