@@ -764,8 +764,8 @@ __device__ __forceinline__ void cl_grow_uf(const KParams &P, const ClusterLayout
 // a pair into the CTA that takes the pair (k mod K), whose warp counts,
 // reverses, seeds and grows it on its own and stores the cluster's rows back
 // into the CTAs that hold them or their halo copies.  Two cluster barriers,
-// where the scans took one each round of six.  2D L=128 x 20 on 8 x 1024:
-// CLROWFIG.
+// where the scans took one each round of six.  2D L=128 x 20 on 8 x 1024, 16
+// sweeps: 4.72 to 1.82 ms; on 8 x 512 189 to 90 us per sweep.
 template <int KIND>
 __device__ __forceinline__ void cl_rows_pairs(const KParams &P, const ClusterLayout &L, const CS &S, int slot, bool trace)
 {

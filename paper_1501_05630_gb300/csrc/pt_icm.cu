@@ -348,6 +348,68 @@ __device__ __forceinline__ void pmj_pass(const KParams &P, const uint32_t (&key)
     }
 }
 
+// Step 1 of Gaussian instances with one temperature (two replicas: simulated
+// annealing): one Philox block and two updates per site, where a pass of 16
+// draws and updates eight.  The energies are the sums of gauss_pass, in its
+// order (the transpose reduction adds lanes 16, 8, 4, 2, 1 apart).
+template <int Z, bool WIDE, bool DIL>
+__device__ __forceinline__ void gauss_pair_sweep(const KParams &P, const uint32_t (&key)[20], const Sm &S, const Team &T,
+                                                 uint32_t t, uint32_t inst)
+{
+    const int half = P.half;
+    const float bl = S.b2l[0];
+    float acc[2];
+#pragma unroll 1
+    for (int color = 0; color < 2; ++color) {
+        acc[0] = acc[1] = 0.f;
+#pragma unroll 1
+        for (int j = T.tid; j < half; j += T.nth) {
+            const int p = color * half + j;
+            const uint32_t sw = S.s[p];
+            uint32_t x[4];
+            philox10k(__ldg(P.pos2site + p), t, 0u, inst, key, x);
+            uint32_t nw[Z], flip = 0u;
+            float J[Z], Jsum = 0.f;
+            int q[Z];
+            load_nbrs<Z>(S.nbr, p, q);
+#pragma unroll
+            for (int d = 0; d < Z; ++d) {
+                nw[d] = S.s[ICM_IDX(q[d], P.N, 1)];
+                J[d] = S.Jd[ICM_IDX(p * Z + d, P.N * Z, 2)];
+                Jsum += J[d];
+            }
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                float h = Jsum;
+#pragma unroll
+                for (int d = 0; d < Z; ++d)
+                    if ((nw[d] >> b) & 1u) h = fmaf(J[d], -2.f, h);
+                const float sh = neg_if(h, sw & (1u << b));
+                const float lim = ex2_approx(fmaf(bl, sh, 32.f));
+                bool a;
+                if constexpr (DIL)
+                    a = (sh < 0.f) || (sh == 0.f ? (!S.tie || x[b] < 0x80000000u) : (__uint2float_rz(x[b]) < lim));
+                else
+                    a = __uint2float_rz(x[b]) < lim;
+                acc[b] -= sh;
+                if (a) {
+                    flip |= 1u << b;
+                    acc[b] += 2.f * sh;
+                }
+            }
+            S.s[p] = sw ^ flip;
+        }
+        team_sync(T);
+    }
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) acc[b] += __shfl_xor_sync(kFull, acc[b], o);
+    }
+    if ((threadIdx.x & 31) < 2) ((float *)S.Epart)[(T.tid >> 5) * 2 + (threadIdx.x & 31)] = (threadIdx.x & 1) ? acc[1] : acc[0];
+    team_sync(T);
+}
+
 // Tiny Gaussian instances with at least twice the threads a colour needs: the
 // threads split into groups of whole warps that run different passes at the
 // same time; every warp writes its energy slots, the ones of passes it did not
@@ -377,12 +439,14 @@ __device__ __forceinline__ void gauss_sweep_concurrent(const KParams &P, const u
 // instruction cache is shared by all CTAs of the SM).  A +-J team with at least
 // twice the threads a colour needs splits into groups of whole warps that
 // take the replicas in shares of 8 at the same time.
-template <bool GAUSS, int Z, bool WIDE, bool DIL>
+template <bool GAUSS, int Z, bool WIDE, bool DIL, bool PAIR>
 __device__ __forceinline__ void metropolis_sweep(const KParams &P, const uint32_t (&key)[20], const Sm &S, const Team &T,
                                                  uint32_t t, uint32_t inst)
 {
     const int gthr = (P.half + 31) & ~31;        // threads of one pass
-    if constexpr (GAUSS) {
+    if constexpr (PAIR) {
+        gauss_pair_sweep<Z, WIDE, DIL>(P, key, S, T, t, inst);
+    } else if constexpr (GAUSS) {
         const int npass = (P.R + 15) >> 4;          // 16-bit passes per colour
         const int conc = min(T.nth / gthr, npass);   // passes at a time
         if (conc >= 2) {
@@ -1053,7 +1117,7 @@ __device__ __forceinline__ void load_tables(const KParams &P, Sm &S, const Team 
 // n_sweeps simulation steps of the instance in slot `slot`, run by team T:
 // load its state into the team's shared memory (the spins and couplings stay
 // in global memory in the wide layout), run the steps, store the state back.
-template <bool GAUSS, int Z, bool WIDE, bool DIL>
+template <bool GAUSS, int Z, bool WIDE, bool DIL, bool PAIR = false>
 __device__ __forceinline__ void run_instance(const KParams &P, const uint32_t (&key)[20], Sm &S, const Team &T,
                                              int slot, uint32_t n_sweeps)
 {
@@ -1128,9 +1192,9 @@ __device__ __forceinline__ void run_instance(const KParams &P, const uint32_t (&
             team_sync(T);
         }
         const bool icm = P.icm_every > 0 && t % (uint32_t)P.icm_every == 0 && P.n_icm > 0;
-        const bool pt = P.swap_every > 0 && t % (uint32_t)P.swap_every == 0 && nT > 1;
+        const bool pt = !PAIR && P.swap_every > 0 && t % (uint32_t)P.swap_every == 0 && nT > 1;
         if (P.enable_metropolis) {  // step 1
-            metropolis_sweep<GAUSS, Z, WIDE, DIL>(P, key, S, T, t, inst);
+            metropolis_sweep<GAUSS, Z, WIDE, DIL, PAIR>(P, key, S, T, t, inst);
             for (int r = tid; r < R; r += nth) {
                 ET e = ET(0);
                 for (int w = 0; w < nwarps; ++w) e += ((const ET *)S.Epart)[w * R + r];
@@ -1186,7 +1250,7 @@ __device__ __forceinline__ void run_instance(const KParams &P, const uint32_t (&
 // like padding) and a diluted instance takes the probability-1/2 rule for
 // zero-energy proposals.  One CTA runs the instances blockIdx.x,
 // blockIdx.x + gridDim.x, ... in turn.
-template <bool GAUSS, int Z, bool WIDE, bool DIL>
+template <bool GAUSS, int Z, bool WIDE, bool DIL, bool PAIR = false>
 __device__ __forceinline__ void fused_body(const KParams &P, uint32_t n_sweeps)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1201,7 +1265,7 @@ __device__ __forceinline__ void fused_body(const KParams &P, uint32_t n_sweeps)
     load_tables<GAUSS, Z, WIDE, DIL>(P, S, T);
     for (int slot = blockIdx.x; slot < P.n_inst; slot += gridDim.x) {
         if (P.active && !P.active[slot]) continue;   // free slot of a serving batch
-        run_instance<GAUSS, Z, WIDE, DIL>(P, P.key, S, T, slot, n_sweeps);
+        run_instance<GAUSS, Z, WIDE, DIL, PAIR>(P, P.key, S, T, slot, n_sweeps);
     }
 }
 
@@ -1211,6 +1275,15 @@ __global__ void __launch_bounds__(kMaxThreads, 7) fused_kernel(const KParams P, 
     fused_body<GAUSS, Z, false, DIL>(P, n_sweeps);
 }
 
+// Gaussian batches with one temperature (see gauss_pair_sweep), as a kernel of
+// their own: the branch in fused_kernel slowed 3D L=8 x 1000 by 0.9%.  16
+// annealing steps of 32 sweeps of 512 3D L=6 instances: 4.64 to 3.49 ms.
+template <int Z, bool DIL>
+__global__ void __launch_bounds__(kMaxThreads, 7) fused_pair_kernel(const KParams P, uint32_t n_sweeps)
+{
+    fused_body<true, Z, false, DIL, true>(P, n_sweeps);
+}
+
 template <bool GAUSS, int Z, bool DIL>
 __global__ void __launch_bounds__(kMaxThreadsWide, 1) fused_wide_kernel(const KParams P, uint32_t n_sweeps)
 {
@@ -1218,7 +1291,8 @@ __global__ void __launch_bounds__(kMaxThreadsWide, 1) fused_wide_kernel(const KP
 }
 
 // A wide CTA with its instance in shared memory: the words that the wide layout
-// reads through L1 and writes through to L2 stay on the SM.  BIGFIG
+// reads through L1 and writes through to L2 stay on the SM.  2D L=64 x 40, 16
+// sweeps: 0.89 to 0.85 ms; 3D Gaussian L=12 x 6: 42.6 to 29.7 us per sweep.
 template <bool GAUSS, int Z, bool DIL>
 __global__ void __launch_bounds__(kMaxThreadsWide, 1) fused_big_kernel(const KParams P, uint32_t n_sweeps)
 {
@@ -1524,6 +1598,8 @@ cudaError_t launch_fused_t(const KParams &P, int threads, int grid, uint32_t n_s
     if (DIL && (!P.nbr_inst || !P.zdeg_inst || !P.nb_inst)) return cudaErrorInvalidValue;
     auto kern = P.wide == kLayoutWide ? fused_wide_kernel<GAUSS, Z, DIL>
                 : P.wide == kLayoutBig ? fused_big_kernel<GAUSS, Z, DIL> : fused_kernel<GAUSS, Z, DIL>;
+    if constexpr (GAUSS)
+        if (P.wide == kLayoutShared && P.R == 2) kern = fused_pair_kernel<Z, DIL>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, P.sm.total);
     if (e != cudaSuccess) return e;
     kern<<<grid, threads, P.sm.total, st>>>(P, n_sweeps);
