@@ -132,6 +132,29 @@ bool build_geometry(int lattice, int L, Geometry &g)
     return true;
 }
 
+// The sites' incident bonds in bond order, by position: neighbour positions and
+// bond indices [N][Z], padded with (the site itself, -1), and degrees [N].
+// False when a site has more than Z bonds.  (A list per site took most of the
+// 1.2 ms that icm_percolation spent on the host for chimera C_32.)
+bool incident_tables(const Geometry &g, const std::vector<int> &pos, std::vector<uint16_t> &nbr,
+                     std::vector<int32_t> &edge_bond, std::vector<uint8_t> &deg)
+{
+    const size_t Z = (size_t)g.Z;
+    nbr.resize(g.N * Z);
+    edge_bond.assign(g.N * Z, -1);
+    deg.assign(g.N, 0);
+    for (int p = 0; p < g.N; ++p) std::fill_n(nbr.begin() + p * Z, Z, (uint16_t)p);
+    for (int e = 0; e < g.Nb; ++e) {
+        const int p = pos[g.bi[e]], q = pos[g.bj[e]];
+        if (deg[p] >= Z || deg[q] >= Z) return false;
+        nbr[p * Z + deg[p]] = (uint16_t)q;
+        edge_bond[p * Z + deg[p]++] = e;
+        nbr[q * Z + deg[q]] = (uint16_t)p;
+        edge_bond[q * Z + deg[q]++] = e;
+    }
+    return true;
+}
+
 // Philox4x32-10 on the host (Salmon, Moraes, Dror, Shaw, SC'11: multipliers
 // 0xD2511F53 / 0xCD9E8D57, Weyl key increments 0x9E3779B9 / 0xBB67AE85), for
 // disorder drawn from the seed when a caller passes no couplings.
@@ -253,35 +276,9 @@ void temperature_tables(const double *T, int n_T, int Nb, int Z, TempTables &t)
     if (t.thr_swap.empty()) t.thr_swap.push_back(0u);
 }
 
-// Byte offsets of a ladder's tables in one block: beta (double), then 4-byte
-// entries, so nothing is padded.
-struct TempBlock {
-    size_t beta, thr_metro, b2l, dbl, off, len, bytes;
-    TempBlock(int n_T, int Z)
-    {
-        const size_t R = 2 * (size_t)n_T, np = (size_t)n_T - 1;
-        beta = 0;
-        thr_metro = beta + 8 * (size_t)n_T;
-        b2l = thr_metro + 4 * R * icm::thr_stride(Z);
-        dbl = b2l + 4 * R;
-        off = dbl + 4 * np;
-        len = off + 4 * np;
-        bytes = len + 4 * np;
-    }
+struct DevBuf {
+    void *p = nullptr;
 };
-
-void fill_temp_block(const TempTables &t, const TempBlock &L, unsigned char *p)
-{
-    auto put = [p](size_t at, const auto &v) {
-        if (!v.empty()) std::memcpy(p + at, v.data(), v.size() * sizeof(v[0]));
-    };
-    put(L.beta, t.beta);
-    put(L.thr_metro, t.thr_metro);
-    put(L.b2l, t.b2l);
-    put(L.dbl, t.dbeta_l2e);
-    put(L.off, t.swap_off);
-    put(L.len, t.swap_len);
-}
 
 }  // namespace
 
@@ -297,14 +294,6 @@ struct icm_batch {
     icm::KParams kp{};
     int threads = 0, grid = 0, ctas_per_sm = 0, n_icm = 0;
     size_t thr_swap_cap = 0;      // entries allocated for the +-J swap thresholds
-    // the ladder's tables, one block on the device (TempBlock), and the pinned
-    // slots that new ladders go through without waiting for the device
-    void *d_temp = nullptr;
-    static constexpr int kTempSlots = 4;
-    unsigned char *h_temp = nullptr;              // [kTempSlots][temp_slot]
-    size_t temp_slot = 0;
-    cudaEvent_t temp_done[kTempSlots] = {};       // the copy out of a slot has run
-    int temp_next = 0;
     int64_t launches = 0;
     std::vector<std::pair<void *, size_t>> allocs;   // device blocks and their sizes
     std::vector<uint16_t> h_pos2site;  // [N] site of each colour-major position
@@ -573,9 +562,6 @@ void destroy_batch(icm_batch *b)
         b->ctx->batches.erase(b);
     }
     for (auto &a : b->allocs) ctx_free(b->ctx, a.first, a.second);
-    for (cudaEvent_t e : b->temp_done)
-        if (e) cudaEventDestroy(e);
-    if (b->h_temp) cudaFreeHost(b->h_temp);
     delete b;
 }
 
@@ -620,22 +606,8 @@ bool host_tables(int lattice, int L, HostTables &t)
         pos[i] = next[g.color[i]]++;
         t.pos2site[pos[i]] = (uint16_t)i;
     }
-    std::vector<std::vector<std::pair<int, int>>> inc(N);
-    for (int e = 0; e < g.Nb; ++e) {
-        inc[g.bi[e]].push_back({g.bj[e], e});
-        inc[g.bj[e]].push_back({g.bi[e], e});
-    }
-    t.nbr.assign((size_t)N * Z, 0);
-    t.edge_bond.assign((size_t)N * Z, -1);
-    for (int i = 0; i < N; ++i) {
-        const int deg = (int)inc[i].size(), p = pos[i];
-        if (deg > Z) return false;
-        for (int d = 0; d < Z; ++d) {
-            t.nbr[(size_t)p * Z + d] = (uint16_t)(d < deg ? pos[inc[i][d].first] : p);
-            t.edge_bond[(size_t)p * Z + d] = d < deg ? inc[i][d].second : -1;
-        }
-    }
-    return true;
+    std::vector<uint8_t> deg;
+    return incident_tables(g, pos, t.nbr, t.edge_bond, deg);
 }
 
 // See ClusterTables.  A CTA's halo entries are numbered in ascending position;
@@ -830,38 +802,22 @@ icm_status icm_batch_create(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t di
         pos[i] = next[g.color[i]]++;
         pos2site[pos[i]] = (uint16_t)i;
     }
-    // incident bonds of every site in bond order, padded to Z with (self, -1)
-    std::vector<std::vector<std::pair<int, int>>> inc(N);
-    for (int e = 0; e < g.Nb; ++e) {
+    for (int e = 0; e < g.Nb; ++e)
         if (g.color[g.bi[e]] == g.color[g.bj[e]]) {
             destroy_batch(b);
             return fail(ctx, ICM_ERR_ARG, "bond inside a colour class");
         }
-        inc[g.bi[e]].push_back({g.bj[e], e});
-        inc[g.bj[e]].push_back({g.bi[e], e});
+    std::vector<uint16_t> nbr;
+    std::vector<int32_t> edge_bond;
+    std::vector<uint8_t> zdeg;
+    bool uniform = true, degrees = incident_tables(g, pos, nbr, edge_bond, zdeg);
+    for (int p = 0; p < N && degrees; ++p) {
+        degrees = zdeg[p] >= 4;
+        if (zdeg[p] != Z) uniform = false;
     }
-    std::vector<uint16_t> nbr((size_t)N * Z);
-    std::vector<int32_t> edge_bond((size_t)N * Z);
-    std::vector<uint8_t> zdeg(N);
-    bool uniform = true;
-    for (int i = 0; i < N; ++i) {
-        const int deg = (int)inc[i].size();
-        if (deg < 4 || deg > Z) {
-            destroy_batch(b);
-            return fail(ctx, ICM_ERR_UNSUPPORTED, "site degree outside 4..8");
-        }
-        if (deg != Z) uniform = false;
-        const int p = pos[i];
-        zdeg[p] = (uint8_t)deg;
-        for (int d = 0; d < Z; ++d) {
-            if (d < deg) {
-                nbr[(size_t)p * Z + d] = (uint16_t)pos[inc[i][d].first];
-                edge_bond[(size_t)p * Z + d] = inc[i][d].second;
-            } else {
-                nbr[(size_t)p * Z + d] = (uint16_t)p;
-                edge_bond[(size_t)p * Z + d] = -1;
-            }
-        }
+    if (!degrees) {
+        destroy_batch(b);
+        return fail(ctx, ICM_ERR_UNSUPPORTED, "site degree outside 4..8");
     }
     // launch shape: the shared-memory layout when several instances fit one
     // SM; the global-resident layout with wider CTAs when the instance does not
@@ -900,10 +856,11 @@ icm_status icm_batch_create(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t di
         destroy_batch(b);
         return fail(ctx, ICM_ERR_STATE, "swap thresholds not monotone in the energy difference");
     }
+    std::vector<double> &beta = tt.beta;
+    std::vector<uint32_t> &thr_metro = tt.thr_metro;
+    std::vector<float> &b2l = tt.b2l, &dbeta_l2e = tt.dbeta_l2e;
     std::vector<uint32_t> &thr_swap = tt.thr_swap;
-    const TempBlock TB(n_T, Z);
-    std::vector<unsigned char> temp(TB.bytes);
-    fill_temp_block(tt, TB, temp.data());
+    std::vector<int32_t> &swap_off = tt.swap_off, &swap_len = tt.swap_len;
     b->thr_swap_cap = thr_swap.size();
 
     icm::KParams &P = b->kp;
@@ -930,11 +887,11 @@ icm_status icm_batch_create(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t di
     icm_status st = ICM_OK;
     uint16_t *d_nbr, *d_pos2site;
     uint8_t *d_zdeg, *d_Jb;
-    float *d_Jd, *d_Ef, *d_treb, *d_trea;
-    int32_t *d_Ei, *d_trn, *d_trf, *d_trs, *d_trc;
-    uint32_t *d_spins, *d_t, *d_id, *d_thrs;
-    double *d_accE;
-    unsigned char *d_temp;
+    float *d_Jd, *d_Ef, *d_b2l, *d_treb, *d_trea;
+    int32_t *d_Ei, *d_off, *d_len, *d_trn, *d_trf, *d_trs, *d_trc;
+    uint32_t *d_spins, *d_t, *d_id, *d_thr, *d_thrs;
+    double *d_beta, *d_accE;
+    float *d_dbl;
     long long *d_acc64, *d_nmeas;
     unsigned long long *d_hist, *d_icmst;
     uint8_t *d_trsw;
@@ -948,11 +905,12 @@ icm_status icm_batch_create(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t di
         (st = dalloc(b, &d_Jd, b->gauss ? (size_t)n_inst * N * Z : 1)) ||
         (st = dalloc(b, &d_spins, (size_t)n_inst * G * N)) || (st = dalloc(b, &d_Ef, (size_t)n_inst * R)) ||
         (st = dalloc(b, &d_Ei, (size_t)n_inst * R)) || (st = dalloc(b, &d_t, n_inst)) ||
-        (st = dalloc(b, &d_id, n_inst)) || (st = dalloc(b, &d_temp, TB.bytes)) ||
-        (st = dalloc(b, &d_nbr_inst, (size_t)n_inst * N * Z)) ||
+        (st = dalloc(b, &d_id, n_inst)) || (st = dalloc(b, &d_thr, (size_t)R * icm::thr_stride(Z))) ||
+        (st = dalloc(b, &d_b2l, R)) || (st = dalloc(b, &d_nbr_inst, (size_t)n_inst * N * Z)) ||
         (st = dalloc(b, &d_zdeg_inst, (size_t)n_inst * N)) || (st = dalloc(b, &d_nb_inst, n_inst)) ||
         (st = dalloc(b, &b->d_bad, n_inst)) ||
-        (st = dalloc(b, &d_thrs, thr_swap.size())) || (st = dalloc(b, &d_accE, nk)) ||
+        (st = dalloc(b, &d_beta, n_T)) || (st = dalloc(b, &d_dbl, n_T - 1)) || (st = dalloc(b, &d_thrs, thr_swap.size())) ||
+        (st = dalloc(b, &d_off, n_T - 1)) || (st = dalloc(b, &d_len, n_T - 1)) || (st = dalloc(b, &d_accE, nk)) ||
         (st = dalloc(b, &d_acc64, 4 * nk)) || (st = dalloc(b, &d_hist, nk * (N + 1))) ||
         (st = dalloc(b, &d_nmeas, n_inst)) || (st = dalloc(b, &d_icmst, 2 * (size_t)n_inst)) || (st = dalloc(b, &d_trn, nk)) || (st = dalloc(b, &d_trf, nk)) ||
         (st = dalloc(b, &d_trs, nk)) || (st = dalloc(b, &d_trc, nk)) || (st = dalloc(b, &d_treb, nk)) ||
@@ -963,14 +921,8 @@ icm_status icm_batch_create(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t di
         return st;
     }
     P.nbr = d_nbr; P.pos2site = d_pos2site; P.zdeg = d_zdeg; P.Jb = d_Jb; P.Jd = d_Jd; P.spins = d_spins;
-    P.Ef = d_Ef; P.Ei = d_Ei; P.tsweep = d_t; P.inst_id = d_id; P.thr_swap = d_thrs; P.accE = d_accE;
-    b->d_temp = d_temp;
-    P.beta = (const double *)(d_temp + TB.beta);
-    P.thr_metro = (const uint32_t *)(d_temp + TB.thr_metro);
-    P.b2l = (const float *)(d_temp + TB.b2l);
-    P.dbeta_l2e = (const float *)(d_temp + TB.dbl);
-    P.swap_off = (const int32_t *)(d_temp + TB.off);
-    P.swap_len = (const int32_t *)(d_temp + TB.len);
+    P.Ef = d_Ef; P.Ei = d_Ei; P.tsweep = d_t; P.inst_id = d_id; P.thr_metro = d_thr; P.b2l = d_b2l;
+    P.beta = d_beta; P.dbeta_l2e = d_dbl; P.thr_swap = d_thrs; P.swap_off = d_off; P.swap_len = d_len; P.accE = d_accE;
     P.acc64 = d_acc64; P.hist = d_hist; P.n_meas = d_nmeas; P.icm_stats = d_icmst; P.tr_n_pre = d_trn; P.tr_flip2a = d_trf;
     P.tr_seed = d_trs; P.tr_csize = d_trc; P.tr_eb = d_treb; P.tr_ea = d_trea; P.tr_swap = d_trsw;
     P.nbr_inst = d_nbr_inst; P.zdeg_inst = d_zdeg_inst; P.nb_inst = d_nb_inst;
@@ -995,8 +947,13 @@ icm_status icm_batch_create(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t di
     if (e == cudaSuccess) e = UP(d_zdeg, zdeg);
     if (e == cudaSuccess) e = UP(b->edge_bond, edge_bond);
     if (e == cudaSuccess) e = UP(d_id, ids);
-    if (e == cudaSuccess) e = UP(d_temp, temp);
+    if (e == cudaSuccess) e = UP(d_thr, thr_metro);
+    if (e == cudaSuccess) e = UP(d_b2l, b2l);
+    if (e == cudaSuccess) e = UP(d_beta, beta);
+    if (e == cudaSuccess) e = UP(d_dbl, dbeta_l2e);
     if (e == cudaSuccess) e = UP(d_thrs, thr_swap);
+    if (e == cudaSuccess) e = UP(d_off, swap_off);
+    if (e == cudaSuccess) e = UP(d_len, swap_len);
 #undef UP
     if (e == cudaSuccess) e = cudaMemsetAsync(d_spins, 0, (size_t)n_inst * G * N * 4, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(d_t, 0, (size_t)n_inst * 4, s);
@@ -2049,47 +2006,21 @@ icm_status icm_set_temperatures(icm_batch *b, const double *T, int32_t n_T, doub
         P.thr_swap = d;
         b->thr_swap_cap = tt.thr_swap.size();
     }
-    // Through a pinned slot, in stream order, without waiting for the device: an
-    // annealing schedule sets a ladder before every launch (seven pageable copies
-    // and a wait each took 220 of the 300 us of a step of 512 3D L=6 instances).
     cudaStream_t s = b->ctx->stream;
-    const TempBlock TB(n_T, P.Z);
-    const size_t swap_bytes = tt.thr_swap.size() * 4;
-    constexpr size_t kSlotMost = 256 << 10;
-    if (TB.bytes + swap_bytes <= kSlotMost) {
-        if (b->temp_slot < TB.bytes + swap_bytes) {
-            ICM_CUDA(b->ctx, cudaStreamSynchronize(s));   // copies out of the old slots
-            if (b->h_temp) cudaFreeHost(b->h_temp);
-            b->h_temp = nullptr;
-            b->temp_slot = 0;
-            const size_t bytes = TB.bytes + b->thr_swap_cap * 4 <= kSlotMost ? TB.bytes + b->thr_swap_cap * 4
-                                                                            : TB.bytes + swap_bytes;
-            ICM_CUDA(b->ctx, cudaHostAlloc((void **)&b->h_temp, icm_batch::kTempSlots * bytes, cudaHostAllocDefault));
-            b->temp_slot = bytes;
-            for (cudaEvent_t &e : b->temp_done)
-                if (!e) ICM_CUDA(b->ctx, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        }
-        const int slot = b->temp_next;
-        ICM_CUDA(b->ctx, cudaEventSynchronize(b->temp_done[slot]));   // returns at once before its first use
-        unsigned char *h = b->h_temp + slot * b->temp_slot;
-        fill_temp_block(tt, TB, h);
-        std::memcpy(h + TB.bytes, tt.thr_swap.data(), swap_bytes);
-        ICM_CUDA(b->ctx, cudaMemcpyAsync(b->d_temp, h, TB.bytes, cudaMemcpyHostToDevice, s));
-        ICM_CUDA(b->ctx, cudaMemcpyAsync((void *)P.thr_swap, h + TB.bytes, swap_bytes, cudaMemcpyHostToDevice, s));
-        ICM_CUDA(b->ctx, cudaEventRecord(b->temp_done[slot], s));
-        b->temp_next = (slot + 1) % icm_batch::kTempSlots;
-    } else {
-        std::vector<unsigned char> temp(TB.bytes);
-        fill_temp_block(tt, TB, temp.data());
-        ICM_CUDA(b->ctx, cudaMemcpyAsync(b->d_temp, temp.data(), TB.bytes, cudaMemcpyHostToDevice, s));
-        ICM_CUDA(b->ctx, cudaMemcpyAsync((void *)P.thr_swap, tt.thr_swap.data(), swap_bytes, cudaMemcpyHostToDevice, s));
-        ICM_CUDA(b->ctx, cudaStreamSynchronize(s));   // the host tables are read by the copies
-    }
+#define UPV(dst, vec) cudaMemcpyAsync((void *)(dst), (vec).data(), (vec).size() * sizeof((vec)[0]), cudaMemcpyHostToDevice, s)
+    ICM_CUDA(b->ctx, UPV(P.thr_metro, tt.thr_metro));
+    ICM_CUDA(b->ctx, UPV(P.b2l, tt.b2l));
+    ICM_CUDA(b->ctx, UPV(P.beta, tt.beta));
+    ICM_CUDA(b->ctx, UPV(P.dbeta_l2e, tt.dbeta_l2e));
+    ICM_CUDA(b->ctx, UPV(P.thr_swap, tt.thr_swap));
+    ICM_CUDA(b->ctx, UPV(P.swap_off, tt.swap_off));
+    ICM_CUDA(b->ctx, UPV(P.swap_len, tt.swap_len));
+#undef UPV
+    ICM_CUDA(b->ctx, cudaStreamSynchronize(s));   // the host tables are read by the copies
     int n_icm = 0;
     while (n_icm < n_T && T[n_icm] <= T_icm) ++n_icm;
     b->T.assign(T, T + n_T);
     b->T_icm = T_icm;
-    if (n_icm == b->n_icm) return ICM_OK;
     b->n_icm = n_icm;
     P.n_icm = n_icm;
     // the shared-memory layout depends on n_icm; a clustered batch stays clustered

@@ -7,7 +7,8 @@
 // with atomicCAS, finds halve paths); then sites are counted per root.  Bound
 // by the latency of the finds; per site the masks take a bit, the parents and
 // counts together 4 bytes, so several CTAs share an SM.  20000 masks of chimera
-// C_32 at p = 0.387: 14.1 to 6.3 ms against all sites as nodes with 8 bytes.
+// C_32 at p = 0.387: 14.1 to 6.3 ms against all sites as nodes with 8 bytes
+// and 256 threads, 3.4 with 1024 and the tables of the lattice built in one pass.
 #include "icmpt.h"
 
 #include <string>
@@ -82,7 +83,7 @@ __host__ __device__ inline int percolation_smem(int N) { return 2 * N + N + N + 
 constexpr uint32_t kNone = 0xffffu, kAlone = 0xfffeu;   // links: empty site, occupied site without neighbours
 
 template <int Z>
-__global__ void __launch_bounds__(256) largest_cluster_kernel(const uint8_t *__restrict__ masks, int n_masks, int N,
+__global__ void __launch_bounds__(1024) largest_cluster_kernel(const uint8_t *__restrict__ masks, int n_masks, int N,
                                                               const uint16_t *__restrict__ nbr,
                                                               const uint16_t *__restrict__ pos2site, uint32_t thr,
                                                               uint32_t k0, uint32_t k1, int32_t *__restrict__ smax)
@@ -210,8 +211,13 @@ icm_status percolation(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t n_masks
     if (e == cudaSuccess) {
         auto kern = Z == 4 ? largest_cluster_kernel<4> : Z == 6 ? largest_cluster_kernel<6> : largest_cluster_kernel<8>;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // CTA width by size, so that the shared memory of the CTAs on an SM leaves
+        // it full of threads (us for 256 / 512 / 1024: chimera C_8 x 40000 546 /
+        // 589 / 884, 3D L=12 x 10000 693 / 661 / 642, C_16 x 20000 1268 / 1121 /
+        // 1022, C_32 x 8000 3291 / 2722 / 2553)
+        const int threads = N >= 2048 ? 1024 : N >= 1024 ? 512 : 256;
         if (e == cudaSuccess)
-            kern<<<grid, 256, smem, st>>>(mk, n_masks, N, d_nbr, d_p2s, thr, (uint32_t)seed, (uint32_t)(seed >> 32), out);
+            kern<<<grid, threads, smem, st>>>(mk, n_masks, N, d_nbr, d_p2s, thr, (uint32_t)seed, (uint32_t)(seed >> 32), out);
         if (e == cudaSuccess) e = cudaGetLastError();
     }
     if (e == cudaSuccess && !dev) e = cudaMemcpyAsync(smax, d_out, (size_t)n_masks * 4, cudaMemcpyDeviceToHost, st);
