@@ -142,7 +142,7 @@ def phase_fractions(b, stream, flush, S, n_inst, updates_per_step, ops_per_updat
 
 # the sources of the fused kernel (its launch shape and arithmetic); host-side
 # files (the API, the request server, other kernels) do not change its traffic
-FUSED_SOURCES = ("pt_icm.cu", "fused_pmj.cu", "fused_gauss.cu", "icm_device.cuh", "icm_internal.h")
+FUSED_SOURCES = ("pt_icm.cu", "fused_pmj.cu", "fused_gauss.cu", "row_growth.cuh", "icm_device.cuh", "icm_internal.h")
 
 
 def kernel_source_digest() -> str:

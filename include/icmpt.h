@@ -280,7 +280,9 @@ icm_status icm_clear_observables(icm_batch *b);
  *               n = 0 has no seed and no move);
  *   out[i][1] : growth scans, the passes over the sites that grew the
  *               clusters of all pairs (bit-parallel, all pairs of a sweep
- *               at once), summed over sweeps.
+ *               at once), summed over sweeps.  On undiluted 2D lattices up
+ *               to L = 128 each pair grows by itself on one warp, and a
+ *               sweep counts the passes of the pair that took the most.
  * They give the cluster-move rate and the work of the growth.  Not part of
  * checkpoints.  Host or device buffer (ICM_DEVICE_PTR); waits for the
  * batch's work.                                                           */
@@ -471,14 +473,14 @@ icm_status icm_percolation_random(icm_ctx *ctx, int32_t lattice, int32_t L, doub
 
 /* ---------------------------------------------------------------- launch shape
  * The threads per CTA of a batch's kernel, a multiple of 32 up to 1024; one
- * CTA runs one instance.  Up to 128 threads the instance lives in shared
- * memory; wider CTAs use the global-resident layout (the only one for
- * instances too large for shared memory).  Gaussian results depend on the
+ * CTA runs one instance.  The instance lives in shared memory where it fits;
+ * larger ones use the global-resident layout, which takes CTAs of more than
+ * 128 threads.  Gaussian results depend on the
  * width through the summation order of the fp32 energies; +-J results do
  * not.                                                                      */
 icm_status icm_batch_set_threads(icm_batch *b, int32_t threads);
 /* Time every valid launch shape on `sweeps` sweeps of this batch and keep
- * the fastest: CTA widths 32..128 (shared memory) when the instance fits,
+ * the fastest: CTA widths 32..128 when the instance fits in shared memory,
  * and for instances with more than 128 sites per colour also wide CTAs
  * (256, 512, 1024) and thread-block clusters (K = 4, 8 of 256 or 512
  * threads).  best_threads is the CTA width; icm_batch_cluster gives K.  The
@@ -542,8 +544,10 @@ icm_status icm_load(icm_batch *b, const void *buf, size_t len);
 
 /* Thread-block-cluster layout: each instance runs on a cluster of K CTAs
  * (K = 2, 4 or 8; K SMs), each holding 1/K of the sites of each colour in
- * its shared memory and reading its neighbours' words through the cluster's
- * distributed shared memory.  The arithmetic and random keys are those of
+ * its shared memory together with copies of the other CTAs' border sites,
+ * which their owners write through the cluster's distributed shared memory.
+ * The lattice's tables of those copies are device memory of the context (its
+ * budget).  The arithmetic and random keys are those of
  * the one-CTA layouts (the same chain, bit for bit for +-J); a single large
  * instance finishes its sweeps up to K times sooner.  Any lattice kind
  * (2D, 3D, chimera, 4D), diluted or not, with N/2 divisible into K blocks
@@ -560,7 +564,9 @@ icm_status icm_batch_cluster(const icm_batch *b, int32_t *K);
  * cluster's shared memory, a few pairs at a time (lock-free hooking of
  * roots by compare-and-swap, path halving); mode 0: label propagation, all
  * pairs at once, one bit per pair and site, in rounds of in-place scans
- * until nothing grows; mode -1 (default): the library's choice, label
+ * until nothing grows (undiluted 2D lattices up to L = 128: pair by pair, a
+ * warp of one CTA growing a pair's rows in its registers); mode -1
+ * (default): the library's choice, label
  * propagation (faster on every size measured: its word operations serve
  * all pairs at once, where union-find works pair by pair).  Both give the
  * same clusters, so the chain is the same bit for bit.

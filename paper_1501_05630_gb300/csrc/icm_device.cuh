@@ -268,23 +268,6 @@ __device__ __forceinline__ uint64_t swap_apply(const SwapMasks &m, uint64_t x)
            (((x & m.st[1]) + m.fw[1]) & m.en[1]);
 }
 
-// Sum of a[j] over the 32 lanes, delivered to lane j (31 shuffles).
-template <typename T>
-__device__ __forceinline__ T transpose_reduce(T (&a)[32], int lane)
-{
-#pragma unroll
-    for (int s = 16; s >= 1; s >>= 1) {
-        const bool upper = (lane & s) != 0;
-#pragma unroll
-        for (int j = 0; j < s; ++j) {
-            const T send = upper ? a[j] : a[j + s];
-            const T keep = upper ? a[j + s] : a[j];
-            a[j] = keep + __shfl_xor_sync(kFull, send, s);
-        }
-    }
-    return a[0];
-}
-
 // Sum of a[j] over the 32 lanes, delivered to lanes 2j and 2j+1 (16 shuffles).
 template <typename T>
 __device__ __forceinline__ T transpose_reduce16(T (&a)[16], int lane)
@@ -300,14 +283,6 @@ __device__ __forceinline__ T transpose_reduce16(T (&a)[16], int lane)
         }
     }
     return a[0] + __shfl_xor_sync(kFull, a[0], 1);
-}
-
-template <typename T>
-__device__ __forceinline__ T warp_sum_lane0(T v)
-{
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) v += __shfl_down_sync(kFull, v, o);
-    return v;
 }
 
 // Add one word to NPL bit-planes of per-bit counters (vertical counters).
@@ -398,36 +373,6 @@ __device__ __forceinline__ void vadd4(uint32_t (&pl)[NPL], uint32_t c0, uint32_t
     }
 }
 
-// Warp totals of vertical counters.  Every lane holds 32 counters as NPL
-// bit-planes (bit b of plane i = binary digit i of counter b).  Five
-// butterfly steps add the lanes' counters plane by plane (a ripple-carry
-// adder on whole words, one plane wider per step), so every lane ends with
-// the warp totals in NPL + 5 planes; lane b returns total b.
-template <int NPL>
-__device__ __forceinline__ int warp_vsum(const uint32_t (&pl)[NPL], int lane)
-{
-    uint32_t a[NPL + 5];
-#pragma unroll
-    for (int i = 0; i < NPL + 5; ++i) a[i] = i < NPL ? pl[i] : 0u;
-#pragma unroll
-    for (int st = 0; st < 5; ++st) {
-        uint32_t c = 0u;
-#pragma unroll
-        for (int i = 0; i < NPL + st; ++i) {
-            const uint32_t o = __shfl_xor_sync(kFull, a[i], 16 >> st);
-            const uint32_t x = a[i] ^ o;
-            const uint32_t cn = (a[i] & o) | (c & x);
-            a[i] = x ^ c;
-            c = cn;
-        }
-        a[NPL + st] = c;
-    }
-    int v = 0;
-#pragma unroll
-    for (int i = 0; i < NPL + 5; ++i) v |= (int)((a[i] >> lane) & 1u) << i;
-    return v;
-}
-
 // Per bit lane: u >= k, where u's binary digits are the bit-planes c3 c2 c1 c0
 // and k (0..15) is the same for all lanes.
 __device__ __forceinline__ uint32_t ge_bitsliced(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, int k)
@@ -443,10 +388,12 @@ __device__ __forceinline__ uint32_t ge_bitsliced(uint32_t c0, uint32_t c1, uint3
     return gt | eq;
 }
 
-// Warp totals of vertical counters: as warp_vsum, plane by plane.  The 32 x 32
-// bit transpose of a plane puts counter b's bits of all lanes into lane b,
-// whose popcount is the plane's total: 5 shuffles per plane where the
-// butterfly of warp_vsum takes 5 and two more for its carries.  Four planes at
+// Warp totals of vertical counters.  Every lane holds 32 counters as NPL
+// bit-planes (bit b of plane i = binary digit i of counter b); lane b returns
+// total b.  The 32 x 32 bit transpose of a plane puts counter b's bits of all
+// lanes into lane b, whose popcount is the plane's total: 5 shuffles per plane
+// where adding the lanes' counters plane by plane takes 5 and two more for its
+// carries.  Four planes at
 // a time, so that their chains of shuffles overlap (one at a time a single 3D
 // L=8 instance lost 8%), in one rolled body for any number of planes np <= NPL
 // (the planes above are zero).

@@ -9,8 +9,8 @@ namespace icm {
 
 constexpr int kMaxZ = 8;          // largest degree of the supported graphs (4D hypercubic)
 constexpr int kMaxR = 64;         // replicas per instance (2 N_T, N_T <= 32)
-constexpr int kMaxThreads = 128;  // threads per CTA of the fused kernel, shared-memory layout
-constexpr int kMaxThreadsWide = 1024;  // threads per CTA of the fused kernel, global-resident layout
+constexpr int kMaxThreads = 128;  // threads per CTA of the fused kernel, kLayoutShared
+constexpr int kMaxThreadsWide = 1024;  // threads per CTA of the fused kernel, kLayoutWide and kLayoutBig
 // One-CTA layouts: the instance in shared memory with CTAs up to kMaxThreads;
 // in global memory with wider CTAs; in shared memory with wider CTAs.
 constexpr int kLayoutShared = 0, kLayoutWide = 1, kLayoutBig = 2;

@@ -16,16 +16,20 @@
 //    checkerboard half-sweep walks contiguous words.
 //  * Step 1 (Metropolis, checkerboard): a thread updates all replica bits of
 //    one site word.  +-J: the number of unsatisfied bonds of all 32 replicas
-//    is counted bit-sliced, then each bit draws its Philox word and compares
-//    it with an integer threshold.  Gaussian: the local field of every bit is
-//    summed in fp32 from sign-injected couplings, accept via ex2.
+//    is counted bit-sliced, each bit's Philox word is compared with the few
+//    thresholds of its temperature, and the count's classes pick the result.
+//    Gaussian: the local field of every bit is summed in fp32 from
+//    sign-injected couplings, accept via ex2.
 //    The energies of all replicas fall out of the colour-1 half-sweep
 //    (every bond touches exactly one colour-1 site).
-//  * Steps 2a/2b: overlap masks of all ICM pairs by a warp bit transpose; one thread
-//    per pair counts, decides the copy-1 reversal and picks the seed by rank;
-//    the clusters of all pairs grow at once, bit-parallel (bit 2k of a site's
-//    cluster word = member of pair k's cluster), until a round adds nothing;
-//    both copies flip by XOR, E_a is recomputed and E_b = (E_a+E_b) - E_a.
+//  * Steps 2a/2b: overlap masks of all ICM pairs by a warp bit transpose.  On
+//    undiluted 2D lattices a pair's mask is rows of sites, which one warp
+//    counts, reverses, seeds and grows in registers (row_growth.cuh).
+//    Elsewhere one thread per pair decides the copy-1 reversal and picks the
+//    seed by rank, and the clusters of all pairs grow at once, bit-parallel
+//    (bit 2k of a site's cluster word = member of pair k's cluster), until a
+//    round adds nothing.  Both copies flip by XOR, E_a is recomputed and E_b =
+//    (E_a+E_b) - E_a.
 //  * Step 3: the draws of all swaps are turned into the form of their test in
 //    parallel; one warp runs both copies' sequential passes (a half-warp
 //    each) as chains of loads and compares; accepted swaps are then applied
