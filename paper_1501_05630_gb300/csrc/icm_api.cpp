@@ -819,11 +819,11 @@ icm_status icm_batch_create(icm_ctx *ctx, int32_t lattice, int32_t L, int32_t di
         destroy_batch(b);
         return fail(ctx, ICM_ERR_UNSUPPORTED, "site degree outside 4..8");
     }
-    // launch shape: the shared-memory layout when several instances fit one
-    // SM; the global-resident layout with wider CTAs when the instance does not
-    // fit one CTA's shared memory, or fits only one or two CTAs per SM and has
-    // more sites per colour than a shared-memory CTA has threads (there the
-    // L1-cached wide CTA keeps more warps busy per SM)
+    // launch shape: narrow CTAs when several instances fit one SM; wider ones
+    // when the instance does not fit one CTA's shared memory, or fits only one
+    // or two CTAs per SM and has more sites per colour than a narrow CTA has
+    // threads (there the wide CTA keeps more warps busy per SM).  Where the
+    // wide CTA keeps the instance is apply_threads' choice.
     int n_icm = 0;
     while (n_icm < n_T && T[n_icm] <= T_icm) ++n_icm;
     int threads = icm::fused_threads(N);
@@ -1385,9 +1385,9 @@ icm_status icm_batch_delta(icm_batch *b, int32_t k, double *delta_mean, double *
 
 // ---------------------------------------------------------------- launch shape, groups, autotuning
 
-// Widths up to 128 threads use the shared-memory layout; wider CTAs (up to
-// 1024 threads) use the global-resident layout, which is also the only one
-// for instances that do not fit one CTA's shared memory.
+// Widths up to 128 threads keep the instance in shared memory; wider CTAs (up
+// to 1024 threads) do where it fits as well, and else take the global-resident
+// layout, the only one for instances that do not fit one CTA's shared memory.
 static icm_status apply_threads(icm_batch *b, int threads)
 {
     icm::KParams &P = b->kp;
