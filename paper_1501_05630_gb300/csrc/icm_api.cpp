@@ -1447,13 +1447,12 @@ static icm_status apply_threads(icm_batch *b, int threads)
     return ICM_OK;
 }
 
-// The cluster layout's tables of the batch's lattice and K CTAs, on the device.
-static icm_status upload_cluster_tables(icm_batch *b, int K)
+// Put the cluster layout's tables t of the batch's lattice and K CTAs on the
+// device (unless they are there) and point the kernels' parameters at them.
+static icm_status upload_cluster_tables(icm_batch *b, int K, const icm::ClusterTables &t)
 {
     icm::KParams &P = b->kp;
     if (b->cl_tab_k != K) {
-        icm::ClusterTables t;
-        icm::cluster_tables(b->h_nbr.data(), P.N, P.Z, K, t);
         // 32-bit tables first, then the 16-bit ones
         std::vector<uint16_t> all;
         auto put = [&](const void *p, size_t bytes) {
@@ -1487,7 +1486,9 @@ static icm_status upload_cluster_tables(icm_batch *b, int K)
 }
 
 // One instance per thread-block cluster of K CTAs (K = 2, 4, 8) of `threads`
-// threads each; see cluster_icm.cu.  K = 0 returns to one CTA per instance.
+// threads each; see cluster_icm.cu.  K = 0 returns to one CTA per instance.  A
+// shape that is refused leaves the batch as it was: the device tables and the
+// kernels' parameters change after the last check.
 static icm_status apply_cluster(icm_batch *b, int K, int threads)
 {
     icm::KParams &P = b->kp;
@@ -1529,16 +1530,12 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
                 seen[li] = 1;
                 ord[(size_t)4 * t + j] = (uint16_t)li;
             }
-        if (!b->d_cl_order) {
-            icm_status st = dalloc(b, &b->d_cl_order, (size_t)P.N);
-            if (st) return st;
-        }
-        ICM_CUDA(b->ctx, cudaMemcpyAsync(b->d_cl_order, ord.data(), ord.size() * 2, cudaMemcpyHostToDevice,
-                                         b->ctx->stream));
-        ICM_CUDA(b->ctx, cudaStreamSynchronize(b->ctx->stream));   // the host table is read by the copy
     }
-    if (icm_status st = upload_cluster_tables(b, K)) return st;
-    const int nh = b->cl_nh, nx = b->cl_nx;
+    icm::ClusterTables tab;                  // of another K than the tables on the device
+    tab.nh = b->cl_nh;
+    tab.nx = b->cl_nx;
+    if (b->cl_tab_k != K) icm::cluster_tables(b->h_nbr.data(), P.N, P.Z, K, tab);
+    const int nh = tab.nh, nx = tab.nx;
     const int rows = ufg1 ? 0 : icm::cluster_row_kind(P.row_kind, b->L, K);
     icm::ClusterLayout L = icm::cluster_layout(P.N, P.Z, P.R, P.G, P.nT, K, threads / 32, b->gauss, ufg1, order, nh, nx,
                                                rows, b->L);
@@ -1568,6 +1565,14 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
         lean = 0;
     }
     L.lean = lean >= b->n_inst ? 1 : 0;
+    if (order && !b->d_cl_order)
+        if (icm_status st = dalloc(b, &b->d_cl_order, (size_t)P.N)) return st;
+    if (icm_status st = upload_cluster_tables(b, K, tab)) return st;
+    if (order) {
+        ICM_CUDA(b->ctx, cudaMemcpyAsync(b->d_cl_order, ord.data(), ord.size() * 2, cudaMemcpyHostToDevice,
+                                         b->ctx->stream));
+        ICM_CUDA(b->ctx, cudaStreamSynchronize(b->ctx->stream));   // the host table is read by the copy
+    }
     b->cluster_k = K;
     b->cl = L;
     P.cl_order = order ? b->d_cl_order : nullptr;
