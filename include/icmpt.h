@@ -547,8 +547,9 @@ icm_status icm_load(icm_batch *b, const void *buf, size_t len);
  * its shared memory together with copies of the other CTAs' border sites,
  * which their owners write through the cluster's distributed shared memory.
  * The lattice's tables of those copies are device memory of the context (its
- * budget).  The arithmetic and random keys are those of
- * the one-CTA layouts (the same chain, bit for bit for +-J); a single large
+ * budget); a group keeps the tables that it was captured with, whatever shape
+ * the batch takes afterwards, and a refused call leaves the batch as it was.
+ * The arithmetic and random keys are those of the one-CTA layouts (the same chain, bit for bit for +-J); a single large
  * instance finishes its sweeps up to K times sooner.  Any lattice kind
  * (2D, 3D, chimera, 4D), diluted or not, with N/2 divisible into K blocks
  * of a multiple of 32 sites.  K = 0 returns to one CTA per instance (CTA

@@ -313,10 +313,12 @@ struct icm_batch {
     // cluster layout: one instance per thread-block cluster of cluster_k CTAs
     int cluster_k = 0;
     int cl_growth = -1;               // cluster growth: -1 = by the library (scans), 0 = scans, 1 = union-find
-    uint16_t *d_cl_order = nullptr;   // [N] growth order of the cluster layout's own sites (KParams::cl_order)
-    uint16_t *d_cl_tab = nullptr;     // ClusterTables of cl_tab_k CTAs, cl_tab_size 16-bit entries in all
-    size_t cl_tab_size = 0;
-    int cl_tab_k = 0, cl_nh = 0, cl_nx = 0;
+    struct ClusterTab {               // device tables of the cluster layout for one K (see upload_cluster_tables)
+        uint16_t *dev = nullptr;
+        size_t size = 0;              // 16-bit entries of the block
+        int nh = 0, nx = 0;
+    };
+    ClusterTab cl_tab[3];             // K = 2, 4, 8: cl_tab[K >> 2]
     icm::ClusterLayout cl{};
     int n_clusters = 0;
     // wide (global-resident) layout: per-CTA scratch, grown on demand (in allocs)
@@ -1447,41 +1449,68 @@ static icm_status apply_threads(icm_batch *b, int threads)
     return ICM_OK;
 }
 
+// Whether the CTAs of a cluster hold whole pairs of rows of a 2D lattice, so that
+// a thread can grow a 2 x 2 block of sites.
+static bool cluster_blocks(const icm_batch *b, int K)
+{
+    const int row = b->L / 2, hs = b->kp.N / 2 / K;      // sites of a colour in a row, in a CTA
+    return b->lattice == ICM_SQUARE2D && hs % row == 0 && (hs / row) % 2 == 0;
+}
+
+// Growth order of the cluster layout's own sites, the same in every CTA (see
+// KParams::cl_order): each thread takes a 2 x 2 block, around the block
+// (a (x0, y0), b (x0 + 1, y0), d (x0 + 1, y0 + 1), c (x0, y0 + 1)), threads along
+// the rows; local index of (x, y) in a CTA's rows: colour c = (x + y) & 1,
+// c hs + y L / 2 + x / 2 (rows per CTA even, so the colour of a local row is that
+// of the lattice row).  Empty where there are no such blocks.
+static std::vector<uint16_t> cluster_order(const icm_batch *b, int K)
+{
+    if (!cluster_blocks(b, K)) return {};
+    const int L = b->L, hs = b->kp.N / 2 / K, nls = 2 * hs;
+    std::vector<uint16_t> ord(nls);
+    const int dy[4] = {0, 0, 1, 1}, dx[4] = {0, 1, 1, 0};
+    for (int i = 0; i < nls; ++i) {
+        const int t = i / 4, y = 2 * (t / (L / 2)) + dy[i % 4], x = 2 * (t % (L / 2)) + dx[i % 4];
+        ord[i] = (uint16_t)(((x + y) & 1) * hs + y * (L / 2) + x / 2);
+    }
+    return ord;
+}
+
 // Put the cluster layout's tables t of the batch's lattice and K CTAs on the
-// device (unless they are there) and point the kernels' parameters at them.
+// device.  One block per K, never rewritten while a group lives: its captured
+// launches hold the addresses of the tables of their K.  Without a group a block
+// of another K that is large enough is taken over (earlier launches on the
+// stream come before the copy).
 static icm_status upload_cluster_tables(icm_batch *b, int K, const icm::ClusterTables &t)
 {
-    icm::KParams &P = b->kp;
-    if (b->cl_tab_k != K) {
-        // 32-bit tables first, then the 16-bit ones
-        std::vector<uint16_t> all;
-        auto put = [&](const void *p, size_t bytes) {
-            all.insert(all.end(), (const uint16_t *)p, (const uint16_t *)p + bytes / 2);
-        };
-        put(t.xl.data(), t.xl.size() * 4);
-        put(t.hown.data(), t.hown.size() * 4);
-        put(t.nb.data(), t.nb.size() * 2);
-        put(t.hpos.data(), t.hpos.size() * 2);
-        put(t.xoff.data(), t.xoff.size() * 2);
-        if (all.size() > b->cl_tab_size) {
-            uint16_t *q = nullptr;
-            if (icm_status st = dalloc(b, &q, all.size())) return st;
-            b->d_cl_tab = q;
-            b->cl_tab_size = all.size();
-        }
-        ICM_CUDA(b->ctx, cudaMemcpyAsync(b->d_cl_tab, all.data(), all.size() * 2, cudaMemcpyHostToDevice,
-                                         b->ctx->stream));
-        ICM_CUDA(b->ctx, cudaStreamSynchronize(b->ctx->stream));   // the host tables are read by the copy
-        b->cl_tab_k = K;
-        b->cl_nh = t.nh;
-        b->cl_nx = t.nx;
+    const std::vector<uint16_t> order = cluster_order(b, K);
+    // 32-bit tables first, then the 16-bit ones
+    std::vector<uint16_t> all;
+    auto put = [&](const void *p, size_t bytes) {
+        all.insert(all.end(), (const uint16_t *)p, (const uint16_t *)p + bytes / 2);
+    };
+    put(t.xl.data(), t.xl.size() * 4);
+    put(t.hown.data(), t.hown.size() * 4);
+    put(t.nb.data(), t.nb.size() * 2);
+    put(t.hpos.data(), t.hpos.size() * 2);
+    put(t.xoff.data(), t.xoff.size() * 2);
+    put(order.data(), order.size() * 2);
+    icm_batch::ClusterTab now;
+    if (!b->groups)
+        for (auto &o : b->cl_tab)
+            if (!now.dev && o.dev && o.size >= all.size()) {
+                now = o;
+                o = {};
+            }
+    if (!now.dev) {
+        if (icm_status st = dalloc(b, &now.dev, all.size())) return st;
+        now.size = all.size();
     }
-    const size_t n = (size_t)P.N, nh = (size_t)K * b->cl_nh, nx = (size_t)K * b->cl_nx;
-    P.cl_xl = (const uint32_t *)b->d_cl_tab;
-    P.cl_hown = P.cl_xl + nx;
-    P.cl_nb = (const uint16_t *)(P.cl_hown + nh);
-    P.cl_hpos = P.cl_nb + n * P.Z;
-    P.cl_xoff = P.cl_hpos + nh;
+    now.nh = t.nh;
+    now.nx = t.nx;
+    ICM_CUDA(b->ctx, cudaMemcpyAsync(now.dev, all.data(), all.size() * 2, cudaMemcpyHostToDevice, b->ctx->stream));
+    ICM_CUDA(b->ctx, cudaStreamSynchronize(b->ctx->stream));   // the host tables are read by the copy
+    b->cl_tab[K >> 2] = now;
     return ICM_OK;
 }
 
@@ -1508,33 +1537,12 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
     // group takes the most pairs (up to kMaxUfGroup) that keep as many
     // clusters resident
     const int ufg1 = b->cl_growth == 1 ? 1 : 0;
-    // 2D lattices whose CTAs hold whole pairs of rows, four sites per thread:
-    // each thread grows a 2 x 2 block of sites, around the block
-    // (a (x0, y0), b (x0 + 1, y0), d (x0 + 1, y0 + 1), c (x0, y0 + 1)),
-    // threads along the rows; local index of (x, y) in a CTA's rows: colour
-    // c = (x + y) & 1, c hs + y L / 2 + x / 2 (rows per CTA even, so the
-    // colour of a local row is that of the lattice row)
-    const int Lx = b->L, nls = 2 * hs;
-    const bool order = b->lattice == ICM_SQUARE2D && hs % (Lx / 2) == 0 && (hs / (Lx / 2)) % 2 == 0 &&
-                       nls == 4 * threads;
-    std::vector<uint16_t> ord;
-    if (order) {
-        ord.assign(nls, 0);
-        std::vector<uint8_t> seen(nls, 0);
-        const int dy[4] = {0, 0, 1, 1}, dx[4] = {0, 1, 1, 0};
-        for (int t = 0; t < threads; ++t)
-            for (int j = 0; j < 4; ++j) {
-                const int y = 2 * (t / (Lx / 2)) + dy[j], x = 2 * (t % (Lx / 2)) + dx[j];
-                const int li = ((x + y) & 1) * hs + y * (Lx / 2) + x / 2;
-                if (li >= nls || seen[li]) return fail(b->ctx, ICM_ERR_STATE, "growth order is not a permutation");
-                seen[li] = 1;
-                ord[(size_t)4 * t + j] = (uint16_t)li;
-            }
-    }
-    icm::ClusterTables tab;                  // of another K than the tables on the device
-    tab.nh = b->cl_nh;
-    tab.nx = b->cl_nx;
-    if (b->cl_tab_k != K) icm::cluster_tables(b->h_nbr.data(), P.N, P.Z, K, tab);
+    const bool order = cluster_blocks(b, K) && 2 * hs == 4 * threads;   // four sites a thread: 2 x 2 blocks
+    const icm_batch::ClusterTab &have = b->cl_tab[K >> 2];
+    icm::ClusterTables tab;                  // unless they are on the device
+    tab.nh = have.nh;
+    tab.nx = have.nx;
+    if (!have.dev) icm::cluster_tables(b->h_nbr.data(), P.N, P.Z, K, tab);
     const int nh = tab.nh, nx = tab.nx;
     const int rows = ufg1 ? 0 : icm::cluster_row_kind(P.row_kind, b->L, K);
     icm::ClusterLayout L = icm::cluster_layout(P.N, P.Z, P.R, P.G, P.nT, K, threads / 32, b->gauss, ufg1, order, nh, nx,
@@ -1565,17 +1573,16 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
         lean = 0;
     }
     L.lean = lean >= b->n_inst ? 1 : 0;
-    if (order && !b->d_cl_order)
-        if (icm_status st = dalloc(b, &b->d_cl_order, (size_t)P.N)) return st;
-    if (icm_status st = upload_cluster_tables(b, K, tab)) return st;
-    if (order) {
-        ICM_CUDA(b->ctx, cudaMemcpyAsync(b->d_cl_order, ord.data(), ord.size() * 2, cudaMemcpyHostToDevice,
-                                         b->ctx->stream));
-        ICM_CUDA(b->ctx, cudaStreamSynchronize(b->ctx->stream));   // the host table is read by the copy
-    }
+    if (!have.dev)
+        if (icm_status st = upload_cluster_tables(b, K, tab)) return st;
+    P.cl_xl = (const uint32_t *)have.dev;
+    P.cl_hown = P.cl_xl + (size_t)K * nx;
+    P.cl_nb = (const uint16_t *)(P.cl_hown + (size_t)K * nh);
+    P.cl_hpos = P.cl_nb + (size_t)P.N * P.Z;
+    P.cl_xoff = P.cl_hpos + (size_t)K * nh;
+    P.cl_order = order ? P.cl_xoff + P.N : nullptr;
     b->cluster_k = K;
     b->cl = L;
-    P.cl_order = order ? b->d_cl_order : nullptr;
     b->threads = threads;
     b->n_clusters = b->n_inst < clusters ? b->n_inst : clusters;
     b->grid = b->n_clusters * K;

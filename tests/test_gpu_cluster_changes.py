@@ -71,3 +71,40 @@ def test_change_beyond_the_budget_keeps_the_batch(icm, kind, L, first, second, d
             _equals_oracle(b, g, J, s0, T, 0x1602, 6)
         b.close()
         ctx.close()
+
+
+@pytest.mark.parametrize("kind,L,shapes,dilution", [
+    (O.CUBIC3D, 8, ((8, 32), (4, 64), (2, 128)), 0.0),
+    (O.SQUARE2D, 32, ((8, 32), (4, 64), (2, 128)), 0.2),       # 2 x 2 growth blocks in all
+    (O.SQUARE2D, 32, ((2, 128), (8, 32), (4, 64)), 0.0),       # row form
+], ids=["3d", "2d_blocks", "2d_rows"])
+def test_captured_group_keeps_its_tables(icm, kind, L, shapes, dilution):
+    """A group captured on one cluster shape runs on unchanged while the batch takes
+    other shapes, by request and by the tuner; without a group the shapes share
+    their memory."""
+    icmpt, ctx = icm
+    T = I.ladder(0.3, 2.0, 8)
+    g, J, s0, ids = _setup(kind, L, I.PM_J, 2, T, 0x1604)
+    if dilution:
+        J = I.dilute(J, dilution, 0x1604, ids)
+    b = icmpt.Batch(ctx, kind, L, I.PM_J, J, T, 1.0, 0x1604, spins=s0)
+    b.set_cluster(*shapes[0])
+    grp = icmpt.Group(ctx, [b], sweeps_per_launch=2)
+    for shape in shapes[1:]:
+        grp.run(1)
+        b.set_cluster(*shape)
+        grp.run(1)
+        b.run(1)
+    b.autotune(1)
+    grp.run(1)
+    _equals_oracle(b, g, J, s0, T, 0x1604, 12)
+    grp.close()
+    held = 0
+    for i in range(6):
+        b.set_cluster(*shapes[i % 3])
+        b.run(1)
+        if i == 2:
+            held = ctx.memory()[0]
+    assert ctx.memory()[0] == held
+    _equals_oracle(b, g, J, s0, T, 0x1604, 18)
+    b.close()
