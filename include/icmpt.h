@@ -549,10 +549,10 @@ icm_status icm_load(icm_batch *b, const void *buf, size_t len);
  * The lattice's tables of those copies are device memory of the context (its
  * budget); a group keeps the tables that it was captured with, whatever shape
  * the batch takes afterwards, and a refused call leaves the batch as it was.
- * The arithmetic and random keys are those of the one-CTA layouts (the same chain, bit for bit for +-J); a single large
- * instance finishes its sweeps up to K times sooner.  Any lattice kind
- * (2D, 3D, chimera, 4D), diluted or not, with N/2 divisible into K blocks
- * of a multiple of 32 sites.  K = 0 returns to one CTA per instance (CTA
+ * The arithmetic and random keys are those of the one-CTA layouts (the same
+ * chain, bit for bit for +-J); a single large instance finishes its sweeps
+ * up to K times sooner.  Any lattice kind (2D, 3D, chimera, 4D), diluted or
+ * not, with N/2 divisible into K blocks of a multiple of 32 sites.  K = 0 returns to one CTA per instance (CTA
  * width `threads`, as icm_batch_set_threads).  A batch keeps the layout when
  * couplings with absent bonds are loaded (its kernels change).            */
 icm_status icm_batch_set_cluster(icm_batch *b, int32_t K, int32_t threads);

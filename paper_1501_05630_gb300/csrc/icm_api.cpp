@@ -1537,7 +1537,6 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
     // group takes the most pairs (up to kMaxUfGroup) that keep as many
     // clusters resident
     const int ufg1 = b->cl_growth == 1 ? 1 : 0;
-    const bool order = cluster_blocks(b, K) && 2 * hs == 4 * threads;   // four sites a thread: 2 x 2 blocks
     const icm_batch::ClusterTab &have = b->cl_tab[K >> 2];
     icm::ClusterTables tab;                  // unless they are on the device
     tab.nh = have.nh;
@@ -1545,6 +1544,8 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
     if (!have.dev) icm::cluster_tables(b->h_nbr.data(), P.N, P.Z, K, tab);
     const int nh = tab.nh, nx = tab.nx;
     const int rows = ufg1 ? 0 : icm::cluster_row_kind(P.row_kind, b->L, K);
+    // growth by scans with four sites a thread: 2 x 2 blocks
+    const bool order = !ufg1 && !rows && cluster_blocks(b, K) && 2 * hs == 4 * threads;
     icm::ClusterLayout L = icm::cluster_layout(P.N, P.Z, P.R, P.G, P.nT, K, threads / 32, b->gauss, ufg1, order, nh, nx,
                                                rows, b->L);
     // the neighbour table holds shared-memory offsets in 16 bits (a slice
@@ -1557,7 +1558,7 @@ static icm_status apply_cluster(icm_batch *b, int K, int threads)
     if (clusters < 1) return fail(b->ctx, ICM_ERR_UNSUPPORTED, "cluster does not fit");
     for (int g = 2; ufg1 && g <= icm::kMaxUfGroup && g <= (P.n_icm > 1 ? P.n_icm : 1); ++g) {
         const icm::ClusterLayout Lg = icm::cluster_layout(P.N, P.Z, P.R, P.G, P.nT, K, threads / 32, b->gauss, g,
-                                                          order, nh, nx, 0, b->L);
+                                                          false, nh, nx, 0, b->L);
         int cg = 0;
         if (Lg.total > b->ctx->max_smem_optin ||
             icm::cluster_occupancy(b->gauss, P.Z, P.diluted != 0, false, K, threads, Lg.total, &cg) != cudaSuccess ||
