@@ -4,6 +4,11 @@ hold one word per site.  +-J: equal to the oracle, bit for bit.  Gaussian: the
 same chain as a wide CTA with its instance in shared memory, bit for bit (the
 same sums in the same order); for instances that fit nowhere else, energies and
 cluster moves against the spins to 1e-5 sum|J|, as in the other layouts."""
+import json
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -113,3 +118,12 @@ def test_gauss_conservation_and_consistency(icm, kind, L, nT, T_hi, dilution):
         moves += _check_icm_only_step(b, g, J, T, 1.0)
     assert moves > 0
     b.close()
+
+
+def test_checked_build_finds_no_out_of_range_index():
+    here = os.path.dirname(os.path.abspath(__file__))
+    r = subprocess.run([sys.executable, os.path.join(here, "checked_wide_run.py")], capture_output=True, text=True,
+                       timeout=900)
+    assert r.returncode == 0, r.stdout + r.stderr
+    out = json.loads(r.stdout.strip().splitlines()[-1])
+    assert out == {"rc": 0, "check": [0, 0, 0, 0], "mismatch": [], "elsewhere": []}
