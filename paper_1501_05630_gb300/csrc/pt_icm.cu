@@ -272,7 +272,10 @@ __device__ __forceinline__ void gauss_pass(const KParams &P, const uint32_t (&ke
                     // sh = s_i h_i, Delta E = 2 sh; accept iff x < 2^32 exp(-2 beta sh),
                     // compared as rz(x) < 2^(32 + b2l sh) in fp32 (b2l = -2 beta log2 e):
                     // for sh <= 0 the right side is >= 2^32 > rz(x), so Delta E <= 0 is
-                    // always accepted
+                    // always accepted (ex2.approx of every fp32 argument from 32 up, all
+                    // checked on the device).  x = 0 passes at any finite Delta E down to
+                    // the smallest normal right side: 2^-32 of the proposals, where the
+                    // cluster kernel's integer threshold rounds such probabilities to 0
                     const float sh = neg_if(h, sw & (1u << b));
                     const uint32_t xr = i < 4 ? x[i] : y[i - 4];
                     const float lim = ex2_approx(fmaf(bl[i >> 1], sh, 32.f));
@@ -1281,7 +1284,7 @@ __global__ void __launch_bounds__(kMaxThreads, 7) fused_kernel(const KParams P, 
 
 // Gaussian batches with one temperature (see gauss_pair_sweep), as a kernel of
 // their own: the branch in fused_kernel slowed 3D L=8 x 1000 by 0.9%.  16
-// annealing steps of 32 sweeps of 512 3D L=6 instances: 4.64 to 3.49 ms.
+// annealing steps of 32 sweeps of 512 3D L=6 instances: 4.79 to 3.64 ms.
 template <int Z, bool DIL>
 __global__ void __launch_bounds__(kMaxThreads, 7) fused_pair_kernel(const KParams P, uint32_t n_sweeps)
 {
