@@ -441,9 +441,12 @@ bool on_device(const icm_ctx *ctx, const void *p, uint32_t flags)
 //     61.2 (2), 82.0 / 66.7 / 90.9 (3), 94.8 / 103.5 (4)
 //   2D L=32 (512), 128 / 256 / 512 / 1024: 40.7 / 27.0 / 22.7 / 24.1 (1), 45.7 /
 //     35.0 / 35.5 (2), 53.4 / 46.7 / 69.7 (3)
-// Instances of 65 to 287 sites of a colour keep 128 threads, the width that a
-// batch of such instances reports by default (chimera C_8, 128 / 256: 24.6 / 18.9
-// alone on an SM, 27.5 / 24.4 with two, 31.3 / 32.2 with three).
+// Instances of 65 to 287 sites of a colour keep 128 threads although one or two
+// on an SM would gain (chimera C_8, 128 / 256: 24.6 / 18.9 alone, 27.5 / 24.4 with
+// two, 31.3 / 32.2 with three): a width up to 128 is what a batch of them reports
+// by default, which callers may rely on.  The rule counts the batch's own
+// instances: several such batches in one group share the SMs, and by the figures
+// above lose up to a tenth with three instances on an SM; set_threads is theirs.
 int roomy_threads(const icm_ctx *ctx, int N, int Z, int R, int G, int n_T, int n_icm, int n_inst, int threads)
 {
     const int per_sm = (n_inst + ctx->num_sms - 1) / ctx->num_sms;

@@ -15,7 +15,7 @@ constexpr uint32_t kFull = 0xffffffffu;
 // (count, then the site code, index and bound of the first one) and replaced
 // by 0, so the access stays inside the array and the kernel runs on; the
 // host reads the word with icm_debug_check.  In normal builds ICM_IDX is the
-// index itself.  (The substitute for a memory checker on this pool.)
+// index itself.  (It stands in for a memory checker.)
 #ifdef ICM_CHECKED
 static __device__ unsigned int g_icm_check[4];
 __device__ __forceinline__ int icm_guard(int idx, int bound, int site)
